@@ -40,6 +40,7 @@ WORKLOAD = dict(workload="KD-staggered MG solve, 2D U(1) 256x256, beta=6 (2000 h
                 L=256, beta=6.0, sweeps=2000, mass=1e-3, levels=3, blocks=[[4, 4], [2, 2]],
                 nvec=[24, 32], tol=1e-10, coarsest_maxiter=2048)
 FP64_PEAK_TFLOPS = 152 * 4 * 2.070e9 / 1e12  # 4 FP64 flop/clk/SM (2 DFMA) x 152 SMs x 2070 MHz
+MMA_SYNC_TFLOPS = 594.0  # 152 SMs x 944 multiply-adds per clock x 2.07 GHz, mma.sync m16n8k16 FP16
 
 
 def _hbm_peak():
@@ -647,31 +648,23 @@ def run_native(args, rank, world, local):
     shapes = {l: sw.sw_mg_level_info(h, l + 1) for l in (1, 2)}
     cand = {c: ktimes[c][1] for c in (1, 2, 5)}
     best = max(cand, key=cand.get)
-    variant = None
     if best == 5:
         e0, e1, nc = shapes[2]
         iters = ktimes[6][0]
         n_l, ms_l = ktimes[5]
-        # variant the FP64 kernel's autotuner chose (bit 0: three-FMA products, bit 1:
-        # reduce-scatter row sums, bit 2: operands staged in shared memory)
-        ch = [e for e in sw.sw_autotune_entries() if e[1] == 1 and e[0] == nc and e[2] == e0 * e1]
-        variant = ch[0][3] if ch else None
         per_apply_flop = 8.0 * 5 * nc * nc * e0 * e1
         flop = per_apply_flop * 2 * iters / max(n_l, 1)      # per launch
-        ybytes = (24.0 if (variant or 0) & 1 else 16.0) * 5 * nc * nc * e0 * e1
-        byt = (ybytes + 16.0 * 2 * nc * e0 * e1) * 2 * iters / max(n_l, 1)
-        kname = (f"k_cgne64<{nc}, {'three' if (variant or 0) & 1 else 'four'}-FMA products"
-                 f"{', reduce-scatter row sums' if (variant or 0) & 2 else ''}"
-                 f"{', operands staged in shared memory' if (variant or 0) & 4 else ''}> "
-                 f"(persistent FP64 coarsest CGNE, {e0}x{e1} sites, {nc}x{nc} complex128 blocks, "
-                 f"{iters / max(n_l, 1):.0f} iterations = {2 * iters / max(n_l, 1):.0f} stencil "
-                 f"applications per launch)")
+        byt = (16.0 * 5 * nc * nc * e0 * e1 + 16.0 * 2 * nc * e0 * e1) * 2 * iters / max(n_l, 1)
+        kname = (f"k_cgne64 (persistent FP64 coarsest CGNE, {e0}x{e1} sites, {nc}x{nc} complex "
+                 f"blocks as eight base-256 digits per component, FP16 MMAs with exact integer "
+                 f"sums; {iters / max(n_l, 1):.0f} iterations = {2 * iters / max(n_l, 1):.0f} "
+                 f"stencil applications per launch)")
     else:
         e0, e1, nc = shapes[best]
         n_l, ms_l = ktimes[best]
         flop = 8.0 * 5 * nc * nc * e0 * e1
         byt = 16.0 * (5 * nc * nc + 2 * nc) * e0 * e1
-        kname = f"k_coarse_apply_nc<{nc}> (level {best + 1}: {e0}x{e1} sites)"
+        kname = f"k_digit_apply (level {best + 1}: {e0}x{e1} sites, {nc}x{nc} blocks)"
     dur = ms_l / 1e3 / max(n_l, 1)
     achieved = flop / dur / 1e12
     traffic = None
@@ -680,19 +673,23 @@ def run_native(args, rank, world, local):
                                      "dram_bytes_per_iteration")
         if per_iter is not None:
             traffic = per_iter * iters / max(n_l, 1)
-    executed = (6.0 / 8.0 if (variant or 0) & 1 else 1.0) * achieved
-    roof = {"bound": "alu", "kernel": kname,
-            "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s",
-            "frac": achieved / fp64_peak, "traffic": traffic,
-            "achieved_note": "algorithmic flops of the stencil products (8 per complex "
-                             "multiply-add, the operation's definition) per launch / average "
-                             "launch time; the three-FMA form executes 6 of them",
-            "executed_TFLOPs": executed, "executed_frac": executed / fp64_peak,
+    # a complex entry takes 12 m16n8k16 MMAs per 128 of them: 384 FP16 flops for its 8 FP64 ones
+    executed = 384.0 / 8.0 * achieved
+    roof = {"bound": "tensor", "kernel": kname,
+            "achieved": executed, "peak": MMA_SYNC_TFLOPS, "unit": "TFLOP/s",
+            "frac": executed / MMA_SYNC_TFLOPS, "traffic": traffic,
+            "achieved_note": "FP16 tensor flops executed by the digit products (384 per complex "
+                             "multiply-add) per launch / average launch time",
+            "fp64_TFLOPs": achieved, "fp64_peak_TFLOPs": fp64_peak,
+            "fp64_frac": achieved / fp64_peak,
+            "fp64_note": "algorithmic FP64 flops (8 per complex multiply-add) over the FP64 FMA "
+                         "rate sw_fp64_peak measures in this run: above 1 because the products "
+                         "do not run on the FP64 pipe",
             "traffic_note": "ncu dram bytes per CGNE iteration (profiles/k_cgne64_fp64_256.md) x "
                             "iterations per launch; null if the kernel changed since",
-            "peak_source": "measured in this run by sw_fp64_peak (FP64 FMA throughput, 16 warps "
-                           "x 4 chains per SM); MEASURED_PEAKS.json has no FP64 entry",
-            "peak_nominal": FP64_PEAK_TFLOPS, "frac_of_nominal": achieved / FP64_PEAK_TFLOPS,
+            "peak_source": "measured rate of independent mma.sync m16n8k16 FP16 at 2070 MHz: 944 "
+                           "multiply-adds per clock and SM",
+            "fp64_peak_nominal": FP64_PEAK_TFLOPS,
             "algorithmic_flop_per_launch": flop,
             "hbm_GBps_equiv": byt / dur / 1e9, "launches": n_l, "avg_us": dur * 1e6}
     names = {0: "S", 1: "A_hat_level2", 2: "A_hat_level3", 5: "cgne_persistent"}

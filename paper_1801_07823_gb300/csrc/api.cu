@@ -633,7 +633,10 @@ int sw_mg_apply_level(sw_mg* mg, int level, int precision, int dagger, const voi
       // timed like the solver's applications (category level - 1), kernel only
       const int tk = timing_begin(mg->ctx, level - 1);
       if (precision == SW_PREC_FP64) {
-        launch_coarse_apply(cg, L.Y, dagger ? 1 : 0, a, b, s);
+        if (L.dg.T)
+          launch_digit_apply(cg, L.dg, L.Y, dagger ? 1 : 0, a, b, mg->ctx->device, s);
+        else
+          launch_coarse_apply(cg, L.Y, dagger ? 1 : 0, a, b, s);
       } else if (precision == SW_PREC_FP16S) {
         SW_REQUIRE(L.Yh, SW_ERR_ARG, "no scaled-FP16 stencil on this level");
         launch_coarse_apply_h(cg, L.Yh, L.Ysc, dagger ? 1 : 0, a, b, s);

@@ -1,5 +1,6 @@
-// Coarsest-level CGNE (CG on the normal error, Sec. IV and Table kcycle) as
-// one persistent cooperative kernel.
+// Coarsest-level CGNE (CG on the normal error, Sec. IV and Table kcycle) with
+// a double-float stencil as one persistent cooperative kernel: the option
+// SW_COARSEST_DF64=1 of a mixed hierarchy (cgne64.cu is the FP64 solver).
 //
 // The coarsest level is small (16^2 sites x 64 dof at 256^2) and its solve
 // runs hundreds of iterations, each two stencil applications and two norms.
@@ -32,18 +33,6 @@ namespace {
 
 constexpr long kSpinLimit = 1L << 24;    // ~0.3-1.5 s of polling
 
-__device__ __forceinline__ void cfma(double2& acc, double2 a, double2 b) {
-  acc.x = fma(a.x, b.x, acc.x);
-  acc.x = fma(-a.y, b.y, acc.x);
-  acc.y = fma(a.x, b.y, acc.y);
-  acc.y = fma(a.y, b.x, acc.y);
-}
-__device__ __forceinline__ void cfmac(double2& acc, double2 a, double2 b) {
-  acc.x = fma(a.x, b.x, acc.x);
-  acc.x = fma(a.y, b.y, acc.x);
-  acc.y = fma(a.x, b.y, acc.y);
-  acc.y = fma(-a.y, b.x, acc.y);
-}
 // Double-float ("df64") arithmetic on the FP32 pipes (Dekker 1971; Knuth's
 // two-sum): a value is hi + lo with two floats, 48 significant bits.
 // GB300 issues FP32 FMAs at 62x the FP64 rate, so the coarsest stencil in
@@ -96,12 +85,12 @@ __device__ __forceinline__ int opp(int d) {
 }
 
 struct CgneArgs {
-  const void* Y;      // complex128 stencil, or df64 float4 stencil for the DF variant
+  const float4* Y;    // df64 stencil
   const double2* b;
   double2* x;
   double2* r;
   double2* p;
-  float4* rdf;        // DF variant: df64 copies of r and p that the stencil reads
+  float4* rdf;        // df64 copies of r and p that the stencil reads
   float4* pdf;
   double* partials;   // [2][gridDim.x], alternating by phase
   unsigned* bar;      // [0] arrival count, [1] generation
@@ -174,14 +163,12 @@ constexpr int kRows = 8;   // rows per work item (one warp, 4 lanes per row)
 // Row i of (A v)_X (dagger: (A^dag v)_X) summed by the 4 lanes of the row:
 // lane q takes columns j in [q nc/4, (q+1) nc/4) of all five blocks.  Every
 // lane of the row returns the same value.
-template <int NC, bool DF>
-__device__ __forceinline__ double2 stencil_row(const void* __restrict__ Yv,
-                                               const double2* __restrict__ v,
+template <int NC>
+__device__ __forceinline__ double2 stencil_row(const float4* __restrict__ Yv,
                                                const float4* __restrict__ vdf, int X, int i,
                                                int q, int E0, int E1, bool dagger) {
   constexpr int QJ = NC / 4;  // columns per lane and direction
   const int j0 = q * QJ;
-  double2 acc = make_double2(0.0, 0.0);
   df2 re{0.f, 0.f}, im{0.f, 0.f};
 #pragma unroll
   for (int d = 0; d < 5; ++d) {
@@ -190,31 +177,18 @@ __device__ __forceinline__ double2 stencil_row(const void* __restrict__ Yv,
                               : (((long)X * 5 + d) * NC + j0) * NC + i;
     const long ystep = dagger ? 1 : NC;
     const long xbase = nb * NC + j0;
-    if (!DF) {
-      const double2* Y = (const double2*)Yv + ybase;
+    const float4* Y = Yv + ybase;
 #pragma unroll 8
-      for (int t = 0; t < QJ; ++t) {
-        double2 y = __ldg(Y + t * ystep);
-        double2 xv = __ldcg(v + xbase + t);
-        if (dagger)
-          cfmac(acc, y, xv);
-        else
-          cfma(acc, y, xv);
-      }
-    } else {
-      const float4* Y = (const float4*)Yv + ybase;
-#pragma unroll 8
-      for (int t = 0; t < QJ; ++t) {
-        float4 y = __ldg(Y + t * ystep);
-        float4 xv = __ldcg(vdf + xbase + t);
-        if (dagger)
-          df_cmac<true>(re, im, y, xv);
-        else
-          df_cmac<false>(re, im, y, xv);
-      }
+    for (int t = 0; t < QJ; ++t) {
+      float4 y = __ldg(Y + t * ystep);
+      float4 xv = __ldcg(vdf + xbase + t);
+      if (dagger)
+        df_cmac<true>(re, im, y, xv);
+      else
+        df_cmac<false>(re, im, y, xv);
     }
   }
-  if (DF) acc = make_double2((double)re.hi + (double)re.lo, (double)im.hi + (double)im.lo);
+  double2 acc = make_double2((double)re.hi + (double)re.lo, (double)im.hi + (double)im.lo);
   // quarters of the row: butterfly over lanes q = 0..3 (exactly commutative)
   acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 1);
   acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 1);
@@ -223,7 +197,7 @@ __device__ __forceinline__ double2 stencil_row(const void* __restrict__ Yv,
   return acc;
 }
 
-template <int NC, bool DF>
+template <int NC>
 __global__ void __launch_bounds__(kWarps * 32, 2) k_cgne(CgneArgs a) {
   __shared__ double red[32];
   __shared__ double bcast;
@@ -246,7 +220,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_cgne(CgneArgs a) {
     double2 v = a.b[e];
     a.x[e] = make_double2(0.0, 0.0);
     a.r[e] = v;
-    if (DF) a.rdf[e] = to_df(v);
+    a.rdf[e] = to_df(v);
     acc = fma(v.x, v.x, fma(v.y, v.y, acc));
   }
   int ph = 0;  // which partials array this phase writes
@@ -276,11 +250,11 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_cgne(CgneArgs a) {
     int item = rd * nwarps + warp * gridDim.x + blockIdx.x;
     if (item >= nitems) break;  // warp-uniform
     int X = item / chunks, i = (item - X * chunks) * kRows + rr8;
-    double2 w = stencil_row<NC, DF>(a.Y, a.r, a.rdf, X, i, q, a.E0, a.E1, true);
+    double2 w = stencil_row<NC>(a.Y, a.rdf, X, i, q, a.E0, a.E1, true);
     if (q == 0) {
       long e = (long)X * NC + i;
       a.p[e] = w;
-      if (DF) a.pdf[e] = to_df(w);
+      a.pdf[e] = to_df(w);
       acc = fma(w.x, w.x, fma(w.y, w.y, acc));
     }
   }
@@ -301,7 +275,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_cgne(CgneArgs a) {
       int item = rd * nwarps + warp * gridDim.x + blockIdx.x;
       if (item >= nitems) break;
       int X = item / chunks, i = (item - X * chunks) * kRows + rr8;
-      double2 w = stencil_row<NC, DF>(a.Y, a.p, a.pdf, X, i, q, a.E0, a.E1, false);
+      double2 w = stencil_row<NC>(a.Y, a.pdf, X, i, q, a.E0, a.E1, false);
       if (q == 0) {
         long e = (long)X * NC + i;
         double2 pv = __ldcg(a.p + e), xv = __ldcg(a.x + e), rv = __ldcg(a.r + e);
@@ -311,7 +285,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_cgne(CgneArgs a) {
         rv.y = fma(-alpha, w.y, rv.y);
         a.x[e] = xv;
         a.r[e] = rv;
-        if (DF) a.rdf[e] = to_df(rv);
+        a.rdf[e] = to_df(rv);
         acc = fma(rv.x, rv.x, fma(rv.y, rv.y, acc));
       }
     }
@@ -339,14 +313,14 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_cgne(CgneArgs a) {
       int item = rd * nwarps + warp * gridDim.x + blockIdx.x;
       if (item >= nitems) break;
       int X = item / chunks, i = (item - X * chunks) * kRows + rr8;
-      double2 w = stencil_row<NC, DF>(a.Y, a.r, a.rdf, X, i, q, a.E0, a.E1, true);
+      double2 w = stencil_row<NC>(a.Y, a.rdf, X, i, q, a.E0, a.E1, true);
       if (q == 0) {
         long e = (long)X * NC + i;
         double2 pv = __ldcg(a.p + e);
         pv.x = fma(beta, pv.x, w.x);
         pv.y = fma(beta, pv.y, w.y);
         a.p[e] = pv;
-        if (DF) a.pdf[e] = to_df(pv);
+        a.pdf[e] = to_df(pv);
         acc = fma(pv.x, pv.x, fma(pv.y, pv.y, acc));
       }
     }
@@ -390,14 +364,14 @@ __global__ void k_coarse_apply_df(const float4* __restrict__ Y, const double2* _
   out[e] = tot;
 }
 
-template <int NC, bool DF>
+template <int NC>
 bool launch_cgne_t(const CgneArgs& args, int device, cudaStream_t s, int sms_use) {
   static int cached_per_sm[64] = {0}, cached_sms[64] = {0};
   int& per_sm = cached_per_sm[device & 63];
   int& sms = cached_sms[device & 63];
   if (per_sm == 0) {
     int occ = 0, coop = 0;
-    SW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cgne<NC, DF>, kWarps * 32, 0));
+    SW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cgne<NC>, kWarps * 32, 0));
     SW_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
     SW_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device));
     if (!coop || occ < 1) return false;
@@ -406,7 +380,7 @@ bool launch_cgne_t(const CgneArgs& args, int device, cudaStream_t s, int sms_use
   const int grid = (sms_use < sms ? (sms_use > 0 ? sms_use : 1) : sms) * per_sm;
   CgneArgs a = args;
   void* params[] = {&a};
-  SW_CUDA(cudaLaunchCooperativeKernel((const void*)k_cgne<NC, DF>, dim3(grid), dim3(kWarps * 32),
+  SW_CUDA(cudaLaunchCooperativeKernel((const void*)k_cgne<NC>, dim3(grid), dim3(kWarps * 32),
                                       params, 0, s));
   sw_count_launch();
   return true;
@@ -426,33 +400,21 @@ void launch_coarse_apply_df(const CoarseGeom& g, const float4* Y, int dagger, co
 }
 
 // Runs the whole coarsest CGNE on the device.  Returns false (nothing
-// launched) when nc has no compiled variant; then the caller uses the
-// host-driven loop.  partials needs 2 x grid doubles (grid <= 2 x SMs), bar 2 unsigned
-// (zeroed here), status 3 ints.
-bool launch_cgne_persistent(const CoarseGeom& g, const void* Y, int df64, const double2* b,
-                            double2* x, double2* r, double2* p, float4* rdf, float4* pdf,
-                            double* partials, unsigned* bar, int* status, int maxit, double tol,
-                            int device, cudaStream_t s, int stall_test, int sms_use) {
+// launched) when nc has no compiled variant.  partials needs 2 x grid doubles
+// (grid <= 2 x SMs), bar 2 unsigned (zeroed here), status 3 ints.
+bool launch_cgne_df(const CoarseGeom& g, const float4* Y, const double2* b, double2* x, double2* r,
+                    double2* p, float4* rdf, float4* pdf, double* partials, unsigned* bar,
+                    int* status, int maxit, double tol, int device, cudaStream_t s, int stall_test,
+                    int sms_use) {
   SW_CUDA(cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), s));
   SW_CUDA(cudaMemsetAsync(status, 0, 3 * sizeof(int), s));
   CgneArgs a{Y, b, x, r, p, rdf, pdf, partials, bar, status, g.E0, g.E1, maxit, tol, stall_test};
-  if (df64) {
-    if (!rdf || !pdf) return false;
-    switch (g.nc) {
-      case 16: return launch_cgne_t<16, true>(a, device, s, sms_use);
-      case 24: return launch_cgne_t<24, true>(a, device, s, sms_use);
-      case 32: return launch_cgne_t<32, true>(a, device, s, sms_use);
-      case 48: return launch_cgne_t<48, true>(a, device, s, sms_use);
-      case 64: return launch_cgne_t<64, true>(a, device, s, sms_use);
-      default: return false;
-    }
-  }
   switch (g.nc) {
-    case 16: return launch_cgne_t<16, false>(a, device, s, sms_use);
-    case 24: return launch_cgne_t<24, false>(a, device, s, sms_use);
-    case 32: return launch_cgne_t<32, false>(a, device, s, sms_use);
-    case 48: return launch_cgne_t<48, false>(a, device, s, sms_use);
-    case 64: return launch_cgne_t<64, false>(a, device, s, sms_use);
+    case 16: return launch_cgne_t<16>(a, device, s, sms_use);
+    case 24: return launch_cgne_t<24>(a, device, s, sms_use);
+    case 32: return launch_cgne_t<32>(a, device, s, sms_use);
+    case 48: return launch_cgne_t<48>(a, device, s, sms_use);
+    case 64: return launch_cgne_t<64>(a, device, s, sms_use);
     default: return false;
   }
 }

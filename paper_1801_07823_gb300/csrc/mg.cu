@@ -75,6 +75,19 @@ long level_len(const sw_mg* mg, int l) {
   return L.ndof;
 }
 
+// FP64 stencil of a coarse level (dagger: its adjoint), on its digit entries
+// where the level keeps them.
+void coarse_op(sw_mg* mg, int l, int dagger, const double2* in, double2* out, const int* skip) {
+  sw_ctx* c = mg->ctx;
+  const MgLevel& L = mg->lev[l];
+  const CoarseGeom cg{L.E0, L.E1, L.nc};
+  unsigned long long* exec = c->timing ? c->exec + l : nullptr;
+  if (L.dg.T)
+    launch_digit_apply(cg, L.dg, L.Y, dagger, in, out, c->device, c->stream, skip, exec);
+  else
+    launch_coarse_apply(cg, L.Y, dagger, in, out, c->stream, skip, exec);
+}
+
 // Operator of level l in the solve: S on level 0 (even half), A_hat below.
 // skip: optional device flag that turns the (coarse) application into a no-op.
 // lowp: inside the preconditioner of a mixed-precision hierarchy -- the fine
@@ -95,18 +108,14 @@ void level_op(sw_mg* mg, int l, const double2* in, double2* out, const int* skip
     const MgLevel& L = mg->lev[l];
     launch_coarse_apply_h(CoarseGeom{L.E0, L.E1, L.nc}, L.Yh, L.Ysc, 0, in, out, c->stream);
   } else {
-    const MgLevel& L = mg->lev[l];
-    launch_coarse_apply(CoarseGeom{L.E0, L.E1, L.nc}, L.Y, 0, in, out, c->stream, skip,
-                        c->timing ? c->exec + l : nullptr);
+    coarse_op(mg, l, 0, in, out, skip);
   }
   timing_end(c, tk);
 }
 void level_opdag(sw_mg* mg, int l, const double2* in, double2* out, const int* skip = nullptr) {
   sw_ctx* c = mg->ctx;
-  const MgLevel& L = mg->lev[l];
   int tk = timing_begin(c, l);
-  launch_coarse_apply(CoarseGeom{L.E0, L.E1, L.nc}, L.Y, 1, in, out, c->stream, skip,
-                      c->timing ? c->exec + l : nullptr);
+  coarse_op(mg, l, 1, in, out, skip);
   timing_end(c, tk);
 }
 // Normal operator used by the setup on level l: A A^dag (full fine vectors on
@@ -310,9 +319,8 @@ class SmLease {
   int dev_, n_ = 0;
 };
 
-// Autotuner records, keyed by (device, nc, batch width, coarse sites, SMs used): for the
-// batched tensor-core kernel the pipeline depth, for the single-right-hand-side
-// FP64 kernel (width 1) its variant (0: four-FMA, 1: three-FMA products).
+// Autotuner records, keyed by (device, nc, batch width, coarse sites, SMs used): the
+// pipeline depth of the batched tensor-core kernel.
 struct TuneRec {
   int stages;
   double us_per_iter;
@@ -320,85 +328,23 @@ struct TuneRec {
 static std::mutex g_tune_mutex;
 static std::map<std::tuple<int, int, int, int, int>, TuneRec> g_tune;  // + SMs used
 
-// Variant of the FP64 coarsest CGNE for this level, chosen on first use per
-// (device, nc, sites) by timing each for a few iterations on the call's own
-// data (the real solve then starts from scratch).
-static int cgne64_variant(sw_mg* mg, MgLevel& L, const double2* b, double2* x, int sms) {
-  sw_ctx* c = mg->ctx;
-  // "0" .. "3" or "7": skip the timing, use this one
-  const char* force = std::getenv("SW_CGNE64");
-  if (force && ((force[0] >= '0' && force[0] <= '3') || force[0] == '7') && !force[1] &&
-      (force[0] != '7' || cgne64_staged_supported(L.nc)))
-    return force[0] - '0';
-  const auto key = std::make_tuple(c->device, L.nc, 1, L.E0 * L.E1, sms);
-  {
-    std::lock_guard<std::mutex> lk(g_tune_mutex);
-    auto it = g_tune.find(key);
-    if (it != g_tune.end()) return it->second.stages;
-  }
-  constexpr int kTuneIters = 8, kReps = 2;
-  cudaEvent_t e0, e1;
-  SW_CUDA(cudaEventCreate(&e0));
-  SW_CUDA(cudaEventCreate(&e1));
-  TuneRec best{0, 1e30};
-  int cand[5] = {0, 1, 2, 3, 7};
-  const int ncand = cgne64_staged_supported(L.nc) ? 5 : 4;
-  for (int ci = 0; ci < ncand; ++ci) {
-    const int v = cand[ci];
-    float tot = 0.f;
-    for (int rep = 0; rep <= kReps; ++rep) {  // rep 0 is a warm-up
-      SW_CUDA(cudaEventRecord(e0, c->stream));
-      bool ran = launch_cgne64(CoarseGeom{L.E0, L.E1, L.nc}, v, L.Y, L.Ys, b, x, L.gr, L.cp,
-                               L.c4, c->partials, c->bar, c->cgstat, kTuneIters, 0.0, c->device,
-                               c->stream, 0, sms);
-      SW_CUDA(cudaEventRecord(e1, c->stream));
-      SW_CUDA(cudaEventSynchronize(e1));
-      SW_REQUIRE(ran, SW_ERR_ARG, "FP64 coarsest CGNE has no variant for this shape");
-      int st[3];
-      SW_CUDA(cudaMemcpy(st, c->cgstat, sizeof(st), cudaMemcpyDeviceToHost));
-      SW_REQUIRE(st[1] == 0, SW_ERR_TIMEOUT, "coarsest CGNE: a grid barrier wait gave up");
-      float ms = 0.f;
-      SW_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-      if (rep > 0) tot += ms;
-    }
-    const double us = 1e3 * tot / kReps / kTuneIters;
-    if (us < best.us_per_iter) best = TuneRec{v, us};
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  std::lock_guard<std::mutex> lk(g_tune_mutex);
-  g_tune[key] = best;
-  return best.stages;
-}
-
 static int cgne(sw_mg* mg, int l, const double2* b, double2* x) {
   sw_ctx* c = mg->ctx;
   MgLevel& L = mg->lev[l];
   long n = level_len(mg, l);
   if (mg->persistent_cgne) {
     SmLease lease(c);  // held until the kernel has finished
-    int tk = -1;
     const char* dfenv = std::getenv("SW_COARSEST_DF64");
-    bool df = mg->mixed && L.Ydf && (!(L.Ys && L.c4) || (dfenv && dfenv[0] == '1'));
-    bool ran;
-    if (!df && L.Ys && L.c4) {
-      const int v = cgne64_variant(mg, L, b, x, lease.sms());
-      tk = timing_begin(c, kCatCgne);  // the bracket covers the solve, not the tuning
-      ran = launch_cgne64(CoarseGeom{L.E0, L.E1, L.nc}, v, L.Y, L.Ys, b, x, L.gr, L.cp, L.c4,
-                          c->partials, c->bar, c->cgstat, mg->p.coarsest_maxiter,
-                          mg->p.coarsest_tol, c->device, c->stream, mg->stall_test,
-                          lease.sms());
-    }
-    else {
-      tk = timing_begin(c, kCatCgne);
-      ran = launch_cgne_persistent(CoarseGeom{L.E0, L.E1, L.nc}, df ? (const void*)L.Ydf
-                                                                   : (const void*)L.Y,
-                                   df ? 1 : 0, b, x, L.gr, L.cp, L.cdf,
-                                   L.cdf ? L.cdf + L.ndof : nullptr,
-                                   c->partials, c->bar, c->cgstat, mg->p.coarsest_maxiter,
-                                   mg->p.coarsest_tol, c->device, c->stream, mg->stall_test,
-                                   lease.sms());
-    }
+    const CoarseGeom cg{L.E0, L.E1, L.nc};
+    const int tk = timing_begin(c, kCatCgne);
+    bool ran = mg->mixed && L.Ydf && dfenv && dfenv[0] == '1' &&
+               launch_cgne_df(cg, L.Ydf, b, x, L.gr, L.cp, L.cdf, L.cdf + L.ndof, c->partials,
+                              c->bar, c->cgstat, mg->p.coarsest_maxiter, mg->p.coarsest_tol,
+                              c->device, c->stream, mg->stall_test, lease.sms());
+    if (!ran && L.dg.T)
+      ran = launch_cgne64(cg, L.dg, b, x, L.gr, L.cp, c->partials, c->bar, c->cgstat,
+                          mg->p.coarsest_maxiter, mg->p.coarsest_tol, c->device, c->stream,
+                          mg->stall_test, lease.sms());
     timing_end(c, tk);
     if (ran) {
       SW_CUDA(cudaMemcpyAsync(c->h_ctl, c->cgstat, 3 * sizeof(int), cudaMemcpyDeviceToHost,
@@ -592,11 +538,16 @@ void mg_setup(sw_mg* mg, const double* const* psi0, uint64_t seed) {
       double2* T = tmp.get((long)L.E0 * L.E1 * 5 * L.nc * 2 * nv);
       launch_build_Y_coarse(CoarseGeom{L.E0, L.E1, L.nc}, L.b0, L.b1, nv, L.Y, L.P, T, C.Y, s);
     }
-    if (l + 2 == mg->nlev && !mg->fine_D && cgne64_supported(C.nc)) {
-      // coarsest level: the sum plane and vector forms of its FP64 CGNE
-      C.Ys = (double*)mg_alloc(mg, (ysz + 1) / 2);
-      launch_sum_planes(C.Y, C.Ys, ysz, s);
-      C.c4 = (double*)mg_alloc(mg, 4 * C.ndof);
+    const CoarseGeom geom{C.E0, C.E1, C.nc};
+    if (digit_entries(geom) <= kMaxDigitEntries) {
+      // digit entries: kept on the coarsest level and by FP64 hierarchies; on the other
+      // levels of a mixed hierarchy only the setup of the next level uses them
+      const bool keep = l + 2 == mg->nlev || !mg->mixed;
+      const long tn = digit_entries(geom), en = (digit_rows(geom) + 3) / 4;
+      uint4* T = (uint4*)(keep ? mg_alloc(mg, tn) : tmp.get(tn));
+      int* ex = (int*)(keep ? mg_alloc(mg, en) : tmp.get(en));
+      launch_pack_digits(geom, C.Y, T, ex, s);
+      C.dg = DigitStencil{T, ex};
     }
     if (mg->mixed) {
       CoarseGeom cg{C.E0, C.E1, C.nc};
@@ -613,6 +564,8 @@ void mg_setup(sw_mg* mg, const double* const* psi0, uint64_t seed) {
     SW_CUDA(cudaStreamSynchronize(s));
     L.sr = L.sp = L.sq = L.st = nullptr;
   }
+  if (mg->mixed)
+    for (int l = 1; l + 1 < mg->nlev; ++l) mg->lev[l].dg = DigitStencil{};
   // solve workspace
   for (int l = 0; l < mg->nlev; ++l) {
     MgLevel& L = mg->lev[l];

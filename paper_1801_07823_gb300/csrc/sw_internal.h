@@ -254,31 +254,30 @@ struct CoarseGeom {
 void launch_coarse_apply(const CoarseGeom& g, const double2* Y, int dagger, const double2* in,
                          double2* out, cudaStream_t s, const int* skip = nullptr,
                          unsigned long long* exec = nullptr);
-// Whole coarsest-level CGNE in one cooperative launch (cgne.cu); false when nc
-// has no compiled variant.
-// Y: complex128 stencil (df64 = 0) or double-float float4 stencil (df64 = 1,
-// then rdf and pdf are n float4 of scratch).
-bool launch_cgne_persistent(const CoarseGeom& g, const void* Y, int df64, const double2* b,
-                            double2* x, double2* r, double2* p, float4* rdf, float4* pdf,
-                            double* partials, unsigned* bar, int* status, int maxit, double tol,
-                            int device, cudaStream_t s, int stall_test = 0,
-                            int sms_use = 1 << 30);
-
-// FP64 coarsest CGNE in one persistent kernel (cgne64.cu).  variant 1: three
-// real FMAs per complex product, reading Ys = Re + Im of every entry of Y
-// (launch_sum_planes); variant 0: four FMAs on Y alone (Ys may be NULL);
-// variants 2 and 3: 0 and 1 with reduce-scatter row sums and a per-component
-// update; variant 7: 3 with its operands staged in shared memory by
-// asynchronous copies (nc a multiple of 32, cgne64_staged_supported).
-// v4: 8 n doubles of 32-byte aligned scratch (forms of r and p).  False when
-// nc has no compiled variant.
-bool cgne64_supported(int nc);
-bool cgne64_staged_supported(int nc);
-void launch_sum_planes(const double2* Y, double* Ys, long n, cudaStream_t s);
-bool launch_cgne64(const CoarseGeom& g, int variant, const double2* Y, const double* Ys,
-                   const double2* b, double2* x, double2* r, double2* p, double* v4,
-                   double* partials, unsigned* bar, int* status, int maxit, double tol,
-                   int device, cudaStream_t s, int stall_test = 0, int sms_use = 1 << 30);
+// A coarse stencil as digit entries (digit.cuh) with the exponent of every row,
+// for FP64 products on the tensor cores (digit.cu).  One copy serves A and A^dag.
+struct DigitStencil {
+  const uint4* T = nullptr;
+  const int* ex = nullptr;
+};
+constexpr long kMaxDigitEntries = (1L << 31) - (1L << 20);  // their kernels index with 32 bits
+long digit_entries(const CoarseGeom& g);  // of 16 bytes
+long digit_rows(const CoarseGeom& g);     // exponents
+void launch_pack_digits(const CoarseGeom& g, const double2* Y, uint4* T, int* ex, cudaStream_t s);
+void launch_digit_apply(const CoarseGeom& g, const DigitStencil& t, const double2* Y, int dagger,
+                        const double2* in, double2* out, int device, cudaStream_t s,
+                        const int* skip = nullptr, unsigned long long* exec = nullptr);
+// Whole coarsest-level CGNE in one cooperative launch: FP64 on digit entries
+// (cgne64.cu), or with a double-float stencil (cgne.cu; rdf, pdf: n float4 of
+// scratch; false when nc has no compiled variant).
+bool launch_cgne64(const CoarseGeom& g, const DigitStencil& t, const double2* b, double2* x,
+                   double2* r, double2* p, double* partials, unsigned* bar, int* status, int maxit,
+                   double tol, int device, cudaStream_t s, int stall_test = 0,
+                   int sms_use = 1 << 30);
+bool launch_cgne_df(const CoarseGeom& g, const float4* Y, const double2* b, double2* x, double2* r,
+                    double2* p, float4* rdf, float4* pdf, double* partials, unsigned* bar,
+                    int* status, int maxit, double tol, int device, cudaStream_t s,
+                    int stall_test = 0, int sms_use = 1 << 30);
 
 // Batched coarsest CGNE (batch_cgne.cu): nb <= 16 right-hand sides, FP32
 // forward stencil Yf and adjoint stencil Yd (launch_adjoint_f32), FP64

@@ -18,8 +18,7 @@ struct MgLevel {
   float* Ysc = nullptr;   // ... with one scale per block
   float4* Ydf = nullptr;  // mixed precision, coarsest level: double-float stencil
   float4* cdf = nullptr;  // [2][ndof] double-float copies of r and p for its CGNE
-  double* Ys = nullptr;   // coarsest level: Re + Im of every stencil entry (FP64 CGNE)
-  double* c4 = nullptr;   // coarsest level: [2][ndof][4] vector forms of its FP64 CGNE
+  DigitStencil dg;        // digit entries of Y: coarsest level, and every level of an FP64 hierarchy
   // setup work vectors
   double2 *sr = nullptr, *sp = nullptr, *sq = nullptr, *st = nullptr;
   // solve work vectors

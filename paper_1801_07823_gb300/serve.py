@@ -54,8 +54,9 @@ def hierarchy_bytes(L: int, blocks, nvec, mixed: bool, outer_restart: int = 32,
         last = l == len(nvec) - 1
         ysz = sites * 5 * nc * nc
         b += ysz * 16                              # Y (FP64)
-        if last:
-            b += ysz * 8 + sites * nc * 64         # sum plane and vector forms of its FP64 CGNE
+        if last or not mixed:                      # digit entries, padded to whole row groups
+            pad = -(-nc // 8) * 8
+            b += sites * 5 * pad * pad * 16 + sites * pad * 4
         if mixed:
             b += ysz * (16 if last else 4) + sites * 5 * 4
         nb = 0 if last else inter_restart
