@@ -71,6 +71,18 @@ T* dmalloc(size_t count) {
   return (T*)p;
 }
 
+bool disjoint(const void* a, const void* b, size_t bytes) {
+  const char *x = (const char*)a, *y = (const char*)b;
+  return x + bytes <= y || y + bytes <= x;
+}
+// Whether a kernel may work on a caller's two fields themselves: device memory, aligned for
+// 16-byte accesses, not overlapping.
+bool direct(const void* in, size_t nin, const void* out, size_t nout, int on_device) {
+  const char *x = (const char*)in, *y = (const char*)out;
+  return on_device && (((size_t)x | (size_t)y) & 15) == 0 &&
+         (x + nin * sizeof(double2) <= y || y + nout * sizeof(double2) <= x);
+}
+
 void gauge_binv(sw_gauge* g, double mass) {
   if (!g->binv) g->binv = dmalloc<double2>((size_t)g->N * 4);
   if (g->binv_mass != mass) {
@@ -326,22 +338,21 @@ int sw_dslash(sw_gauge* g, double mass, int op, int precision, const void* in, v
       else
         launch_dslash_lex32(g, (float)mass, op == SW_OP_DDAG, (const float2*)din, (float2*)dout, s);
     } else {
-      for (int t = 2; t < 4; ++t)
-        if (!g->tmp[t]) g->tmp[t] = dmalloc<double2>(N);
+      if (!g->tmp[2]) g->tmp[2] = dmalloc<double2>(N);
       gauge_binv(g, mass);
-      double2* a = g->tmp[2];
-      double2* b = g->tmp[3];
-      double2* w = (double2*)dout;  // scratch before the final unpack
-      launch_pack(g, (const double2*)din, a, s);
-      if (op == SW_OP_A) {
-        fine_apply_A(g, g->binv, a, b, w, s);
-      } else if (op == SW_OP_ADAG) {
-        fine_apply_Adag(g, g->binv, a, b, s);
-      } else {
-        fine_apply_S(g, g->binv, a, b, w, s);
-        SW_CUDA(cudaMemsetAsync(b + N / 2, 0, N / 2 * sizeof(double2), s));
+      const double2* x = (const double2*)din;
+      double2* y = (double2*)dout;
+      if (!disjoint(x, y, N * sizeof(double2))) {  // the operators read in while they write out
+        if (!g->tmp[3]) g->tmp[3] = dmalloc<double2>(N);
+        SW_CUDA(cudaMemcpyAsync(g->tmp[3], x, N * sizeof(double2), cudaMemcpyDeviceToDevice, s));
+        x = g->tmp[3];
       }
-      launch_unpack(g, b, (double2*)dout, s);
+      if (op == SW_OP_A)
+        fine_lex_A(g, g->binv, x, y, g->tmp[2], s);
+      else if (op == SW_OP_ADAG)
+        fine_lex_Adag(g, g->binv, x, y, s);
+      else
+        fine_lex_S(g, g->binv, x, y, g->tmp[2], s);
     }
     if (!on_device) {
       SW_CUDA(cudaMemcpyAsync(out, dout, N * esz, cudaMemcpyDeviceToHost, s));
@@ -610,24 +621,34 @@ int sw_mg_apply_level(sw_mg* mg, int level, int precision, int dagger, const voi
     sw_gauge* g = mg->g;
     size_t n = level == 1 ? (size_t)g->N : (size_t)L.ndof;
     ScopedBuffers scratch;
-    double2* a = scratch.get(n);
-    double2* b = scratch.get(n);
-    double2* t = scratch.get(n);
-    SW_CUDA(cudaMemcpyAsync(a, in, n * sizeof(double2),
-                            on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+    const double2* a = (const double2*)in;
+    double2* b = (double2*)out;
+    // host fields, and device fields a kernel cannot work on in place, go through copies
+    const bool staged = !direct(in, n, out, n, on_device);
+    if (staged) {
+      double2* t = scratch.get(n);
+      SW_CUDA(cudaMemcpyAsync(t, in, n * sizeof(double2),
+                              on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+      a = t;
+      b = scratch.get(n);
+    }
     if (level == 1) {
       SW_REQUIRE(!dagger, SW_ERR_ARG, "level 1 has no adjoint here");
       SW_REQUIRE(precision == SW_PREC_FP64 || (precision == SW_PREC_FP32 && mg->mixed), SW_ERR_ARG,
                  "level 1: FP64, or FP32 on a mixed-precision hierarchy");
-      launch_pack(g, a, t, s);
-      SW_CUDA(cudaMemsetAsync(a, 0, n * sizeof(double2), s));
-      if (mg->fine_D)
-        launch_dslash_ps(g, mg->mass, 0, t, a, s);
-      else if (precision == SW_PREC_FP64)
-        fine_apply_S(g, mg->binv, t, a, b, s);
-      else
-        fine_apply_S32(g, g->W_ps32, mg->binv32, t, a, mg->s32tmp, s);
-      launch_unpack(g, a, b, s);
+      if (precision == SW_PREC_FP64 && !mg->fine_D) {
+        fine_lex_S(g, mg->binv, a, b, mg->lext, s);
+      } else {
+        double2* t = scratch.get(n);
+        double2* u = scratch.get(n);
+        launch_pack(g, a, t, s);
+        SW_CUDA(cudaMemsetAsync(u, 0, n * sizeof(double2), s));
+        if (mg->fine_D)
+          launch_dslash_ps(g, mg->mass, 0, t, u, s);
+        else
+          fine_apply_S32(g, g->W_ps32, mg->binv32, t, u, mg->s32tmp, s);
+        launch_unpack(g, u, b, s);
+      }
     } else {
       CoarseGeom cg{L.E0, L.E1, L.nc};
       // timed like the solver's applications (category level - 1), kernel only
@@ -648,8 +669,9 @@ int sw_mg_apply_level(sw_mg* mg, int level, int precision, int dagger, const voi
       }
       timing_end(mg->ctx, tk);
     }
-    SW_CUDA(cudaMemcpyAsync(out, b, n * sizeof(double2),
-                            on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
+    if (staged)
+      SW_CUDA(cudaMemcpyAsync(out, b, n * sizeof(double2),
+                              on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
     SW_CUDA(cudaStreamSynchronize(s));
     return SW_OK;
   });
@@ -666,29 +688,29 @@ int sw_mg_transfer(sw_mg* mg, int level, int dir, const void* in, void* out, int
     size_t nf = L.ndof, nc = C.ndof;
     size_t nin = dir == 0 ? nf : nc, nout = dir == 0 ? nc : nf;
     ScopedBuffers scratch;
-    double2* a = scratch.get(nin);
-    double2* b = scratch.get(nout);
-    double2* t = scratch.get(nf);
-    SW_CUDA(cudaMemcpyAsync(a, in, nin * sizeof(double2),
-                            on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-    if (level == 1) {
-      if (dir == 0) {
-        launch_pack(g, a, t, s);
-        launch_restrict_fine(g, L.b0, L.b1, L.nv, L.P, t, b, s, mg->fine_D ? 1 : 0);
-      } else {
-        SW_CUDA(cudaMemsetAsync(t, 0, nf * sizeof(double2), s));
-        launch_prolong_fine(g, L.b0, L.b1, L.nv, L.P, a, t, s, mg->fine_D ? 1 : 0);
-        launch_unpack(g, t, b, s);
-      }
-    } else {
-      CoarseGeom cg{L.E0, L.E1, L.nc};
-      if (dir == 0)
-        launch_restrict_coarse(cg, L.b0, L.b1, L.nv, L.P, a, b, s);
-      else
-        launch_prolong_coarse(cg, L.b0, L.b1, L.nv, L.P, a, b, s);
+    const double2* a = (const double2*)in;
+    double2* b = (double2*)out;
+    const bool staged = !direct(in, nin, out, nout, on_device);
+    if (staged) {
+      double2* t = scratch.get(nin);
+      SW_CUDA(cudaMemcpyAsync(t, in, nin * sizeof(double2),
+                              on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+      a = t;
+      b = scratch.get(nout);
     }
-    SW_CUDA(cudaMemcpyAsync(out, b, nout * sizeof(double2),
-                            on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
+    const int full = mg->fine_D ? 1 : 0;
+    CoarseGeom cg{L.E0, L.E1, L.nc};
+    if (level == 1 && dir == 0)
+      launch_restrict_fine(g, L.b0, L.b1, L.nv, L.P, a, b, s, full, true);
+    else if (level == 1)
+      launch_prolong_fine(g, L.b0, L.b1, L.nv, L.P, a, b, s, full, true);
+    else if (dir == 0)
+      launch_restrict_coarse(cg, L.b0, L.b1, L.nv, L.P, a, b, s);
+    else
+      launch_prolong_coarse(cg, L.b0, L.b1, L.nv, L.P, a, b, s);
+    if (staged)
+      SW_CUDA(cudaMemcpyAsync(out, b, nout * sizeof(double2),
+                              on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
     SW_CUDA(cudaStreamSynchronize(s));
     return SW_OK;
   });

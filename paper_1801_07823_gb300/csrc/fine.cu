@@ -31,9 +31,13 @@ __device__ __forceinline__ void cfmac(double2& acc, double2 a, double2 b) {  // 
 // sg = +1 for D, -1 for D^dag (D - m is anti-Hermitian, Sec. II).
 // One thread per site; consecutive threads take consecutive x0, so every
 // load of in and W is coalesced; neighbour values are re-read from L1/L2.
-template <typename C2, typename R>
+// In FP64 the kernel is bound by the FP64 pipe (two FMAs per clock and SM), so
+// the sum starts from m in(s) and the sign is an operand's: 18 FP64 operations
+// per site, where a separate sum and a final m x + sg h took 20 (2044 x 2052:
+// 149.6 -> 132.8 us).  In FP32 it is bound by HBM.
+template <typename C2, typename R, bool DAG>
 __global__ void __launch_bounds__(256) k_dslash_lex(const C2* __restrict__ in, C2* __restrict__ out,
-                                                    const C2* __restrict__ W, R mass, R sg, int L0,
+                                                    const C2* __restrict__ W, R mass, int L0,
                                                     int L1) {
   int x0 = blockIdx.x * blockDim.x + threadIdx.x;
   int x1 = blockIdx.y;
@@ -49,20 +53,24 @@ __global__ void __launch_bounds__(256) k_dslash_lex(const C2* __restrict__ in, C
   C2 a = __ldg(in + sp0), b = __ldg(in + sm0), c = __ldg(in + sp1), d = __ldg(in + sm1);
   C2 w0 = __ldg(W + s), w1 = __ldg(W + N + s);
   C2 w0m = __ldg(W + sm0), w1m = __ldg(W + N + sm1);
-  R hx = 0, hy = 0;
-  // forward hops: + W x
-  hx = fma(w0.x, a.x, hx); hx = fma(-w0.y, a.y, hx);
-  hy = fma(w0.x, a.y, hy); hy = fma(w0.y, a.x, hy);
-  hx = fma(w1.x, c.x, hx); hx = fma(-w1.y, c.y, hx);
-  hy = fma(w1.x, c.y, hy); hy = fma(w1.y, c.x, hy);
-  // backward hops: - conj(W) x
-  hx = fma(-w0m.x, b.x, hx); hx = fma(-w0m.y, b.y, hx);
-  hy = fma(-w0m.x, b.y, hy); hy = fma(w0m.y, b.x, hy);
-  hx = fma(-w1m.x, d.x, hx); hx = fma(-w1m.y, d.y, hx);
-  hy = fma(-w1m.x, d.y, hy); hy = fma(w1m.y, d.x, hy);
+  R hx = mass * xs.x, hy = mass * xs.y;
+  auto fwd = [&](C2 w, C2 v) {  // +- w v
+    if (DAG) { w.x = -w.x; w.y = -w.y; }
+    hx = fma(w.x, v.x, hx); hx = fma(-w.y, v.y, hx);
+    hy = fma(w.x, v.y, hy); hy = fma(w.y, v.x, hy);
+  };
+  auto bwd = [&](C2 w, C2 v) {  // -+ conj(w) v
+    if (DAG) { w.x = -w.x; w.y = -w.y; }
+    hx = fma(-w.x, v.x, hx); hx = fma(-w.y, v.y, hx);
+    hy = fma(-w.x, v.y, hy); hy = fma(w.y, v.x, hy);
+  };
+  fwd(w0, a);
+  fwd(w1, c);
+  bwd(w0m, b);
+  bwd(w1m, d);
   C2 o;
-  o.x = fma(sg, hx, mass * xs.x);
-  o.y = fma(sg, hy, mass * xs.y);
+  o.x = hx;
+  o.y = hy;
   out[s] = o;
 }
 
@@ -315,6 +323,139 @@ __global__ void k_dslash_ps(const double2* __restrict__ Wps, double mass, double
   out[f] = make_double2(fma(sg, h.x, mass * xs.x), fma(sg, h.y, mass * xs.y));
 }
 
+// ---------------------------------------------------------------------------
+// KD operators on lexicographic fields, for callers that hand over fields in
+// that order: no packing passes, and no division in an index (row of KD blocks
+// = blockIdx.y).  One thread per KD block; its four sites are 32-byte pieces of
+// two rows, whole sectors.  Bound by the FP64 pipe (S: 176 FMAs per pair of
+// blocks, 44 us at 1036 x 1012 at 1.66 FMAs per clock and SM): 97.8 -> 72.5 us
+// there against packing, three kernels on packed halves, a clear and unpacking.
+struct KdBlock {
+  int x0, x1, par;  // corner; parity
+  long b;           // index in the B^-1 table (parity-split)
+};
+// Blocks of parity `par`, or (par < 0) all of them, in row X1.
+__device__ __forceinline__ bool kd_block(int L0, int L1, int par, int X1, KdBlock& k) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int X0 = par < 0 ? i : 2 * i + ((X1 + par) & 1);
+  if (X0 >= L0 / 2) return false;
+  k.x0 = 2 * X0;
+  k.x1 = 2 * X1;
+  k.par = (X0 + X1) & 1;
+  k.b = (long)k.par * ((long)L0 * L1 / 8) + (long)X1 * (L0 >> 2) + (X0 >> 1);
+  return true;
+}
+__device__ __forceinline__ long kd_site(const KdBlock& k, int j, int L0) {
+  return (long)(k.x1 + (j >> 1)) * L0 + k.x0 + (j & 1);
+}
+// C in at site j of a block: the two hops that leave the block.
+__device__ __forceinline__ double2 kd_hop(const double2* __restrict__ W,
+                                          const double2* __restrict__ in, const KdBlock& k, int j,
+                                          int L0, int L1) {
+  const long N = (long)L0 * L1;
+  const int x0 = k.x0 + (j & 1), x1 = k.x1 + (j >> 1);
+  double2 acc = make_double2(0.0, 0.0);
+  auto back = [&](double2 w, double2 v) {
+    acc.x = fma(-w.x, v.x, acc.x);
+    acc.x = fma(-w.y, v.y, acc.x);
+    acc.y = fma(-w.x, v.y, acc.y);
+    acc.y = fma(w.y, v.x, acc.y);
+  };
+  if (j & 1) {
+    const long t = (long)x1 * L0 + (x0 + 1 == L0 ? 0 : x0 + 1);
+    cfma(acc, W[(long)x1 * L0 + x0], in[t]);
+  } else {
+    const long t = (long)x1 * L0 + (x0 == 0 ? L0 - 1 : x0 - 1);
+    back(W[t], in[t]);
+  }
+  if (j >> 1) {
+    const long t = (long)(x1 + 1 == L1 ? 0 : x1 + 1) * L0 + x0;
+    cfma(acc, W[N + (long)x1 * L0 + x0], in[t]);
+  } else {
+    const long t = (long)(x1 == 0 ? L1 - 1 : x1 - 1) * L0 + x0;
+    back(W[N + t], in[t]);
+  }
+  return acc;
+}
+template <bool DAG>
+__device__ __forceinline__ double2 kd_row(const double2* __restrict__ m, int i, const double2 (&u)[4]) {
+  double2 acc = make_double2(0.0, 0.0);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (j == i) {  // real: B - m is anti-Hermitian and couples the two site parities only
+      const double d = m[5 * i].x;
+      acc.x = fma(d, u[i].x, acc.x);
+      acc.y = fma(d, u[i].y, acc.y);
+    } else if (DAG) {
+      cfmac(acc, m[4 * j + i], u[j]);
+    } else {
+      cfma(acc, m[4 * i + j], u[j]);
+    }
+  }
+  return acc;
+}
+// out = B^-1 in on the blocks of parity par (all: par < 0).
+__global__ void __launch_bounds__(128) k_kd_block(const double2* __restrict__ binv, int par,
+                                                  const double2* __restrict__ in,
+                                                  double2* __restrict__ out, int L0, int L1) {
+  KdBlock k;
+  for (int X1 = blockIdx.y; X1 < L1 / 2; X1 += gridDim.y) {
+    if (!kd_block(L0, L1, par, X1, k)) return;
+    double2 u[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) u[j] = in[kd_site(k, j, L0)];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) out[kd_site(k, i, L0)] = kd_row<false>(binv + 16 * k.b, i, u);
+  }
+}
+// out = M C in (DAG: src - M^dag C in) on the blocks of parity par (all: par < 0), M = B^-1.
+template <bool DAG>
+__global__ void __launch_bounds__(128) k_kd_hop_block(const double2* __restrict__ W,
+                                                      const double2* __restrict__ binv, int par,
+                                                      const double2* __restrict__ in,
+                                                      double2* __restrict__ out, int L0, int L1) {
+  KdBlock k;
+  for (int X1 = blockIdx.y; X1 < L1 / 2; X1 += gridDim.y) {
+    if (!kd_block(L0, L1, par, X1, k)) return;
+    double2 u[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) u[j] = kd_hop(W, in, k, j, L0, L1);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const long s = kd_site(k, i, L0);
+      const double2 v = kd_row<DAG>(binv + 16 * k.b, i, u);
+      if (DAG) {
+        const double2 o = in[s];
+        out[s] = make_double2(o.x - v.x, o.y - v.y);
+      } else {
+        out[s] = v;
+      }
+    }
+  }
+}
+// out = src + sign C in; EVEN: on the even blocks, and 0 on the odd block beside each (a
+// thread per pair: a warp of alternating blocks would spend its FP64 issue on idle lanes).
+template <bool EVEN>
+__global__ void __launch_bounds__(128) k_kd_hop(const double2* __restrict__ W, double sign,
+                                                const double2* __restrict__ src,
+                                                const double2* __restrict__ in,
+                                                double2* __restrict__ out, int L0, int L1) {
+  KdBlock k;
+  for (int X1 = blockIdx.y; X1 < L1 / 2; X1 += gridDim.y) {
+    if (!kd_block(L0, L1, EVEN ? 0 : -1, X1, k)) return;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const long s = kd_site(k, j, L0);
+      const double2 c = kd_hop(W, in, k, j, L0, L1);
+      double2 o = src[s];
+      o.x = fma(sign, c.x, o.x);
+      o.y = fma(sign, c.y, o.y);
+      out[s] = o;
+      if (EVEN) out[s + ((k.x0 & 2) ? -2 : 2)] = make_double2(0.0, 0.0);
+    }
+  }
+}
+
 inline int nblocks(long n, int t) { return (int)((n + t - 1) / t); }
 
 }  // namespace
@@ -339,15 +480,15 @@ void launch_dslash_ps(const sw_gauge* g, double mass, int dagger, const double2*
 void launch_dslash_lex(const sw_gauge* g, double mass, int dagger, const double2* in, double2* out,
                        cudaStream_t s) {
   dim3 grid(nblocks(g->L0, 256), g->L1);
-  k_dslash_lex<double2, double><<<grid, 256, 0, s>>>(in, out, g->W_lex, mass, dagger ? -1.0 : 1.0,
-                                                     g->L0, g->L1);
+  auto k = dagger ? k_dslash_lex<double2, double, true> : k_dslash_lex<double2, double, false>;
+  k<<<grid, 256, 0, s>>>(in, out, g->W_lex, mass, g->L0, g->L1);
   SW_LAUNCH_CHECK();
 }
 void launch_dslash_lex32(const sw_gauge* g, float mass, int dagger, const float2* in, float2* out,
                          cudaStream_t s) {
   dim3 grid(nblocks(g->L0, 256), g->L1);
-  k_dslash_lex<float2, float><<<grid, 256, 0, s>>>(in, out, g->W_lex32, mass, dagger ? -1.0f : 1.0f,
-                                                   g->L0, g->L1);
+  auto k = dagger ? k_dslash_lex<float2, float, true> : k_dslash_lex<float2, float, false>;
+  k<<<grid, 256, 0, s>>>(in, out, g->W_lex32, mass, g->L0, g->L1);
   SW_LAUNCH_CHECK();
 }
 void launch_pack(const sw_gauge* g, const double2* lex, double2* ps, cudaStream_t s) {
@@ -410,4 +551,32 @@ void fine_apply_S(const sw_gauge* g, const double2* binv, const double2* in_e, d
   launch_block_apply(g, binv, 0, 0, in_e, tmp, s);
   launch_hop_block(g, binv, 1, 0, 1.0, nullptr, tmp, tmp + half, s);
   launch_hop(g, 0, -1.0, in_e, tmp + half, out_e, s);
+}
+
+static dim3 kd_grid(const sw_gauge* g, bool half) {
+  const int rows = g->L1 / 2;
+  return dim3(nblocks(g->L0 / (half ? 4 : 2), 128), rows < 32768 ? rows : 32768);
+}
+// The same operators on lexicographic fields; tmp must hold N complex, out may be neither in
+// nor tmp.
+void fine_lex_A(const sw_gauge* g, const double2* binv, const double2* in, double2* out,
+                double2* tmp, cudaStream_t s) {
+  k_kd_block<<<kd_grid(g, false), 128, 0, s>>>(binv, -1, in, tmp, g->L0, g->L1);
+  SW_LAUNCH_CHECK();
+  k_kd_hop<false><<<kd_grid(g, false), 128, 0, s>>>(g->W_lex, 1.0, in, tmp, out, g->L0, g->L1);
+  SW_LAUNCH_CHECK();
+}
+void fine_lex_Adag(const sw_gauge* g, const double2* binv, const double2* in, double2* out,
+                   cudaStream_t s) {
+  k_kd_hop_block<true><<<kd_grid(g, false), 128, 0, s>>>(g->W_lex, binv, -1, in, out, g->L0, g->L1);
+  SW_LAUNCH_CHECK();
+}
+void fine_lex_S(const sw_gauge* g, const double2* binv, const double2* in, double2* out,
+                double2* tmp, cudaStream_t s) {
+  k_kd_block<<<kd_grid(g, true), 128, 0, s>>>(binv, 0, in, tmp, g->L0, g->L1);
+  SW_LAUNCH_CHECK();
+  k_kd_hop_block<false><<<kd_grid(g, true), 128, 0, s>>>(g->W_lex, binv, 1, tmp, tmp, g->L0, g->L1);
+  SW_LAUNCH_CHECK();
+  k_kd_hop<true><<<kd_grid(g, true), 128, 0, s>>>(g->W_lex, -1.0, in, tmp, out, g->L0, g->L1);
+  SW_LAUNCH_CHECK();
 }

@@ -7,9 +7,8 @@
 // of fixed size.
 //
 // Scratch layout for N = L0 L1 <= kNoAllocMaxSites (complex128 units):
-//   [0, N)      input packed to parity-split order
-//   [N, 2N)     output in parity-split order (odd half cleared every call)
-//   [2N, 3N)    intermediate vectors of the Schur operator
+//   [0, N)      copy of an input that overlaps the output
+//   [2N, 3N)    intermediate vector of the Schur operator
 //   [3N, 7N)    B^-1 table for the requested mass (rebuilt every call)
 #include <cmath>
 #include <mutex>
@@ -53,15 +52,16 @@ extern "C" int sw_dslash_schur_noalloc(sw_gauge* g, double mass, const void* in,
     cudaStream_t s = c->stream;
     long N = g->N;
     double2* base = noalloc_scratch(c->device);
-    double2* a = base;
-    double2* b = base + N;
     double2* w = base + 2 * N;
     double2* binv = base + 3 * N;
     launch_binv_build(g, mass, binv, s);
-    launch_pack(g, (const double2*)in, a, s);
-    fine_apply_S(g, binv, a, b, w, s);
-    SW_CUDA(cudaMemsetAsync(b + N / 2, 0, N / 2 * sizeof(double2), s));
-    launch_unpack(g, b, (double2*)out, s);
+    const double2* x = (const double2*)in;
+    double2* y = (double2*)out;
+    if (x < y + N && y < x + N) {
+      SW_CUDA(cudaMemcpyAsync(base, x, N * sizeof(double2), cudaMemcpyDeviceToDevice, s));
+      x = base;
+    }
+    fine_lex_S(g, binv, x, y, w, s);
     return SW_OK;
   });
 }

@@ -217,6 +217,14 @@ void fine_apply_Adag(const sw_gauge* g, const double2* binv, const double2* in, 
 void fine_apply_S(const sw_gauge* g, const double2* binv, const double2* in_e, double2* out_e,
                   double2* tmp, cudaStream_t s);
 
+// The same on lexicographic fields (out neither in nor tmp; tmp: N).
+void fine_lex_A(const sw_gauge* g, const double2* binv, const double2* in, double2* out,
+                double2* tmp, cudaStream_t s);
+void fine_lex_Adag(const sw_gauge* g, const double2* binv, const double2* in, double2* out,
+                   cudaStream_t s);
+void fine_lex_S(const sw_gauge* g, const double2* binv, const double2* in, double2* out,
+                double2* tmp, cudaStream_t s);
+
 // ------------------------------------------------------------- blas.cu
 // skip: optional device flag; when it holds a non-zero value the kernel does nothing.
 void blas_dot(sw_ctx* c, const double2* a, const double2* b, long n, int slot,
@@ -327,10 +335,13 @@ void launch_coarse_apply_df(const CoarseGeom& g, const float4* Y, int dagger, co
                             double2* out, cudaStream_t s);
 // Level-1 transfer on the even parity half.  P: [N][nv] parity-split rows.
 // full = 1: full parity-split vectors (fine operator D) instead of the even half.
+// lex: the fine vector is a whole lexicographic field (odd sites ignored, or written as 0).
 void launch_restrict_fine(const sw_gauge* g, int a0, int a1, int nv, const double2* P,
-                          const double2* r_e, double2* out, cudaStream_t s, int full = 0);
+                          const double2* r_e, double2* out, cudaStream_t s, int full = 0,
+                          bool lex = false);
 void launch_prolong_fine(const sw_gauge* g, int a0, int a1, int nv, const double2* P,
-                         const double2* ehat, double2* e_e, cudaStream_t s, int full = 0);
+                         const double2* ehat, double2* e_e, cudaStream_t s, int full = 0,
+                         bool lex = false);
 void launch_build_W_identity(const sw_gauge* g, int nv, const double2* P, double2* Wv,
                              cudaStream_t s);
 // Level >= 2 transfer.  P: [sites][nc][nv].
