@@ -8,11 +8,26 @@
 // and 0 on odd ones, so CG stops when its residual is below m tol ||b||.
 //
 // Layout: half-lattice vectors, site (x0, x1) of parity p at (x1 L0 + x0) / 2.
+//
+// The iteration is one persistent cooperative kernel (k_cg_eo).  As eight
+// launches per iteration it took 55 us at 256^2, most of it launch gaps; now 14.6
+// us, and 13 on any smaller lattice: three barriers (1.2 us each), two sums over
+// the grid with an FP64 division each (1.5 us), three round trips to the L2 and
+// chains of dependent FP64 operations at 64 clocks each.  A CTA owns a contiguous run
+// of the half lattice; per iteration three grid barriers order
+//   A  t_o = D_oe p with p = r + beta p_old formed where it is read (two FMAs per
+//      neighbour instead of one more barrier), and p written in the other buffer
+//   B  q = m^2 p - D_eo t, <p, q>          -> alpha
+//   C  x += alpha p, r -= alpha q, |r|^2   -> beta, stopping test
+// Every CTA forms the two scalars from all CTAs' parts in the same order.
 #include <chrono>
 #include <cmath>
 #include <cstring>
 
-#include "sw_internal.h"
+#include <atomic>
+
+#include "lease.h"
+#include "sums.cuh"
 
 namespace {
 
@@ -79,6 +94,213 @@ void hop_eo(const sw_gauge* g, int par, double a, const double2* src, double c, 
   SW_LAUNCH_CHECK();
 }
 
+// ---------------------------------------------------------------- the iteration
+constexpr int kCgThreads = 512;
+constexpr int kCgWarps = kCgThreads / 32;
+constexpr long kCgSpins = 1L << 21;
+
+struct CgArgs {
+  const double2* W;
+  double2 *x, *r, *q, *t;
+  double2* p[2];
+  double* partials;  // [2][gridDim.x]
+  unsigned* bar;     // monotone arrival counter
+  int* status;       // [0] iterations, [1] barrier timeout, [2] non-finite residual
+  int L0, L1, maxit;
+  double m2, rr, stop;
+};
+struct CgShared {
+  swsum::Aligned sum[kCgWarps];
+  double total;
+  int ok;
+};
+
+// Neighbours of site h of the half of parity par: half-lattice indices of the
+// other parity (forward 0, 1, backward 0, 1), and the lexicographic sites of the
+// links between.
+struct CgSite {
+  long s, sm0, sm1;
+  int n[4];
+};
+__device__ __forceinline__ CgSite cg_site(int h, int par, int L0, int L1) {
+  const int half = L0 >> 1;
+  const int x1 = h / half, x0 = 2 * (h - x1 * half) + ((x1 + par) & 1);
+  const long row = (long)x1 * L0;
+  CgSite c;
+  c.s = row + x0;
+  const long sp0 = row + (x0 + 1 == L0 ? 0 : x0 + 1);
+  const long sp1 = (x1 + 1 == L1 ? 0 : row + L0) + x0;
+  c.sm0 = row + (x0 == 0 ? L0 - 1 : x0 - 1);
+  c.sm1 = (x1 == 0 ? (long)(L1 - 1) * L0 : row - L0) + x0;
+  c.n[0] = (int)(sp0 >> 1);
+  c.n[1] = (int)(sp1 >> 1);
+  c.n[2] = (int)(c.sm0 >> 1);
+  c.n[3] = (int)(c.sm1 >> 1);
+  return c;
+}
+// sum_mu [W_mu(s) v(s+mu) - conj(W_mu(s-mu)) v(s-mu)]
+__device__ __forceinline__ double2 cg_hop(const double2* __restrict__ W, long N, const CgSite& c,
+                                          const double2 (&v)[4]) {
+  double2 h = make_double2(0.0, 0.0);
+  cfma(h, __ldg(W + c.s), v[0]);
+  cfma(h, __ldg(W + N + c.s), v[1]);
+  auto back = [&](double2 w, double2 u) {
+    h.x = fma(-w.x, u.x, h.x);
+    h.x = fma(-w.y, u.y, h.x);
+    h.y = fma(-w.x, u.y, h.y);
+    h.y = fma(w.y, u.x, h.y);
+  };
+  back(__ldg(W + c.sm0), v[2]);
+  back(__ldg(W + N + c.sm1), v[3]);
+  return h;
+}
+
+// Grid barrier; with parts: also the sum over the grid of every thread's v (in sh.total).
+// False if a wait gave up here or elsewhere.
+__device__ bool cg_barrier(const CgArgs& a, CgShared& sh, unsigned gen, double v, double* parts) {
+  if (parts) {
+    const swsum::Aligned w = swsum::warp_sum(v);
+    if ((threadIdx.x & 31) == 0) sh.sum[threadIdx.x >> 5] = w;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (parts) parts[blockIdx.x] = swsum::total<kCgWarps>(sh.sum);
+    __threadfence();
+    atomicAdd(a.bar, 1u);
+    const unsigned target = gen * gridDim.x;
+    unsigned n;
+    long spins = 0;
+    for (;;) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(a.bar) : "memory");
+      if (n >= target) break;
+      if (++spins > kCgSpins) {
+        atomicExch(a.status + 1, 1);
+        break;
+      }
+    }
+    __threadfence();
+    sh.ok = *((volatile int*)(a.status + 1)) == 0;
+  }
+  if (parts) {
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      const double s = swsum::grid_total(parts, gridDim.x);
+      if (threadIdx.x == 0) sh.total = s;
+    }
+  }
+  __syncthreads();
+  return sh.ok;
+}
+
+__global__ void __launch_bounds__(kCgThreads, 1) k_cg_eo(CgArgs a) {
+  __shared__ CgShared sh;
+  __shared__ double coef;
+  const long N = (long)a.L0 * a.L1, half = N / 2;
+  const int h0 = (int)(half * blockIdx.x / gridDim.x), h1 = (int)(half * (blockIdx.x + 1) / gridDim.x);
+  double rr = a.rr, beta = 0.0;
+  unsigned gen = 0;
+  int k = 0;
+  for (;;) {
+    const double2* po = a.p[k & 1];
+    double2* pn = a.p[(k + 1) & 1];
+    for (int h = h0 + threadIdx.x; h < h1; h += kCgThreads) {
+      const CgSite c = cg_site(h, 1, a.L0, a.L1);
+      double2 v[4], w[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = __ldcg(a.r + c.n[j]);
+      double2 own = __ldcg(a.r + h);
+      if (k > 0) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[j] = __ldcg(po + c.n[j]);
+        const double2 o = __ldcg(po + h);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          v[j].x = fma(beta, w[j].x, v[j].x);
+          v[j].y = fma(beta, w[j].y, v[j].y);
+        }
+        own.x = fma(beta, o.x, own.x);
+        own.y = fma(beta, o.y, own.y);
+      }
+      pn[h] = own;
+      a.t[h] = cg_hop(a.W, N, c, v);
+    }
+    if (!cg_barrier(a, sh, ++gen, 0.0, nullptr)) return;
+    double acc = 0.0;
+    for (int h = h0 + threadIdx.x; h < h1; h += kCgThreads) {
+      const CgSite c = cg_site(h, 0, a.L0, a.L1);
+      double2 v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = __ldcg(a.t + c.n[j]);
+      const double2 p = __ldcg(pn + h), d = cg_hop(a.W, N, c, v);
+      const double2 q = make_double2(fma(a.m2, p.x, -d.x), fma(a.m2, p.y, -d.y));
+      a.q[h] = q;
+      acc = fma(p.x, q.x, fma(p.y, q.y, acc));
+    }
+    if (!cg_barrier(a, sh, ++gen, acc, a.partials)) return;
+    if (threadIdx.x == 0) coef = rr / sh.total;  // alpha
+    __syncthreads();
+    const double alpha = coef;
+    acc = 0.0;
+    for (int h = h0 + threadIdx.x; h < h1; h += kCgThreads) {
+      const double2 p = __ldcg(pn + h), q = __ldcg(a.q + h);
+      double2 x = __ldcg(a.x + h), r = __ldcg(a.r + h);
+      x.x = fma(alpha, p.x, x.x);
+      x.y = fma(alpha, p.y, x.y);
+      r.x = fma(-alpha, q.x, r.x);
+      r.y = fma(-alpha, q.y, r.y);
+      a.x[h] = x;
+      a.r[h] = r;
+      acc = fma(r.x, r.x, fma(r.y, r.y, acc));
+    }
+    if (!cg_barrier(a, sh, ++gen, acc, a.partials + gridDim.x)) return;
+    ++k;
+    const double rn = sh.total;
+    if (!isfinite(rn) || k >= a.maxit || !(sqrt(rn) > a.stop)) {
+      if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.status[0] = k;
+        if (!isfinite(rn)) a.status[2] = 1;
+      }
+      return;
+    }
+    if (threadIdx.x == 0) coef = rn / rr;  // beta
+    __syncthreads();
+    beta = coef;
+    rr = rn;
+  }
+}
+
+// Runs CG from the residual a.r (rr = |r|^2) for at most a.maxit iterations; returns them.
+int run_cg_eo(sw_ctx* c, CgArgs a) {
+  static std::atomic<bool> checked[64];
+  SmLease lease(c);  // held until the kernel has finished
+  if (!checked[c->device & 63].load()) {
+    int coop = 0, occ = 0;
+    SW_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device));
+    SW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg_eo, kCgThreads, 0));
+    SW_REQUIRE(coop && occ >= 1, SW_ERR_CUDA, "the device cannot run the persistent CG kernel");
+    checked[c->device & 63].store(true);
+  }
+  // one CTA per SM; fewer where a CTA would have less than a warp of sites
+  const long half = (long)a.L0 * a.L1 / 2;
+  long grid = (half + 31) / 32;
+  if (grid > lease.sms()) grid = lease.sms();
+  if (grid > kReduceBlocks) grid = kReduceBlocks;
+  a.partials = c->partials;
+  a.bar = c->bar;
+  a.status = c->cgstat;
+  SW_CUDA(cudaMemsetAsync(a.bar, 0, 2 * sizeof(unsigned), c->stream));
+  SW_CUDA(cudaMemsetAsync(a.status, 0, 3 * sizeof(int), c->stream));
+  void* params[] = {&a};
+  SW_CUDA(cudaLaunchCooperativeKernel((const void*)k_cg_eo, dim3((unsigned)grid), dim3(kCgThreads),
+                                      params, 0, c->stream));
+  sw_count_launch();
+  SW_CUDA(cudaMemcpyAsync(c->h_ctl, c->cgstat, 3 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  SW_CUDA(cudaStreamSynchronize(c->stream));
+  if (c->h_ctl[1]) throw SwError{SW_ERR_TIMEOUT, "even/odd CG: a grid barrier wait gave up"};
+  if (c->h_ctl[2]) throw SwError{SW_ERR_NAN, "non-finite CG residual"};
+  return c->h_ctl[0];
+}
+
 }  // namespace
 
 // Solves D x = b by CG on the even normal system; b, x lexicographic device
@@ -102,7 +324,6 @@ int cg_eo_device(sw_gauge* g, double m, const double2* b, double2* x, double tol
   hop_eo(g, 0, m, be, -1.0, bo, be, s);
   blas_zero(c, xe, h);
   double stop = bn > 0.0 ? tol * m * bn : 0.0;
-  int* ctl = c->ctl + 4 * 7;
   int total = 0;
   // CG with reliable restarts: when the recurrence residual meets the target,
   // the true residual rhs - M x_e is recomputed; if it is still above the
@@ -111,32 +332,25 @@ int cg_eo_device(sw_gauge* g, double m, const double2* b, double2* x, double tol
     hop_eo(g, 1, 0.0, nullptr, 1.0, xe, t, s);
     hop_eo(g, 0, m * m, xe, -1.0, t, q, s);
     blas_sub(c, r, be, q, h);
-    blas_copy(c, p, r, h);
     blas_norm2(c, r, h, sb + 1);
     double rr0 = slot_read(c, sb + 1).x;
     if (!std::isfinite(rr0)) throw SwError{SW_ERR_NAN, "non-finite CG residual"};
     if (std::sqrt(rr0) <= stop) break;
-    int budget = maxit - total;
-    iter_init(c, ctl, sb + 1, stop, budget);
-    int cur = 0, s_rr[2] = {sb + 1, sb + 2}, s_pq = sb + 3;
-    for (int issued = 0;;) {
-      for (int qq = 0; qq < 8 && issued < budget; ++qq, ++issued) {
-        // q = (m^2 - D_eo D_oe) p
-        hop_eo(g, 1, 0.0, nullptr, 1.0, p, t, s);      // t_o = D_oe p
-        hop_eo(g, 0, m * m, p, -1.0, t, q, s);          // q = m^2 p - D_eo t
-        blas_dot(c, p, q, h, s_pq, ctl);
-        blas_axpy(c, xe, p, h, coef_ratio(s_rr[cur], s_pq, 1.0), ctl);
-        blas_axpy(c, r, q, h, coef_ratio(s_rr[cur], s_pq, -1.0), ctl);
-        blas_norm2(c, r, h, s_rr[1 - cur], ctl);
-        iter_check(c, ctl, s_rr[1 - cur], stop, budget);
-        blas_xpay(c, p, r, h, coef_ratio(s_rr[1 - cur], s_rr[cur], 1.0), ctl);
-        cur = 1 - cur;
-      }
-      iter_read(c, ctl, c->h_ctl);
-      if (c->h_ctl[2]) throw SwError{SW_ERR_NAN, "non-finite CG residual"};
-      if (c->h_ctl[0] || issued >= budget) break;
-    }
-    total += c->h_ctl[1];
+    CgArgs a{};
+    a.W = g->W_lex;
+    a.x = xe;
+    a.r = r;
+    a.q = q;
+    a.t = t;
+    a.p[0] = full;  // overwritten by the residual check afterwards
+    a.p[1] = p;
+    a.L0 = g->L0;
+    a.L1 = g->L1;
+    a.maxit = maxit - total;
+    a.m2 = m * m;
+    a.rr = rr0;
+    a.stop = stop;
+    total += run_cg_eo(c, a);
   }
   *iters = total;
   // x_o = (b_o - D_oe x_e) / m

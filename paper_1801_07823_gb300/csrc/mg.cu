@@ -22,11 +22,11 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <condition_variable>
 #include <map>
 #include <mutex>
 #include <tuple>
 
+#include "lease.h"
 #include "sw_internal.h"
 #include "sw_mg.h"
 
@@ -275,49 +275,6 @@ static GcrResult fgcr(sw_mg* mg, int l, const double2* b, double2* x, double tol
 // iterations need no host round trip.  Iterates and counts are those of the
 // sequential loop: every kernel after the stopping iteration is a no-op.
 constexpr int kIterBatch = 8;
-
-// SMs that persistent (cooperative) kernels of this process hold, per device.
-// A persistent launch takes its context's share of the SMs (sw_context_set_
-// sm_share; all of them by default) and waits while the kernels of other
-// contexts hold too many for it to fit beside them.  Grids whose shares add
-// up to at most the SM count run concurrently (one CTA per SM each); others
-// run one after the other, so no cooperative grid waits at a barrier for CTAs
-// that cannot become resident.
-class SmLease {
- public:
-  explicit SmLease(sw_ctx* c) : dev_(c->device & 63) {
-    int total = 0;
-    SW_CUDA(cudaDeviceGetAttribute(&total, cudaDevAttrMultiProcessorCount, c->device));
-    n_ = (int)((long)total * c->sm_num / (c->sm_den > 0 ? c->sm_den : 1));
-    n_ = n_ < 1 ? 1 : (n_ > total ? total : n_);
-    std::unique_lock<std::mutex> lk(mu());
-    cv().wait(lk, [&] { return used()[dev_] + n_ <= total; });
-    used()[dev_] += n_;
-  }
-  ~SmLease() {
-    {
-      std::lock_guard<std::mutex> lk(mu());
-      used()[dev_] -= n_;
-    }
-    cv().notify_all();
-  }
-  int sms() const { return n_; }
-
- private:
-  static std::mutex& mu() {
-    static std::mutex m;
-    return m;
-  }
-  static std::condition_variable& cv() {
-    static std::condition_variable v;
-    return v;
-  }
-  static int* used() {
-    static int u[64] = {0};
-    return u;
-  }
-  int dev_, n_ = 0;
-};
 
 // Autotuner records, keyed by (device, nc, batch width, coarse sites, SMs used): the
 // pipeline depth of the batched tensor-core kernel.

@@ -104,3 +104,26 @@ def test_level_calls_on_device_fields(sw, torch, L0, L1, block, nvec, fine_d):
     g.free()
     ctx.free()
 
+
+# one CTA, part of a CTA's warps idle, ragged runs, several sites per thread; a few SMs only
+@pytest.mark.parametrize("L0,L1,den", [(4, 4, 1), (4, 12, 1), (20, 12, 1), (64, 128, 1),
+                                       (64, 64, 76), (32, 32, 152)])
+def test_even_odd_cg_sizes(sw, L0, L1, den):
+    m = 0.05
+    th = si.heatbath_u1(L0, L1, 6.0, 10, seed=3, device="cuda")
+    ctx = sw.sw_context_create(0)
+    sw.sw_context_set_sm_share(ctx, 1, den)
+    g = sw.sw_gauge_load(ctx, th)
+    b = si.gaussian_complex(7, L0 * L1)
+    D = operators.dirac(th, m)
+    for cap in (1, 2, 100000):
+        x = np.zeros_like(b)
+        st = sw.sw_cg_eo_solve(g, m, b, x, 1e-10, cap, allow_noconv=True)
+        r = np.linalg.norm(b - D @ x) / np.linalg.norm(b)
+        assert st["outer_iters"] <= cap and abs(r - st["true_resid"]) <= 1e-12
+    assert st["converged"] and r <= 1e-10
+    b[3] = np.nan
+    with pytest.raises(sw.SwError):
+        sw.sw_cg_eo_solve(g, m, b, x, 1e-10)
+    g.free()
+    ctx.free()
