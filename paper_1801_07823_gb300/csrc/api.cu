@@ -10,6 +10,7 @@
 #include <new>
 
 #include "sw_internal.h"
+#include "many.h"
 #include "sw_mg.h"
 
 void report_stale_error(cudaError_t e) {
@@ -183,6 +184,12 @@ int sw_context_create(int device, void* cuda_stream, sw_ctx** out) {
     c->bar = dmalloc<unsigned>(2);
     c->cgstat = dmalloc<int>(4);
     c->exec = dmalloc<unsigned long long>(kTimeCats);
+    c->many_partials = dmalloc<double>(4 * kManyBlocks * kMaxBatch);
+    c->many_counters = dmalloc<unsigned>(kMaxBatch);
+    c->many_ctl = dmalloc<int>(4 * kMaxBatch);
+    SW_CUDA(cudaMemset(c->many_counters, 0, kMaxBatch * sizeof(unsigned)));
+    SW_CUDA(cudaMallocHost(&c->h_many, sizeof(HostMany)));
+    std::memset(c->h_many, 0, sizeof(HostMany));
     SW_CUDA(cudaMemset(c->ctl, 0, 4 * 8 * sizeof(int)));
     SW_CUDA(cudaMemset(c->exec, 0, kTimeCats * sizeof(unsigned long long)));
     SW_CUDA(cudaMallocHost(&c->h_ctl, 4 * sizeof(int)));
@@ -215,10 +222,14 @@ void sw_context_free(sw_ctx* c) {
   dev_free(c->flag, "flag");
   dev_free(c->ctl, "ctl");
   dev_free(c->exec, "exec");
+  dev_free(c->many_partials, "partials");
+  dev_free(c->many_counters, "counters");
+  dev_free(c->many_ctl, "ctl");
   dev_free(c->bar, "bar");
   dev_free(c->cgstat, "cgstat");
   if (c->h_slots) cudaFreeHost(c->h_slots);
   if (c->h_ctl) cudaFreeHost(c->h_ctl);
+  if (c->h_many) cudaFreeHost(c->h_many);
   delete c;
 }
 
@@ -646,7 +657,7 @@ int sw_mg_apply_level(sw_mg* mg, int level, int precision, int dagger, const voi
         if (mg->fine_D)
           launch_dslash_ps(g, mg->mass, 0, t, u, s);
         else
-          fine_apply_S32(g, g->W_ps32, mg->binv32, t, u, mg->s32tmp, s);
+          many_S32(g, g->W_ps32, mg->binv32, Many<3>(0, t, u, mg->lext), s);
         launch_unpack(g, u, b, s);
       }
     } else {
@@ -701,13 +712,13 @@ int sw_mg_transfer(sw_mg* mg, int level, int dir, const void* in, void* out, int
     const int full = mg->fine_D ? 1 : 0;
     CoarseGeom cg{L.E0, L.E1, L.nc};
     if (level == 1 && dir == 0)
-      launch_restrict_fine(g, L.b0, L.b1, L.nv, L.P, a, b, s, full, true);
+      many_restrict_fine(g, L.b0, L.b1, L.nv, L.P, Many<2>(0, a, b), s, full, true);
     else if (level == 1)
-      launch_prolong_fine(g, L.b0, L.b1, L.nv, L.P, a, b, s, full, true);
+      many_prolong_fine(g, L.b0, L.b1, L.nv, L.P, Many<2>(0, a, b), s, full, true);
     else if (dir == 0)
-      launch_restrict_coarse(cg, L.b0, L.b1, L.nv, L.P, a, b, s);
+      many_restrict_coarse(cg, L.b0, L.b1, L.nv, L.P, Many<2>(0, a, b), s);
     else
-      launch_prolong_coarse(cg, L.b0, L.b1, L.nv, L.P, a, b, s);
+      many_prolong_coarse(cg, L.b0, L.b1, L.nv, L.P, Many<2>(0, a, b), s);
     if (staged)
       SW_CUDA(cudaMemcpyAsync(out, b, nout * sizeof(double2),
                               on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));

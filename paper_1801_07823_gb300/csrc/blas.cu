@@ -1,4 +1,5 @@
-// BLAS-1 on complex128 vectors with device-resident Krylov coefficients.
+// BLAS-1 on complex128 vectors with device-resident Krylov coefficients, for
+// single vectors (many.cu has those of the Krylov loops).
 //
 // Reductions are single launches with a fixed grid (at most kReduceBlocks
 // CTAs, chosen from n only): each CTA sums a grid-stride slice with a warp
@@ -15,48 +16,34 @@ __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-// Block-wide sum of two values; result valid in thread 0.
-__device__ __forceinline__ void block_sum2(double& a, double& b) {
-  __shared__ double sa[32], sb[32];
+// Block-wide sum; result valid in thread 0.
+__device__ __forceinline__ double block_sum(double a) {
+  __shared__ double sa[32];
   a = warp_sum(a);
-  b = warp_sum(b);
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   __syncthreads();
-  if (lane == 0) { sa[w] = a; sb[w] = b; }
+  if (lane == 0) sa[w] = a;
   __syncthreads();
-  int nw = blockDim.x >> 5;
-  if (w == 0) {
-    a = lane < nw ? sa[lane] : 0.0;
-    b = lane < nw ? sb[lane] : 0.0;
-    a = warp_sum(a);
-    b = warp_sum(b);
-  }
+  if (w == 0) a = warp_sum(lane < (int)(blockDim.x >> 5) ? sa[lane] : 0.0);
+  return a;
 }
 
-template <int MODE>  // 0: <a, b> = sum conj(a) b;  1: ||a||^2
-__global__ void __launch_bounds__(kThreads) k_reduce(const double2* __restrict__ a,
-                                                     const double2* __restrict__ b, long n,
-                                                     double* partials, unsigned* counter,
-                                                     double2* slots, int slot,
-                                                     const int* __restrict__ skip) {
+// ||a||^2
+__global__ void __launch_bounds__(kThreads) k_norm2(const double2* __restrict__ a, long n,
+                                                    double* partials, unsigned* counter,
+                                                    double2* slots, int slot,
+                                                    const int* __restrict__ skip) {
   if (skip && *skip) return;
-  double re = 0.0, im = 0.0;
+  double re = 0.0;
   long stride = (long)gridDim.x * blockDim.x;
   for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     double2 x = a[i];
-    if (MODE == 0) {
-      double2 y = b[i];
-      re = fma(x.x, y.x, re); re = fma(x.y, y.y, re);
-      im = fma(x.x, y.y, im); im = fma(-x.y, y.x, im);
-    } else {
-      re = fma(x.x, x.x, re); re = fma(x.y, x.y, re);
-    }
+    re = fma(x.x, x.x, re); re = fma(x.y, x.y, re);
   }
-  block_sum2(re, im);
+  re = block_sum(re);
   __shared__ bool last;
   if (threadIdx.x == 0) {
-    partials[2 * blockIdx.x] = re;
-    partials[2 * blockIdx.x + 1] = im;
+    partials[blockIdx.x] = re;
     __threadfence();
     unsigned t = atomicAdd(counter, 1u);
     last = (t == gridDim.x - 1);
@@ -64,15 +51,12 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const double2* __restrict__
   __syncthreads();
   if (last) {
     __threadfence();
-    double r2 = 0.0, i2 = 0.0;
+    double r2 = 0.0;
     const volatile double* vp = partials;
-    for (int j = threadIdx.x; j < (int)gridDim.x; j += blockDim.x) {
-      r2 += vp[2 * j];
-      i2 += vp[2 * j + 1];
-    }
-    block_sum2(r2, i2);
+    for (int j = threadIdx.x; j < (int)gridDim.x; j += blockDim.x) r2 += vp[j];
+    r2 = block_sum(r2);
     if (threadIdx.x == 0) {
-      slots[slot] = make_double2(r2, i2);
+      slots[slot] = make_double2(r2, 0.0);
       *counter = 0u;
     }
   }
@@ -100,13 +84,6 @@ __global__ void k_xpay(double2* __restrict__ y, const double2* __restrict__ x, l
   o.y = fma(a.x, v.y, o.y); o.y = fma(a.y, v.x, o.y);
   y[i] = o;
 }
-__global__ void k_scale(double2* __restrict__ y, long n, const double2* __restrict__ S, Coef c) {
-  long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double2 a = coef_eval(S, c);
-  double2 v = y[i];
-  y[i] = make_double2(a.x * v.x - a.y * v.y, a.x * v.y + a.y * v.x);
-}
 __global__ void k_sub(double2* __restrict__ o, const double2* __restrict__ a,
                       const double2* __restrict__ b, long n) {
   long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -114,14 +91,6 @@ __global__ void k_sub(double2* __restrict__ o, const double2* __restrict__ a,
   double2 u = a[i], v = b[i];
   o[i] = make_double2(u.x - v.x, u.y - v.y);
 }
-__global__ void k_add3(double2* __restrict__ o, const double2* __restrict__ a,
-                       const double2* __restrict__ b, const double2* __restrict__ d, long n) {
-  long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double2 u = a[i], v = b[i], w = d[i];
-  o[i] = make_double2((u.x + v.x) + w.x, (u.y + v.y) + w.y);
-}
-
 inline int grid_for(long n) { return (int)((n + kThreads - 1) / kThreads); }
 inline int reduce_grid(long n) {
   long g = (n + kThreads - 1) / kThreads;
@@ -132,14 +101,9 @@ inline int reduce_grid(long n) {
 
 }  // namespace
 
-void blas_dot(sw_ctx* c, const double2* a, const double2* b, long n, int slot, const int* skip) {
-  k_reduce<0><<<reduce_grid(n), kThreads, 0, c->stream>>>(a, b, n, c->partials, c->counter,
-                                                          c->slots, slot, skip);
-  SW_LAUNCH_CHECK();
-}
 void blas_norm2(sw_ctx* c, const double2* a, long n, int slot, const int* skip) {
-  k_reduce<1><<<reduce_grid(n), kThreads, 0, c->stream>>>(a, nullptr, n, c->partials, c->counter,
-                                                          c->slots, slot, skip);
+  k_norm2<<<reduce_grid(n), kThreads, 0, c->stream>>>(a, n, c->partials, c->counter, c->slots, slot,
+                                                      skip);
   SW_LAUNCH_CHECK();
 }
 void blas_axpy(sw_ctx* c, double2* y, const double2* x, long n, Coef a, const int* skip) {
@@ -150,11 +114,6 @@ void blas_axpy(sw_ctx* c, double2* y, const double2* x, long n, Coef a, const in
 void blas_xpay(sw_ctx* c, double2* y, const double2* x, long n, Coef a, const int* skip) {
   if (n <= 0) return;
   k_xpay<<<grid_for(n), kThreads, 0, c->stream>>>(y, x, n, c->slots, a, skip);
-  SW_LAUNCH_CHECK();
-}
-void blas_scale(sw_ctx* c, double2* y, long n, Coef a) {
-  if (n <= 0) return;
-  k_scale<<<grid_for(n), kThreads, 0, c->stream>>>(y, n, c->slots, a);
   SW_LAUNCH_CHECK();
 }
 void blas_copy(sw_ctx* c, double2* y, const double2* x, long n) {
@@ -168,12 +127,6 @@ void blas_zero(sw_ctx* c, double2* y, long n) {
 void blas_sub(sw_ctx* c, double2* out, const double2* a, const double2* b, long n) {
   if (n <= 0) return;
   k_sub<<<grid_for(n), kThreads, 0, c->stream>>>(out, a, b, n);
-  SW_LAUNCH_CHECK();
-}
-void blas_add3(sw_ctx* c, double2* out, const double2* a, const double2* b, const double2* d,
-               long n) {
-  if (n <= 0) return;
-  k_add3<<<grid_for(n), kThreads, 0, c->stream>>>(out, a, b, d, n);
   SW_LAUNCH_CHECK();
 }
 double2 slot_read(sw_ctx* c, int slot) {
@@ -194,9 +147,9 @@ static cudaEvent_t take_event(sw_ctx* c) {
   SW_CUDA(cudaEventCreate(&e));
   return e;
 }
-int timing_begin(sw_ctx* c, int cat) {
+int timing_begin(sw_ctx* c, int cat, int members) {
   if (!c->timing) return -1;
-  TimedPair t{cat, take_event(c), take_event(c)};
+  TimedPair t{cat, members, take_event(c), take_event(c)};
   SW_CUDA(cudaEventRecord(t.a, c->stream));
   c->pending.push_back(t);
   return (int)c->pending.size() - 1;
@@ -210,7 +163,7 @@ void timing_harvest(sw_ctx* c) {
     float ms = 0.f;
     SW_CUDA(cudaEventElapsedTime(&ms, t.a, t.b));
     c->t_ms[t.cat] += ms;
-    c->t_count[t.cat] += 1;
+    c->t_count[t.cat] += t.n;
     c->spare.push_back(t.a);
     c->spare.push_back(t.b);
   }
@@ -247,11 +200,4 @@ void iter_read(sw_ctx* c, const int* ctl, int* host3) {
   SW_CUDA(cudaMemcpyAsync(host3, ctl, 3 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   SW_CUDA(cudaStreamSynchronize(c->stream));
   if (!c->pending.empty()) timing_harvest(c);
-}
-
-void slot_set(sw_ctx* c, int slot, double2 v) {
-  c->h_slots[slot] = v;
-  SW_CUDA(cudaMemcpyAsync(c->slots + slot, c->h_slots + slot, sizeof(double2),
-                          cudaMemcpyHostToDevice, c->stream));
-  SW_CUDA(cudaStreamSynchronize(c->stream));
 }

@@ -12,6 +12,7 @@
 // Direction d collects the couplings carried by fine hops that leave the
 // aggregate in direction d, so the stencil is exact for any coarse extent,
 // including 1 and 2 where X + 0hat and X - 0hat coincide.
+#include "many.h"
 #include "sw_internal.h"
 
 namespace {
@@ -151,12 +152,14 @@ __global__ void __launch_bounds__(5 * NC) k_coarse_apply_nc(const double2* __res
 // through the C ABI on device fields took 339 us with one thread per column,
 // a serial sum over 32 sites and three allocations, and takes 50 us.
 // LEX: r is a lexicographic field.
-template <bool LEX>
+// One member of a batch per blockIdx.y.
+template <bool LEX, int W>
 __global__ void __launch_bounds__(128) k_restrict_fine(const double2* __restrict__ P,
-                                                       const double2* __restrict__ r,
-                                                       double2* __restrict__ out, int L0, int L1,
+                                                       Pack<2, W> io, int L0, int L1,
                                                        int a0, int a1, int nv, int groups,
                                                        int full) {
+  const double2* __restrict__ r = io.v[0][blockIdx.y];
+  double2* __restrict__ out = io.v[1][blockIdx.y];
   __shared__ double2 part[2 * 128];
   const int A = blockIdx.x, E0 = L0 / (2 * a0);
   const int A0 = A % E0, A1 = A / E0;
@@ -214,12 +217,32 @@ __device__ __forceinline__ void coarse_dof_map(long dof, int E0, int nc, int b0,
   c = k >= nc / 2;
 }
 
+// sum_i p[i] e[i] as four chains of FMAs (a dependent FP64 operation waits 64 clocks:
+// one chain of 2 x 24 takes 1.6 us, these 0.5).
+__device__ __forceinline__ double2 row_times(const double2* __restrict__ p,
+                                             const double2* __restrict__ e, int n) {
+  double2 s[4] = {};
+  int i = 0;
+  for (; i + 1 < n; i += 2)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const double2 a = p[i + q], b = e[i + q];
+      s[q].x = fma(a.x, b.x, s[q].x);
+      s[q].y = fma(a.x, b.y, s[q].y);
+      s[2 + q].x = fma(-a.y, b.y, s[2 + q].x);
+      s[2 + q].y = fma(a.y, b.x, s[2 + q].y);
+    }
+  if (i < n) cfma(s[0], p[i], e[i]);
+  return make_double2((s[0].x + s[1].x) + (s[2].x + s[3].x), (s[0].y + s[1].y) + (s[2].y + s[3].y));
+}
+
 // One thread per fine site, in the order of P's rows.  LEX: e is a whole
 // lexicographic field, whose odd sites get 0.
-template <bool LEX>
-__global__ void k_prolong_fine(const double2* __restrict__ P, const double2* __restrict__ ehat,
-                               double2* __restrict__ e, int L0, int L1, int a0, int a1, int nv,
-                               int full) {
+template <bool LEX, int W>
+__global__ void k_prolong_fine(const double2* __restrict__ P, Pack<2, W> io, int L0, int L1, int a0,
+                               int a1, int nv, int full) {
+  const double2* __restrict__ ehat = io.v[0][blockIdx.y];
+  double2* __restrict__ e = io.v[1][blockIdx.y];
   int N = L0 * L1;
   int h = blockIdx.x * blockDim.x + threadIdx.x;
   if (h >= (full || LEX ? N : N / 2)) return;
@@ -229,7 +252,7 @@ __global__ void k_prolong_fine(const double2* __restrict__ P, const double2* __r
     fine_dof_map(h, L0, L1, a0, a1, A, c);
     const double2* p = P + (long)h * nv;
     const double2* eh = ehat + (long)A * 2 * nv + c * nv;
-    for (int i = 0; i < nv; ++i) cfma(acc, p[i], eh[i]);
+    acc = row_times(p, eh, nv);
   }
   if (LEX) {
     int x0, x1;
@@ -262,41 +285,52 @@ __global__ void k_level_maps_coarse(int* __restrict__ agg, int* __restrict__ chi
   chir[dof] = c ? -1 : 1;
 }
 
-// Level >= 2 transfer: chirality sigma3 = + for k < nc/2, - otherwise.
-__global__ void k_restrict_coarse(const double2* __restrict__ P, const double2* __restrict__ r,
-                                  double2* __restrict__ out, int E0, int b0, int b1, int nc,
-                                  int nv) {
-  int A = blockIdx.x;
-  int F0 = E0 / b0;
-  int A0 = A % F0, A1 = A / F0;
-  int t = threadIdx.x;
-  if (t >= 2 * nv) return;
-  int c = t / nv, i = t - c * nv;
-  int hn = nc / 2;
-  double2 acc = make_double2(0.0, 0.0);
-  for (int y = 0; y < b1; ++y)
-    for (int x = 0; x < b0; ++x) {
-      int X = (A0 * b0 + x) + E0 * (A1 * b1 + y);
-      for (int k = c * hn; k < (c + 1) * hn; ++k) {
-        long dof = (long)X * nc + k;
-        cfmac(acc, P[dof * nv + i], r[dof]);
-      }
+// Level >= 2 transfer: chirality sigma3 = + for k < nc/2, - otherwise.  Thread
+// (group, t) sums column t over every nth dof of its chirality in the aggregate,
+// then the groups are added in order: one thread per column took a chain of
+// b0 b1 nc FMAs of 64 clocks each (2 x 2 sites of 24 dof: 3 us, now 1).
+constexpr int kRestrictThreads = 256;
+template <int W>
+__global__ void __launch_bounds__(kRestrictThreads) k_restrict_coarse(const double2* __restrict__ P,
+                                                                      Pack<2, W> io, int E0, int b0,
+                                                                      int b1, int nc, int nv,
+                                                                      int groups) {
+  __shared__ double2 part[kRestrictThreads];
+  const double2* __restrict__ r = io.v[0][blockIdx.y];
+  double2* __restrict__ out = io.v[1][blockIdx.y];
+  const int A = blockIdx.x, F0 = E0 / b0, A0 = A % F0, A1 = A / F0;
+  const int grp = threadIdx.x / (2 * nv), t = threadIdx.x - grp * 2 * nv;
+  const int c = t / nv, i = t - c * nv, hn = nc / 2;
+  if (grp < groups) {
+    double2 acc = make_double2(0.0, 0.0);
+    for (int d = grp; d < b0 * b1 * hn; d += groups) {
+      const int q = d / hn, y = q / b0, x = q - y * b0;
+      const long dof = (long)((A0 * b0 + x) + E0 * (A1 * b1 + y)) * nc + c * hn + (d - q * hn);
+      cfmac(acc, P[dof * nv + i], r[dof]);
     }
-  out[(long)A * 2 * nv + t] = acc;
+    part[threadIdx.x] = acc;
+  }
+  __syncthreads();
+  if (grp > 0) return;
+  double2 s = part[t];
+  for (int q = 1; q < groups; ++q) {
+    const double2 v = part[q * 2 * nv + t];
+    s.x += v.x;
+    s.y += v.y;
+  }
+  out[(long)A * 2 * nv + t] = s;
 }
 
-__global__ void k_prolong_coarse(const double2* __restrict__ P, const double2* __restrict__ ehat,
-                                 double2* __restrict__ e, int E0, int E1, int b0, int b1, int nc,
-                                 int nv) {
+template <int W>
+__global__ void k_prolong_coarse(const double2* __restrict__ P, Pack<2, W> io, int E0, int E1,
+                                 int b0, int b1, int nc, int nv) {
+  const double2* __restrict__ ehat = io.v[0][blockIdx.y];
+  double2* __restrict__ e = io.v[1][blockIdx.y];
   long dof = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (dof >= (long)E0 * E1 * nc) return;
   int A, c;
   coarse_dof_map(dof, E0, nc, b0, b1, A, c);
-  const double2* p = P + dof * nv;
-  const double2* eh = ehat + (long)A * 2 * nv + c * nv;
-  double2 acc = make_double2(0.0, 0.0);
-  for (int i = 0; i < nv; ++i) cfma(acc, p[i], eh[i]);
-  e[dof] = acc;
+  e[dof] = row_times(P + dof * nv, ehat + (long)A * 2 * nv + c * nv, nv);
 }
 
 // ---------------------------------------------------------------------------
@@ -642,34 +676,48 @@ void launch_coarse_apply(const CoarseGeom& g, const double2* Y, int dagger, cons
                                                               dagger, skip, exec);
   SW_LAUNCH_CHECK();
 }
-void launch_restrict_fine(const sw_gauge* g, int a0, int a1, int nv, const double2* P,
-                          const double2* r_e, double2* out, cudaStream_t s, int full, bool lex) {
+void many_restrict_fine(const sw_gauge* g, int a0, int a1, int nv, const double2* P,
+                        const Many<2>& io, cudaStream_t s, int full, bool lex) {
   int nagg = (g->L0 / (2 * a0)) * (g->L1 / (2 * a1));
   const int blocks = a0 * a1 / (full ? 1 : 2);
   const int groups = 128 / nv < blocks ? 128 / nv : blocks;
-  auto k = lex ? k_restrict_fine<true> : k_restrict_fine<false>;
-  k<<<nagg, 128, 0, s>>>(P, r_e, out, g->L0, g->L1, a0, a1, nv, groups, full);
-  SW_LAUNCH_CHECK();
+  with_width(io.n, [&](auto w) {
+    constexpr int W = decltype(w)::value;
+    auto k = lex ? k_restrict_fine<true, W> : k_restrict_fine<false, W>;
+    k<<<dim3(nagg, io.n), 128, 0, s>>>(P, Pack<2, W>(io), g->L0, g->L1, a0, a1, nv, groups, full);
+    SW_LAUNCH_CHECK();
+  });
 }
-void launch_prolong_fine(const sw_gauge* g, int a0, int a1, int nv, const double2* P,
-                         const double2* ehat, double2* e_e, cudaStream_t s, int full, bool lex) {
-  auto k = lex ? k_prolong_fine<true> : k_prolong_fine<false>;
-  k<<<cdiv(full || lex ? g->N : g->N / 2, 128), 128, 0, s>>>(P, ehat, e_e, g->L0, g->L1, a0, a1,
-                                                            nv, full);
-  SW_LAUNCH_CHECK();
+void many_prolong_fine(const sw_gauge* g, int a0, int a1, int nv, const double2* P,
+                       const Many<2>& io, cudaStream_t s, int full, bool lex) {
+  with_width(io.n, [&](auto w) {
+    constexpr int W = decltype(w)::value;
+    auto k = lex ? k_prolong_fine<true, W> : k_prolong_fine<false, W>;
+    k<<<dim3(cdiv(full || lex ? g->N : g->N / 2, 128), io.n), 128, 0, s>>>(
+        P, Pack<2, W>(io), g->L0, g->L1, a0, a1, nv, full);
+    SW_LAUNCH_CHECK();
+  });
 }
-void launch_restrict_coarse(const CoarseGeom& g, int b0, int b1, int nv, const double2* P,
-                            const double2* r, double2* out, cudaStream_t s) {
-  int nagg = (g.E0 / b0) * (g.E1 / b1);
-  int threads = cdiv(2 * nv, 32) * 32;
-  k_restrict_coarse<<<nagg, threads, 0, s>>>(P, r, out, g.E0, b0, b1, g.nc, nv);
-  SW_LAUNCH_CHECK();
+void many_restrict_coarse(const CoarseGeom& g, int b0, int b1, int nv, const double2* P,
+                          const Many<2>& io, cudaStream_t s) {
+  const int nagg = (g.E0 / b0) * (g.E1 / b1), dofs = b0 * b1 * (g.nc / 2);
+  const int groups = kRestrictThreads / (2 * nv) < dofs ? kRestrictThreads / (2 * nv) : dofs;
+  with_width(io.n, [&](auto w) {
+    constexpr int W = decltype(w)::value;
+    k_restrict_coarse<W><<<dim3(nagg, io.n), kRestrictThreads, 0, s>>>(
+        P, Pack<2, W>(io), g.E0, b0, b1, g.nc, nv, groups);
+    SW_LAUNCH_CHECK();
+  });
 }
-void launch_prolong_coarse(const CoarseGeom& g, int b0, int b1, int nv, const double2* P,
-                           const double2* ehat, double2* e, cudaStream_t s) {
+void many_prolong_coarse(const CoarseGeom& g, int b0, int b1, int nv, const double2* P,
+                         const Many<2>& io, cudaStream_t s) {
   long n = (long)g.E0 * g.E1 * g.nc;
-  k_prolong_coarse<<<cdiv(n, 128), 128, 0, s>>>(P, ehat, e, g.E0, g.E1, b0, b1, g.nc, nv);
-  SW_LAUNCH_CHECK();
+  with_width(io.n, [&](auto w) {
+    constexpr int W = decltype(w)::value;
+    k_prolong_coarse<W><<<dim3(cdiv(n, 128), io.n), 128, 0, s>>>(P, Pack<2, W>(io), g.E0, g.E1, b0,
+                                                                 b1, g.nc, nv);
+    SW_LAUNCH_CHECK();
+  });
 }
 void launch_build_W(const sw_gauge* g, int nv, const double2* binv, const double2* P,
                     double2* Wv, cudaStream_t s) {

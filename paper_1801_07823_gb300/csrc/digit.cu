@@ -3,6 +3,7 @@
 #include <atomic>
 
 #include "digit.cuh"
+#include "many.h"
 
 namespace {
 
@@ -51,18 +52,20 @@ constexpr int kCtas = 3;
 constexpr int kPer = 5;     // complex vector elements per thread: nc <= 128
 constexpr int kSupers = 16 / kGroups;
 
-template <bool DAG>
+// One member of a batch per blockIdx.y.
+template <bool DAG, int W>
 __global__ void __launch_bounds__(kNT, kCtas) k_digit_apply(Shape s, const uint4* __restrict__ T,
                                                             const int* __restrict__ ex,
                                                             const double2* __restrict__ Y,
-                                                            const double2* __restrict__ in,
-                                                            double2* __restrict__ out, int parts,
+                                                            Pack<2, W> io, int parts,
                                                             const int* __restrict__ skip,
                                                             unsigned long long* exec) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int em;
   __shared__ Super sup[2][kSupers];  // of this unit and the next
-  if (skip && *skip) return;
+  const double2* __restrict__ in = io.v[0][blockIdx.y];
+  double2* __restrict__ out = io.v[1][blockIdx.y];
+  if (skip && skip[4 * blockIdx.y]) return;
   if (exec && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(exec, 1ull);
   unsigned char* B = smem;
   int4* quads = reinterpret_cast<int4*>(smem + (size_t)s.KS * 4 * kQuadBytes);
@@ -173,26 +176,33 @@ void launch_pack_digits(const CoarseGeom& g, const double2* Y, uint4* T, int* ex
   SW_LAUNCH_CHECK();
 }
 
-void launch_digit_apply(const CoarseGeom& g, const DigitStencil& t, const double2* Y, int dagger,
-                        const double2* in, double2* out, int device, cudaStream_t st,
-                        const int* skip, unsigned long long* exec) {
+void many_digit(const CoarseGeom& g, const DigitStencil& t, const double2* Y, int dagger,
+                const Many<2>& io, int device, cudaStream_t st, const int* ctl,
+                unsigned long long* exec) {
   const Shape s = shape_of(g);
   const int sites = s.E0 * s.E1;
   // rows of a site are split over CTAs while there are fewer units than CTA slots
   int parts = 1;
-  while (2 * parts <= s.RG && (long)sites * parts < kCtas * 152) parts *= 2;
+  while (2 * parts <= s.RG && (long)sites * parts * io.n < kCtas * 152) parts *= 2;
   const int units = sites * parts;
   const size_t smem = (size_t)s.KS * (4 * kQuadBytes + 32) + (size_t)s.RG * kSItem * sizeof(int);
-  static std::atomic<bool> wide[64];
-  if (!wide[device & 63].exchange(true)) {
-    constexpr int most = 40 * (4 * kQuadBytes + 32) + 16 * kSItem * (int)sizeof(int);  // nc = 128
-    for (auto f : {k_digit_apply<true>, k_digit_apply<false>})
-      SW_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-  }
-  const int grid = units < kCtas * 152 ? units : kCtas * 152;
-  if (dagger)
-    k_digit_apply<true><<<grid, kNT, smem, st>>>(s, t.T, t.ex, Y, in, out, parts, skip, exec);
-  else
-    k_digit_apply<false><<<grid, kNT, smem, st>>>(s, t.T, t.ex, Y, in, out, parts, skip, exec);
-  SW_LAUNCH_CHECK();
+  const int slots = (kCtas * 152 + io.n - 1) / io.n;  // per member
+  const dim3 grid(units < slots ? units : slots, io.n);
+  with_width(io.n, [&](auto w) {
+    constexpr int W = decltype(w)::value;
+    static std::atomic<bool> wide[64];
+    if (!wide[device & 63].exchange(true)) {
+      constexpr int most = 40 * (4 * kQuadBytes + 32) + 16 * kSItem * (int)sizeof(int);  // nc = 128
+      for (auto f : {k_digit_apply<true, W>, k_digit_apply<false, W>})
+        SW_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    }
+    auto k = dagger ? k_digit_apply<true, W> : k_digit_apply<false, W>;
+    k<<<grid, kNT, smem, st>>>(s, t.T, t.ex, Y, Pack<2, W>(io), parts, ctl, exec);
+    SW_LAUNCH_CHECK();
+  });
+}
+void launch_digit_apply(const CoarseGeom& g, const DigitStencil& t, const double2* Y, int dagger,
+                        const double2* in, double2* out, int device, cudaStream_t st,
+                        const int* skip, unsigned long long* exec) {
+  many_digit(g, t, Y, dagger, Many<2>(0, in, out), device, st, skip, exec);
 }

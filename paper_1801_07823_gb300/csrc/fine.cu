@@ -6,6 +6,7 @@
 // Links are stored pre-multiplied as W_mu(s) = eta_mu(s) U_mu(s) / 2.  In 2D
 // eta_mu(s - mu) = eta_mu(s) (eta_1 depends on x0 only), so the backward hop of
 // Eq. staggeredD is -conj(W_mu(s - mu)) x(s - mu).
+#include "many.h"
 #include "sw_internal.h"
 
 namespace {
@@ -155,9 +156,13 @@ __global__ void k_binv_build(const double2* __restrict__ Wps, double mass, doubl
     for (int j = 0; j < 4; ++j) binv[16 * b + 4 * i + j] = I[i][j];
 }
 
-// out = M in (or M^dag in) on every KD block of one parity half.
-__global__ void k_block_apply(const double2* __restrict__ M, const double2* __restrict__ in,
-                              double2* __restrict__ out, int nblk, int dagger) {
+// out = M in (or M^dag in) on nblk KD blocks; one member of a batch per blockIdx.y.
+template <int W>
+__global__ void k_block_apply(const double2* __restrict__ M, Pack<2, W> io, int nblk, int dagger,
+                              const int* __restrict__ ctl) {
+  if (ctl && ctl[4 * blockIdx.y]) return;
+  const double2* __restrict__ in = io.v[0][blockIdx.y];
+  double2* __restrict__ out = io.v[1][blockIdx.y];
   int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= nblk) return;
   double2 v[4];
@@ -185,51 +190,65 @@ __device__ __forceinline__ double2 hop_out(const double2* __restrict__ Wps,
   // direction 0
   if (x0 & 1) {  // forward neighbour is in the next block
     int t = ps_index(x0 + 1 == L0 ? 0 : x0 + 1, x1, L0, N);
-    cfma(acc, Wps[f], in[t % half]);
+    cfma(acc, Wps[f], in[t < half ? t : t - half]);
   } else {
     int t = ps_index(x0 == 0 ? L0 - 1 : x0 - 1, x1, L0, N);
     double2 w = Wps[t];
-    double2 v = in[t % half];
+    double2 v = in[t < half ? t : t - half];
     acc.x -= w.x * v.x + w.y * v.y;
     acc.y -= w.x * v.y - w.y * v.x;
   }
   // direction 1
   if (x1 & 1) {
     int t = ps_index(x0, x1 + 1 == L1 ? 0 : x1 + 1, L0, N);
-    cfma(acc, Wps[N + f], in[t % half]);
+    cfma(acc, Wps[N + f], in[t < half ? t : t - half]);
   } else {
     int t = ps_index(x0, x1 == 0 ? L1 - 1 : x1 - 1, L0, N);
     double2 w = Wps[N + t];
-    double2 v = in[t % half];
+    double2 v = in[t < half ? t : t - half];
     acc.x -= w.x * v.x + w.y * v.y;
     acc.y -= w.x * v.y - w.y * v.x;
   }
   return acc;
 }
 
-__global__ void k_hop(const double2* __restrict__ Wps, int par, double sign,
-                      const double2* __restrict__ src, const double2* __restrict__ in,
-                      double2* __restrict__ out, int L0, int L1) {
+// out_p = src_p + sign C in_{1-p} on parity half p = par, or (par < 0) on both halves of
+// full vectors; operands (src or null, in, out) of one member of a batch per blockIdx.y.
+template <int W>
+__global__ void k_hop(const double2* __restrict__ Wps, int par, double sign, Pack<3, W> io, int L0,
+                      int L1, const int* __restrict__ ctl) {
+  if (ctl && ctl[4 * blockIdx.y]) return;
+  const double2* src = io.v[0][blockIdx.y];
+  const double2* in = io.v[1][blockIdx.y];
+  double2* out = io.v[2][blockIdx.y];
   int N = L0 * L1, half = N >> 1;
   int h = blockIdx.x * blockDim.x + threadIdx.x;
-  if (h >= half) return;
-  double2 c = hop_out(Wps, in, par * half + h, L0, L1, N);
+  if (h >= (par < 0 ? N : half)) return;
+  if (par < 0 && h < half) in += half;
+  double2 c = hop_out(Wps, in, par < 0 ? h : par * half + h, L0, L1, N);
   double2 o = src ? src[h] : make_double2(0.0, 0.0);
   o.x = fma(sign, c.x, o.x);
   o.y = fma(sign, c.y, o.y);
   out[h] = o;
 }
 
+// out_p = src_p + sign M C in_{1-p} (M^dag: dagger), as above.  M: B^-1 of all blocks.
+template <int W>
 __global__ void k_hop_block(const double2* __restrict__ Wps, const double2* __restrict__ M,
-                            int par, int dagger, double sign, const double2* __restrict__ src,
-                            const double2* __restrict__ in, double2* __restrict__ out, int L0,
-                            int L1) {
-  int N = L0 * L1, half = N >> 1;
+                            int par, int dagger, double sign, Pack<3, W> io, int L0, int L1,
+                            const int* __restrict__ ctl) {
+  if (ctl && ctl[4 * blockIdx.y]) return;
+  const double2* src = io.v[0][blockIdx.y];
+  const double2* in = io.v[1][blockIdx.y];
+  double2* out = io.v[2][blockIdx.y];
+  int N = L0 * L1, half = N >> 1, nblk = half >> 2;
   int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= (half >> 2)) return;
+  if (b >= (par < 0 ? 2 * nblk : nblk)) return;
+  if (par < 0 && b < nblk) in += half;
+  const int gb = par < 0 ? b : par * nblk + b;
   double2 u[4];
-  for (int k = 0; k < 4; ++k) u[k] = hop_out(Wps, in, par * half + 4 * b + k, L0, L1, N);
-  const double2* m = M + 16 * b;
+  for (int k = 0; k < 4; ++k) u[k] = hop_out(Wps, in, 4 * gb + k, L0, L1, N);
+  const double2* m = M + 16 * (long)gb;
   for (int i = 0; i < 4; ++i) {
     double2 acc = make_double2(0.0, 0.0);
     if (!dagger)
@@ -505,52 +524,65 @@ void launch_binv_build(const sw_gauge* g, double mass, double2* binv, cudaStream
                                                       g->L1);
   SW_LAUNCH_CHECK();
 }
+void many_block_apply(const sw_gauge* g, const double2* binv, int par, int dagger,
+                      const Many<2>& io, cudaStream_t s, const int* ctl) {
+  const int half = g->N / 8, nblk = par < 0 ? 2 * half : half;
+  with_width(io.n, [&](auto w) {
+    k_block_apply<decltype(w)::value><<<dim3(nblocks(nblk, 128), io.n), 128, 0, s>>>(
+        binv + (par > 0 ? (long)half * 16 : 0), Pack<2, decltype(w)::value>(io), nblk, dagger, ctl);
+    SW_LAUNCH_CHECK();
+  });
+}
+void many_hop(const sw_gauge* g, int par, double sign, const Many<3>& io, cudaStream_t s,
+              const int* ctl) {
+  with_width(io.n, [&](auto w) {
+    k_hop<decltype(w)::value><<<dim3(nblocks(par < 0 ? g->N : g->N / 2, 256), io.n), 256, 0, s>>>(
+        g->W_ps, par, sign, Pack<3, decltype(w)::value>(io), g->L0, g->L1, ctl);
+    SW_LAUNCH_CHECK();
+  });
+}
+void many_hop_block(const sw_gauge* g, const double2* binv, int par, int dagger, double sign,
+                    const Many<3>& io, cudaStream_t s, const int* ctl) {
+  with_width(io.n, [&](auto w) {
+    k_hop_block<decltype(w)::value>
+        <<<dim3(nblocks(par < 0 ? g->N / 4 : g->N / 8, 128), io.n), 128, 0, s>>>(
+            g->W_ps, binv, par, dagger, sign, Pack<3, decltype(w)::value>(io), g->L0, g->L1, ctl);
+    SW_LAUNCH_CHECK();
+  });
+}
 void launch_block_apply(const sw_gauge* g, const double2* binv, int par, int dagger,
                         const double2* in, double2* out, cudaStream_t s) {
-  int nblk = g->N / 8;
-  k_block_apply<<<nblocks(nblk, 128), 128, 0, s>>>(binv + (long)par * nblk * 16, in, out, nblk,
-                                                   dagger);
-  SW_LAUNCH_CHECK();
+  many_block_apply(g, binv, par, dagger, Many<2>(0, in, out), s);
 }
 void launch_hop(const sw_gauge* g, int par, double sign, const double2* src, const double2* in,
                 double2* out, cudaStream_t s) {
-  k_hop<<<nblocks(g->N / 2, 256), 256, 0, s>>>(g->W_ps, par, sign, src, in, out, g->L0, g->L1);
-  SW_LAUNCH_CHECK();
-}
-void launch_hop_block(const sw_gauge* g, const double2* binv, int par, int dagger, double sign,
-                      const double2* src, const double2* in, double2* out, cudaStream_t s) {
-  int nblk = g->N / 8;
-  k_hop_block<<<nblocks(nblk, 128), 128, 0, s>>>(g->W_ps, binv + (long)par * nblk * 16, par, dagger,
-                                                 sign, src, in, out, g->L0, g->L1);
-  SW_LAUNCH_CHECK();
+  many_hop(g, par, sign, Many<3>(0, src, in, out), s);
 }
 
-// A x = x + C B^-1 x on a full parity-split vector: t = B^-1 x per block, then
-// y_p = x_p + C_{p,1-p} t_{1-p} for p = even, odd.
-void fine_apply_A(const sw_gauge* g, const double2* binv, const double2* in, double2* out,
-                  double2* tmp, cudaStream_t s) {
-  long half = g->N / 2;
-  launch_block_apply(g, binv, 0, 0, in, tmp, s);
-  launch_block_apply(g, binv, 1, 0, in + half, tmp + half, s);
-  launch_hop(g, 0, 1.0, in, tmp + half, out, s);
-  launch_hop(g, 1, 1.0, in + half, tmp, out + half, s);
+// Member-wise Many of operands k... of another.
+template <int K, typename... I>
+static Many<sizeof...(I)> pick(const Many<K>& a, I... k) {
+  Many<sizeof...(I)> o;
+  for (int m = 0; m < a.n; ++m) o.add(a.slot[m], a.v[k][m]...);
+  return o;
 }
-// A^dag x = x + B^-dag C^dag x = x - B^-dag C x (C is anti-Hermitian).
-void fine_apply_Adag(const sw_gauge* g, const double2* binv, const double2* in, double2* out,
-                     cudaStream_t s) {
-  long half = g->N / 2;
-  launch_hop_block(g, binv, 0, 1, -1.0, in, in + half, out, s);
-  launch_hop_block(g, binv, 1, 1, -1.0, in + half, in, out + half, s);
+// A A^dag x with A^dag x = x + B^-dag C^dag x = x - B^-dag C x (C is anti-Hermitian) and
+// A t = t + C B^-1 t.
+void many_normal_A(const sw_gauge* g, const double2* binv, const Many<4>& v, cudaStream_t s,
+                   const int* ctl) {
+  many_hop_block(g, binv, -1, 1, -1.0, pick(v, 0, 0, 2), s, ctl);
+  many_block_apply(g, binv, -1, 0, pick(v, 2, 3), s, ctl);
+  many_hop(g, -1, 1.0, pick(v, 2, 3, 1), s, ctl);
 }
 // S x_e = x_e - A_eo A_oe x_e with A_oe = C_oe B_e^-1 and A_eo = C_eo B_o^-1
 // (A_ee = A_oo = I on KD-block parity):
 //   t_e = B_e^-1 x_e;  v_o = B_o^-1 C_oe t_e;  y_e = x_e - C_eo v_o.
-void fine_apply_S(const sw_gauge* g, const double2* binv, const double2* in_e, double2* out_e,
-                  double2* tmp, cudaStream_t s) {
-  long half = g->N / 2;
-  launch_block_apply(g, binv, 0, 0, in_e, tmp, s);
-  launch_hop_block(g, binv, 1, 0, 1.0, nullptr, tmp, tmp + half, s);
-  launch_hop(g, 0, -1.0, in_e, tmp + half, out_e, s);
+void many_S(const sw_gauge* g, const double2* binv, const Many<3>& v, cudaStream_t s) {
+  Many<3> hb;
+  for (int m = 0; m < v.n; ++m) hb.add(0, (const double2*)nullptr, v.v[1][m], v.v[2][m]);
+  many_block_apply(g, binv, 0, 0, pick(v, 0, 1), s);
+  many_hop_block(g, binv, 1, 0, 1.0, hb, s);
+  many_hop(g, 0, -1.0, pick(v, 0, 2, 1), s);
 }
 
 static dim3 kd_grid(const sw_gauge* g, bool half) {

@@ -27,6 +27,7 @@
 #include <tuple>
 
 #include "lease.h"
+#include "many.h"
 #include "sw_internal.h"
 #include "sw_mg.h"
 
@@ -75,62 +76,65 @@ long level_len(const sw_mg* mg, int l) {
   return L.ndof;
 }
 
-// FP64 stencil of a coarse level (dagger: its adjoint), on its digit entries
-// where the level keeps them.
-void coarse_op(sw_mg* mg, int l, int dagger, const double2* in, double2* out, const int* skip) {
+// FP64 stencil of a coarse level (dagger: its adjoint) on the members of v, on
+// its digit entries where the level keeps them.  ctl: see many.h.
+void coarse_op(sw_mg* mg, int l, int dagger, const Many<2>& v, const int* ctl) {
   sw_ctx* c = mg->ctx;
   const MgLevel& L = mg->lev[l];
   const CoarseGeom cg{L.E0, L.E1, L.nc};
   unsigned long long* exec = c->timing ? c->exec + l : nullptr;
   if (L.dg.T)
-    launch_digit_apply(cg, L.dg, L.Y, dagger, in, out, c->device, c->stream, skip, exec);
+    many_digit(cg, L.dg, L.Y, dagger, v, c->device, c->stream, ctl, exec);
   else
-    launch_coarse_apply(cg, L.Y, dagger, in, out, c->stream, skip, exec);
+    for (int m = 0; m < v.n; ++m)
+      launch_coarse_apply(cg, L.Y, dagger, v.v[0][m], v.v[1][m], c->stream,
+                          ctl ? ctl + 4 * m : nullptr, exec);
 }
 
-// Operator of level l in the solve: S on level 0 (even half), A_hat below.
-// skip: optional device flag that turns the (coarse) application into a no-op.
-// lowp: inside the preconditioner of a mixed-precision hierarchy -- the fine
-// Schur operator then runs in FP32 and intermediate stencils in scaled FP16.
-void level_op(sw_mg* mg, int l, const double2* in, double2* out, const int* skip = nullptr,
-              bool lowp = false) {
+// Operator of level l in the solve on (in, out, tmp) of every member: S on level
+// 0 (even half), A_hat below.  lowp: inside the preconditioner of a
+// mixed-precision hierarchy -- the fine Schur operator then runs in FP32 and
+// intermediate stencils in scaled FP16.
+void level_op(sw_mg* mg, int l, const Many<3>& v, bool lowp, const int* ctl = nullptr) {
   sw_ctx* c = mg->ctx;
-  int tk = timing_begin(c, l);
-  if (l == 0) {
-    if (mg->fine_D)
-      launch_dslash_ps(mg->g, mg->mass, 0, in, out, c->stream);
-    else if (lowp && mg->mixed)
-      fine_apply_S32(mg->g, mg->g->W_ps32, mg->binv32, in, out, mg->s32tmp, c->stream);
-    else
-      fine_apply_S(mg->g, mg->binv, in, out, mg->lev[0].stmp, c->stream);
-    mg->st_fine_applies++;
-  } else if (lowp && mg->mixed && mg->lev[l].Yh) {
-    const MgLevel& L = mg->lev[l];
-    launch_coarse_apply_h(CoarseGeom{L.E0, L.E1, L.nc}, L.Yh, L.Ysc, 0, in, out, c->stream);
+  int tk = timing_begin(c, l, v.n);
+  if (l == 0 && mg->fine_D) {
+    for (int m = 0; m < v.n; ++m)
+      launch_dslash_ps(mg->g, mg->mass, 0, v.v[0][m], v.v[1][m], c->stream);
+  } else if (l == 0 && lowp && mg->mixed) {
+    many_S32(mg->g, mg->g->W_ps32, mg->binv32, v, c->stream);
+  } else if (l == 0) {
+    many_S(mg->g, mg->binv, v, c->stream);
   } else {
-    coarse_op(mg, l, 0, in, out, skip);
+    const MgLevel& L = mg->lev[l];
+    Many<2> io;
+    for (int m = 0; m < v.n; ++m) io.add(0, v.v[0][m], v.v[1][m]);
+    if (lowp && mg->mixed && L.Yh)
+      many_coarse_h(CoarseGeom{L.E0, L.E1, L.nc}, L.Yh, L.Ysc, 0, io, c->stream);
+    else
+      coarse_op(mg, l, 0, io, ctl);
   }
   timing_end(c, tk);
 }
-void level_opdag(sw_mg* mg, int l, const double2* in, double2* out, const int* skip = nullptr) {
+// Normal operator used by the setup on level l: A A^dag on (in, out, t, u) of every
+// member (full fine vectors on level 0).
+void level_normal(sw_mg* mg, int l, const Many<4>& v, const int* ctl) {
   sw_ctx* c = mg->ctx;
-  int tk = timing_begin(c, l);
-  coarse_op(mg, l, 1, in, out, skip);
-  timing_end(c, tk);
-}
-// Normal operator used by the setup on level l: A A^dag (full fine vectors on
-// level 0).
-void level_normal(sw_mg* mg, int l, const double2* in, double2* out, double2* tmp) {
-  cudaStream_t s = mg->ctx->stream;
   if (l == 0 && mg->fine_D) {
-    launch_dslash_ps(mg->g, mg->mass, 1, in, tmp, s);
-    launch_dslash_ps(mg->g, mg->mass, 0, tmp, out, s);
+    for (int m = 0; m < v.n; ++m) {
+      launch_dslash_ps(mg->g, mg->mass, 1, v.v[0][m], v.v[2][m], c->stream);
+      launch_dslash_ps(mg->g, mg->mass, 0, v.v[2][m], v.v[1][m], c->stream);
+    }
   } else if (l == 0) {
-    fine_apply_Adag(mg->g, mg->binv, in, tmp, s);
-    fine_apply_A(mg->g, mg->binv, tmp, out, mg->lev[0].stmp, s);
+    many_normal_A(mg->g, mg->binv, v, c->stream, ctl);
   } else {
-    level_opdag(mg, l, in, tmp);
-    level_op(mg, l, tmp, out);
+    for (int dagger = 1; dagger >= 0; --dagger) {
+      Many<2> io;
+      for (int m = 0; m < v.n; ++m) io.add(0, v.v[dagger ? 0 : 2][m], v.v[dagger ? 2 : 1][m]);
+      const int tk = timing_begin(c, l, v.n);
+      coarse_op(mg, l, dagger, io, ctl);
+      timing_end(c, tk);
+    }
   }
 }
 
@@ -138,137 +142,7 @@ static void check_norm(double v, const char* where) {
   if (!std::isfinite(v)) throw SwError{SW_ERR_NAN, std::string("non-finite norm in ") + where};
 }
 
-// SW_VERBOSE >= 3: the 2-norm of a work vector on stderr (a trace of where a
-// non-finite value first appears).  Costs a host round trip per call.
-static void trace_norm(sw_mg* mg, int l, const char* what, const double2* v, long n) {
-  if (mg->verbose < 3) return;
-  blas_norm2(mg->ctx, v, n, slot_base(l) + 63);
-  std::fprintf(stderr, "[sw]       level %d %s |v| %.6e\n", l + 1, what,
-               std::sqrt(slot_read(mg->ctx, slot_base(l) + 63).x));
-}
-
 // ---------------------------------------------------------------- Krylov
-// MR smoother with zero initial guess: x, r = b - op x.
-static void mr(sw_mg* mg, int l, const double2* b, double2* x, double2* r, double2* q) {
-  const bool lowp = true;  // the smoother always belongs to the preconditioner
-  sw_ctx* c = mg->ctx;
-  long n = level_len(mg, l);
-  int sq = slot_base(l) + 8, sqq = slot_base(l) + 9;
-  blas_zero(c, x, n);
-  blas_copy(c, r, b, n);
-  double om = mg->p.omega;
-  for (int it = 0; it < mg->p.smoother_iters; ++it) {
-    level_op(mg, l, r, q, nullptr, lowp);
-    blas_dot(c, q, r, n, sq);
-    blas_norm2(c, q, n, sqq);
-    if (mg->verbose >= 3) {
-      const double2 a = slot_read(c, sq), b = slot_read(c, sqq);
-      std::fprintf(stderr, "[sw]       level %d MR %d (q, r) %.6e %+.6ei |q|^2 %.6e\n", l + 1,
-                   it, a.x, a.y, b.x);
-    }
-    blas_axpy(c, x, r, n, coef_ratio(sq, sqq, om));
-    blas_axpy(c, r, q, n, coef_ratio(sq, sqq, -om));
-  }
-}
-
-static void solve_level(sw_mg* mg, int l, const double2* rhs, double2* sol);
-
-// K-cycle preconditioner of level l: out = M(r).
-static void kcycle(sw_mg* mg, int l, const double2* r, double2* out) {
-  sw_ctx* c = mg->ctx;
-  MgLevel& L = mg->lev[l];
-  MgLevel& C = mg->lev[l + 1];
-  long n = level_len(mg, l);
-  cudaStream_t s = c->stream;
-  trace_norm(mg, l, "K-cycle input", r, n);
-  mr(mg, l, r, L.kx1, L.kr1, L.kq);
-  trace_norm(mg, l, "pre-smoothed x", L.kx1, n);
-  trace_norm(mg, l, "pre-smoothed r", L.kr1, n);
-  if (l == 0)
-    launch_restrict_fine(mg->g, L.b0, L.b1, L.nv, L.P, L.kr1, C.rhs, s, mg->fine_D ? 1 : 0);
-  else
-    launch_restrict_coarse(CoarseGeom{L.E0, L.E1, L.nc}, L.b0, L.b1, L.nv, L.P, L.kr1, C.rhs, s);
-  trace_norm(mg, l + 1, "restricted r", C.rhs, level_len(mg, l + 1));
-  solve_level(mg, l + 1, C.rhs, C.sol);
-  if (l == 0)
-    launch_prolong_fine(mg->g, L.b0, L.b1, L.nv, L.P, C.sol, L.ke, s, mg->fine_D ? 1 : 0);
-  else
-    launch_prolong_coarse(CoarseGeom{L.E0, L.E1, L.nc}, L.b0, L.b1, L.nv, L.P, C.sol, L.ke, s);
-  level_op(mg, l, L.ke, L.kq, nullptr, true);
-  blas_sub(c, L.kr2, L.kr1, L.kq, n);
-  mr(mg, l, L.kr2, L.kx3, L.kr3, L.kq);
-  blas_add3(c, out, L.kx1, L.ke, L.kx3, n);
-}
-
-struct GcrResult {
-  int iters, restarts;
-  bool converged;
-};
-
-// Flexible restarted GCR on level l (see the oracle's fgcr for the steps).
-static GcrResult fgcr(sw_mg* mg, int l, const double2* b, double2* x, double tol_abs, int restart,
-                      int maxiter, bool confirm) {
-  sw_ctx* c = mg->ctx;
-  MgLevel& L = mg->lev[l];
-  long n = level_len(mg, l);
-  int sb = slot_base(l);
-  int s_rr = sb + 0, s_qq = sb + 2, s_a = sb + 3, s_b = sb + 4;
-  blas_zero(c, x, n);
-  blas_copy(c, L.gr, b, n);
-  int k = 0, it = 0, restarts = 0;
-  const bool lowp = l > 0;  // intermediate solves are part of the preconditioner
-  for (;;) {
-    blas_norm2(c, L.gr, n, s_rr);
-    double rn = std::sqrt(slot_read(c, s_rr).x);
-    check_norm(rn, "GCR residual");
-    if (rn <= tol_abs) {
-      if (!confirm) return GcrResult{it, restarts, true};
-      level_op(mg, l, x, L.gtmp, nullptr, lowp);
-      blas_sub(c, L.gtmp, b, L.gtmp, n);
-      blas_norm2(c, L.gtmp, n, s_rr);
-      double rt = std::sqrt(slot_read(c, s_rr).x);
-      check_norm(rt, "GCR true residual");
-      if (rt <= tol_abs) return GcrResult{it, restarts, true};
-      blas_copy(c, L.gr, L.gtmp, n);
-      k = 0;
-      ++restarts;
-      continue;
-    }
-    if (it >= maxiter) return GcrResult{it, restarts, false};
-    double2* p = L.gp[k];
-    double2* q = L.gq[k];
-    if (l + 1 < mg->nlev)
-      kcycle(mg, l, L.gr, p);
-    else
-      blas_copy(c, p, L.gr, n);
-    level_op(mg, l, p, q, nullptr, lowp);
-    for (int j = 0; j < k; ++j) {
-      blas_dot(c, L.gq[j], q, n, s_b);
-      blas_axpy(c, q, L.gq[j], n, coef_ratio(s_b, -1, -1.0));
-      blas_axpy(c, p, L.gp[j], n, coef_ratio(s_b, -1, -1.0));
-    }
-    blas_norm2(c, q, n, s_qq);
-    blas_scale(c, q, n, coef_ratio(-1, s_qq, 1.0, COEF_SQRT_DEN));
-    blas_scale(c, p, n, coef_ratio(-1, s_qq, 1.0, COEF_SQRT_DEN));
-    blas_dot(c, q, L.gr, n, s_a);
-    blas_axpy(c, x, p, n, coef_ratio(s_a, -1, 1.0));
-    blas_axpy(c, L.gr, q, n, coef_ratio(s_a, -1, -1.0));
-    ++k;
-    ++it;
-    if (l == 1 && mg->verbose > 1) std::fprintf(stderr, "[sw]   level-2 GCR %d |r| %.3e (tol %.3e)\n", it, rn, tol_abs);
-    if (l == 0 && mg->verbose)
-      std::fprintf(stderr, "[sw] outer %d |r| %.3e  inter %lld/%lld coarsest %lld/%lld\n", it, rn,
-                   mg->st_inter_iters, mg->st_inter_solves, mg->st_coarsest_iters,
-                   mg->st_coarsest_solves);
-    if (k == restart && it < maxiter) {
-      level_op(mg, l, x, L.gtmp, nullptr, lowp);
-      blas_sub(c, L.gr, b, L.gtmp, n);
-      k = 0;
-      ++restarts;
-    }
-  }
-}
-
 // CG on the normal error (Craig): x = op^dag y with op op^dag y = b.  The
 // stopping test runs on the device (iter_check); the host queues kIterBatch
 // iterations at a time and reads the control block between batches, so the
@@ -327,18 +201,23 @@ static int cgne(sw_mg* mg, int l, const double2* b, double2* x) {
   double rr = slot_read(c, s_rr[0]).x;
   check_norm(rr, "CGNE residual");
   double stop = mg->p.coarsest_tol * std::sqrt(rr);
-  level_opdag(mg, l, L.gr, L.cp);
+  const auto op = [&](int dagger, const double2* in, double2* out, const int* skip) {
+    const int tk = timing_begin(c, l);
+    coarse_op(mg, l, dagger, Many<2>(0, in, out), skip);
+    timing_end(c, tk);
+  };
+  op(1, L.gr, L.cp, nullptr);
   iter_init(c, ctl, s_rr[0], stop, maxit);
   int cur = 0;
   for (int issued = 0;;) {
     for (int q = 0; q < kIterBatch && issued < maxit; ++q, ++issued) {
       blas_norm2(c, L.cp, n, s_pp, ctl);
       blas_axpy(c, x, L.cp, n, coef_ratio(s_rr[cur], s_pp, 1.0), ctl);
-      level_op(mg, l, L.cp, L.cw, ctl);
+      op(0, L.cp, L.cw, ctl);
       blas_axpy(c, L.gr, L.cw, n, coef_ratio(s_rr[cur], s_pp, -1.0), ctl);
       blas_norm2(c, L.gr, n, s_rr[1 - cur], ctl);
       iter_check(c, ctl, s_rr[1 - cur], stop, maxit);
-      level_opdag(mg, l, L.gr, L.cw, ctl);
+      op(1, L.gr, L.cw, ctl);
       blas_xpay(c, L.cp, L.cw, n, coef_ratio(s_rr[1 - cur], s_rr[cur], 1.0), ctl);
       cur = 1 - cur;
     }
@@ -349,52 +228,53 @@ static int cgne(sw_mg* mg, int l, const double2* b, double2* x) {
   return c->h_ctl[1];
 }
 
-static void solve_level(sw_mg* mg, int l, const double2* rhs, double2* sol) {
+// CG on the Hermitian positive semi-definite A A^dag (setup) for all members of the
+// set in lockstep: x from zero, right-hand sides -q.  Stopping tests on the device;
+// the host looks at them after kIterBatch iterations.  Returns the iterations of each.
+struct SetupVecs {
+  std::vector<double2*> x, r, p, q, t, u;
+};
+static std::vector<int> cg_setup(sw_mg* mg, int l, const SetupVecs& v, int w) {
   sw_ctx* c = mg->ctx;
-  if (l == mg->nlev - 1) {
-    mg->st_coarsest_iters += cgne(mg, l, rhs, sol);
-    mg->st_coarsest_solves++;
-    return;
+  const long n = mg->lev[l].ndof;
+  const int maxit = mg->p.setup_maxiter;
+  constexpr int s_pq = 22, s_stop = 23;
+  int s_rr[2] = {20, 21};
+  Many<4> start, op, step;
+  Many<2> pq, pr;
+  for (int m = 0; m < w; ++m) {
+    const int slot = slot_base(l) + (m + 1) * kSlotPage;
+    start.add(slot, v.x[m], v.r[m], v.p[m], v.q[m]);
+    op.add(slot, v.p[m], v.q[m], v.t[m], v.u[m]);
+    step.add(slot, v.x[m], v.r[m], v.p[m], v.q[m]);
+    pq.add(slot, v.p[m], v.q[m]);
+    pr.add(slot, v.p[m], v.r[m]);
   }
-  long n = level_len(mg, l);
-  int s = slot_base(l) + 1;
-  blas_norm2(c, rhs, n, s);
-  double bn = std::sqrt(slot_read(c, s).x);
-  check_norm(bn, "intermediate right-hand side");
-  GcrResult r = fgcr(mg, l, rhs, sol, mg->p.inter_tol * bn, mg->p.inter_restart,
-                     mg->p.inter_maxiter, false);
-  mg->st_inter_iters += r.iters;
-  mg->st_inter_solves++;
-}
-
-// CG on a Hermitian positive semi-definite normal operator (setup).
-static int cg_setup(sw_mg* mg, int l, const double2* b, double2* x) {
-  sw_ctx* c = mg->ctx;
-  MgLevel& L = mg->lev[l];
-  long n = L.ndof;
-  int sb = slot_base(l);
-  int s_rr[2] = {sb + 20, sb + 21}, s_pq = sb + 22;
-  blas_zero(c, x, n);
-  blas_copy(c, L.sr, b, n);
-  blas_copy(c, L.sp, L.sr, n);
-  blas_norm2(c, L.sr, n, s_rr[0]);
-  double rr = slot_read(c, s_rr[0]).x;
-  check_norm(rr, "setup CG residual");
-  double stop = mg->p.setup_tol * std::sqrt(rr);
-  int k = 0, cur = 0;
-  while (k < mg->p.setup_maxiter && std::sqrt(rr) > stop) {
-    level_normal(mg, l, L.sp, L.sq, L.st);
-    blas_dot(c, L.sp, L.sq, n, s_pq);
-    blas_axpy(c, x, L.sp, n, coef_ratio(s_rr[cur], s_pq, 1.0));
-    blas_axpy(c, L.sr, L.sq, n, coef_ratio(s_rr[cur], s_pq, -1.0));
-    blas_norm2(c, L.sr, n, s_rr[1 - cur]);
-    rr = slot_read(c, s_rr[1 - cur]).x;
-    check_norm(rr, "setup CG residual");
-    blas_xpay(c, L.sp, L.sr, n, coef_ratio(s_rr[1 - cur], s_rr[cur], 1.0));
-    cur = 1 - cur;
-    ++k;
+  int* ctl = c->many_ctl;
+  many_cg_start(c, n, start, s_rr[0], s_stop, mg->p.setup_tol, maxit, ctl);
+  for (int issued = 0;;) {
+    SW_CUDA(cudaMemcpyAsync(c->h_many->ctl, ctl, 4 * w * sizeof(int), cudaMemcpyDeviceToHost,
+                            c->stream));
+    SW_CUDA(cudaStreamSynchronize(c->stream));
+    if (!c->pending.empty()) timing_harvest(c);
+    bool done = true;
+    for (int m = 0; m < w; ++m) {
+      if (c->h_many->ctl[4 * m + 2])
+        throw SwError{SW_ERR_NAN, "non-finite norm in setup CG residual"};
+      done = done && c->h_many->ctl[4 * m];
+    }
+    if (done) break;
+    for (int q = 0; q < kIterBatch && issued < maxit; ++q, ++issued) {
+      level_normal(mg, l, op, ctl);
+      many_dot(c, n, pq, s_pq, ctl);
+      many_cg_step(c, n, step, s_rr[0], s_pq, s_rr[1], s_stop, maxit, ctl);
+      many_xpay(c, n, pr, s_rr[1], s_rr[0], ctl);
+      std::swap(s_rr[0], s_rr[1]);
+    }
   }
-  return k;
+  std::vector<int> its(w);
+  for (int m = 0; m < w; ++m) its[m] = c->h_many->ctl[4 * m + 1];
+  return its;
 }
 
 int mg_coarsest_solve(sw_mg* mg, const double2* b, double2* x) {
@@ -413,7 +293,6 @@ void mg_setup(sw_mg* mg, const double* const* psi0, uint64_t seed) {
   if (mg->mixed) {
     mg->binv32 = (float2*)mg_alloc(mg, N * 2);
     launch_to_f32(mg->binv, mg->binv32, N * 4, s);
-    mg->s32tmp = (float2*)mg_alloc(mg, (N + 1) / 2);
   }
   ScopedBuffers tmp;
   for (int l = 0; l + 1 < mg->nlev; ++l) {
@@ -421,53 +300,72 @@ void mg_setup(sw_mg* mg, const double* const* psi0, uint64_t seed) {
     MgLevel& C = mg->lev[l + 1];
     int nv = L.nv;
     long n = L.ndof;
-    // work vectors of the setup
-    L.sr = tmp.get(n); L.sp = tmp.get(n); L.sq = tmp.get(n);
-    L.st = tmp.get(n);
+    // Null vectors advance in groups whose vectors are small enough for a launch per
+    // operation and vector to be mostly latency (64^2: 4096 elements, 3 us); from 2 M
+    // elements on one vector fills the device by itself and the scratch is one
+    // vector's.
+    const int w = (int)std::min<long>(nv, std::max<long>(1, (1L << 21) / n));
     double2* V = tmp.get(n * nv);
-    double2* e = tmp.get(n);
-    double2* start = tmp.get(n);
     double2* lex = l == 0 ? tmp.get(n) : nullptr;
-    int sb = slot_base(l);
-    for (int i = 0; i < nv; ++i) {
-      double2* target = l == 0 ? lex : start;
-      if (psi0 && psi0[l]) {
-        SW_CUDA(cudaMemcpyAsync(target, psi0[l] + 2 * (long)i * n, n * sizeof(double2),
-                                cudaMemcpyHostToDevice, s));
-      } else {
-        launch_gaussian(sw_stream_seed(seed, l, i), n, target, s);
+    SetupVecs wk;
+    for (auto* f : {&wk.x, &wk.r, &wk.p, &wk.q, &wk.t, &wk.u}) {
+      f->assign(w, nullptr);
+      if (f == &wk.u && l > 0) continue;
+      double2* base = tmp.get(n * w);
+      for (int m = 0; m < w; ++m) (*f)[m] = base + (long)m * n;
+    }
+    const int sb = slot_base(l);
+    const auto page = [&](int m) { return sb + (m + 1) * kSlotPage; };
+    const size_t it0 = mg->setup_iters.size();
+    const int passes = mg->p.setup_passes;
+    mg->setup_iters.resize(it0 + (size_t)nv * passes);
+    for (int i0 = 0; i0 < nv; i0 += w) {
+      const int m1 = std::min(w, nv - i0);
+      Many<1> psi;
+      Many<2> psi_e;
+      Many<4> first;
+      for (int m = 0; m < m1; ++m) {
+        double2* v = V + (long)(i0 + m) * n;
+        double2* target = l == 0 ? lex : v;
+        if (psi0 && psi0[l])
+          SW_CUDA(cudaMemcpyAsync(target, psi0[l] + 2 * (long)(i0 + m) * n, n * sizeof(double2),
+                                  cudaMemcpyHostToDevice, s));
+        else
+          launch_gaussian(sw_stream_seed(seed, l, i0 + m), n, target, s);
+        if (l == 0) launch_pack(g, lex, v, s);
+        psi.add(page(m), v);
+        psi_e.add(page(m), v, wk.x[m]);
+        first.add(page(m), v, wk.q[m], wk.t[m], wk.u[m]);
       }
-      if (l == 0) launch_pack(g, lex, start, s);
-      double2* psi = V + (long)i * n;
-      for (int pass = 0; pass < mg->p.setup_passes; ++pass) {
+      for (int pass = 0; pass < passes; ++pass) {
         if (pass > 0) {
-          blas_copy(c, start, psi, n);
-          blas_norm2(c, start, n, sb + 30);
-          blas_scale(c, start, n, coef_ratio(-1, sb + 30, 1.0, COEF_SQRT_DEN));
+          many_norm(c, n, psi, 30);
+          many_normalise(c, n, psi, 30);
         }
-        level_normal(mg, l, start, L.sq, L.st);
-        blas_zero(c, L.sp, n);
-        blas_sub(c, L.st, L.sp, L.sq, n);  // r = -A A^dag start
-        int its = cg_setup(mg, l, L.st, e);  // L.st is read before CG reuses it
-        mg->setup_iters.push_back(its);
-        blas_copy(c, psi, start, n);  // psi = psi0 + e
-        blas_axpy(c, psi, e, n, coef_const(1.0));
+        level_normal(mg, l, first, nullptr);  // e solves A A^dag e = -A A^dag psi
+        const std::vector<int> its = cg_setup(mg, l, wk, m1);
+        for (int m = 0; m < m1; ++m) mg->setup_iters[it0 + (size_t)(i0 + m) * passes + pass] = its[m];
+        many_add(c, n, psi_e);
       }
     }
-    // global modified Gram-Schmidt in index order
-    for (int i = 0; i < nv; ++i) {
-      double2* vi = V + (long)i * n;
-      for (int j = 0; j < i; ++j) {
-        blas_dot(c, V + (long)j * n, vi, n, sb + 31);
-        blas_axpy(c, vi, V + (long)j * n, n, coef_ratio(sb + 31, -1, -1.0));
+    // global modified Gram-Schmidt: vector j is normalised and taken out of the later ones
+    for (int j = 0; j < nv; ++j) {
+      double2* vj = V + (long)j * n;
+      many_norm(c, n, Many<1>(page(j), vj), 32, c->h_many->norm + j);
+      many_normalise(c, n, Many<1>(page(j), vj), 32);
+      Many<2> dots, later;
+      for (int i = j + 1; i < nv; ++i) {
+        dots.add(page(i), vj, V + (long)i * n);
+        later.add(page(i), V + (long)i * n, vj);
       }
-      blas_norm2(c, vi, n, sb + 32);
-      double nn = slot_read(c, sb + 32).x;
-      if (!(nn > 0.0) || !std::isfinite(nn))
+      many_dot(c, n, dots, 31);
+      many_project(c, n, later, 31);
+    }
+    SW_CUDA(cudaStreamSynchronize(s));
+    for (int i = 0; i < nv; ++i)
+      if (!(c->h_many->norm[i] > 0.0) || !std::isfinite(c->h_many->norm[i]))
         throw SwError{SW_ERR_BREAKDOWN, "global Gram-Schmidt: vector " + std::to_string(i) +
                                             " on level " + std::to_string(l + 1) + " has norm 0"};
-      blas_scale(c, vi, n, coef_ratio(-1, sb + 32, 1.0, COEF_SQRT_DEN));
-    }
     // chiral doubling + block orthonormalisation
     L.P = mg_alloc(mg, n * nv);
     SW_CUDA(cudaMemsetAsync(c->flag, 0, sizeof(int), s));
@@ -519,7 +417,6 @@ void mg_setup(sw_mg* mg, const double* const* psi0, uint64_t seed) {
       }
     }
     SW_CUDA(cudaStreamSynchronize(s));
-    L.sr = L.sp = L.sq = L.st = nullptr;
   }
   if (mg->mixed)
     for (int l = 1; l + 1 < mg->nlev; ++l) mg->lev[l].dg = DigitStencil{};
@@ -540,10 +437,10 @@ void mg_setup(sw_mg* mg, const double* const* psi0, uint64_t seed) {
     L.cw = mg_alloc(mg, n);
     if (l + 1 < mg->nlev) {
       L.kx1 = mg_alloc(mg, n); L.kr1 = mg_alloc(mg, n); L.kq = mg_alloc(mg, n);
-      L.ke = mg_alloc(mg, n); L.kr2 = mg_alloc(mg, n); L.kx3 = mg_alloc(mg, n);
-      L.kr3 = mg_alloc(mg, n);
+      L.ke = mg_alloc(mg, n); L.kx3 = mg_alloc(mg, n);
     }
     if (l == 0) {
+      L.tmp = L.stmp;
       mg->bps = mg_alloc(mg, N);
       mg->xps = mg_alloc(mg, N);
       mg->lexb = mg_alloc(mg, N);
@@ -553,280 +450,310 @@ void mg_setup(sw_mg* mg, const double* const* psi0, uint64_t seed) {
   }
 }
 
-// ---------------------------------------------------------------- solve
-int mg_solve_device(sw_mg* mg, const double2* b_lex, double2* x_lex, double tol,
-                    sw_solve_stats* st) {
-  sw_ctx* c = mg->ctx;
-  sw_gauge* g = mg->g;
-  cudaStream_t s = c->stream;
-  long N = g->N, half = N / 2;
-  auto t0 = std::chrono::steady_clock::now();
-  mg->st_fine_applies = mg->st_inter_iters = mg->st_inter_solves = 0;
-  mg->st_coarsest_iters = mg->st_coarsest_solves = 0;
-  MgLevel& L = mg->lev[0];
-  launch_pack(g, b_lex, mg->bps, s);
-  int sb = slot_base(0);
-  blas_norm2(c, mg->bps, N, sb + 40);
-  double bn = std::sqrt(slot_read(c, sb + 40).x);
-  check_norm(bn, "right-hand side");
-  if (bn == 0.0) {
-    blas_zero(c, x_lex, N);
-    SW_CUDA(cudaStreamSynchronize(s));
-    if (st) {
-      std::memset(st, 0, sizeof(*st));
-      st->converged = 1;
-    }
-    return SW_OK;
-  }
-  GcrResult r;
-  if (mg->fine_D) {
-    // Galerkin MG of D itself: flexible GCR on the full D, no KD preconditioning
-    r = fgcr(mg, 0, mg->bps, L.sol, tol * bn, mg->p.outer_restart, mg->p.outer_maxiter, true);
-    launch_unpack(g, L.sol, x_lex, s);
-  } else {
-    // b~_e = b_e - A_eo b_o = b_e - C_eo B_o^-1 b_o
-    launch_block_apply(g, mg->binv, 1, 0, mg->bps + half, L.stmp + half, s);
-    launch_hop(g, 0, -1.0, mg->bps, L.stmp + half, L.rhs, s);
-    r = fgcr(mg, 0, L.rhs, L.sol, tol * bn, mg->p.outer_restart, mg->p.outer_maxiter, true);
-    // z_o = b_o - C_oe B_e^-1 z_e ; x = B^-1 z
-    launch_block_apply(g, mg->binv, 0, 0, L.sol, L.stmp, s);
-    launch_hop(g, 1, -1.0, mg->bps + half, L.stmp, L.stmp + half, s);
-    launch_block_apply(g, mg->binv, 0, 0, L.sol, mg->xps, s);
-    launch_block_apply(g, mg->binv, 1, 0, L.stmp + half, mg->xps + half, s);
-    launch_unpack(g, mg->xps, x_lex, s);
-  }
-  // true residual ||b - D x|| / ||b|| in FP64
-  launch_dslash_lex(g, mg->mass, 0, x_lex, mg->lext, s);
-  blas_sub(c, mg->lext, b_lex, mg->lext, N);
-  blas_norm2(c, mg->lext, N, sb + 41);
-  double tr = std::sqrt(slot_read(c, sb + 41).x) / bn;
-  auto t1 = std::chrono::steady_clock::now();
-  if (st) {
-    st->converged = r.converged ? 1 : 0;
-    st->outer_iters = r.iters;
-    st->restarts = r.restarts;
-    st->fine_applies = mg->st_fine_applies;
-    st->inter_iters = mg->st_inter_iters;
-    st->inter_solves = mg->st_inter_solves;
-    st->coarsest_iters = mg->st_coarsest_iters;
-    st->coarsest_solves = mg->st_coarsest_solves;
-    st->true_resid = tr;
-    st->seconds = std::chrono::duration<double>(t1 - t0).count();
-  }
-  return r.converged ? SW_OK : SW_ERR_NOCONV;
-}
-
-// ================================================================ batched solves
-// Several right-hand sides of one mixed-precision hierarchy advance in
-// lockstep through the same K-cycle: every step is issued for each of them
-// in turn (own work vectors, own page of Krylov scalars, own stopping tests),
-// so that all of them reach the coarsest level together and share one
-// batched coarsest CGNE launch, which reads the coarsest stencil once for the
-// whole batch.  A right-hand side that has met a stopping test drops out of
-// the step while the others go on.  Operator scratch (fine S temporaries) is
-// shared: all steps run in order on the one context stream.
+// ================================================================ lockstep solves
+// One solve, or several right-hand sides of one mixed-precision hierarchy, which
+// advance through the same K-cycle together: every step is one launch for all
+// of them (own work vectors, own page of Krylov scalars, own stopping tests), and
+// all of them reach the coarsest level together and share one batched
+// coarsest CGNE launch, which reads the coarsest stencil once for the whole
+// batch.  A right-hand side that has met a stopping test drops out of the step
+// while the others go on.
 
 namespace {
 
 using Set = std::vector<int>;
 
-inline int page(int r) { return (r + 1) * kSlotPage; }
-
-// Reads the slot pages of the batch (page 0 and those of its nb right-hand
-// sides) back once after the queued reductions.
-const double2* slots_read_all(sw_ctx* c, int nb) {
-  SW_CUDA(cudaMemcpyAsync(c->h_slots, c->slots, (size_t)kSlotPage * (nb + 1) * sizeof(double2),
-                          cudaMemcpyDeviceToHost, c->stream));
-  SW_CUDA(cudaStreamSynchronize(c->stream));
-  if (!c->pending.empty()) timing_harvest(c);
-  return c->h_slots;
-}
-
-struct BatchCounters {
+struct Solve {
+  sw_mg* mg;
+  bool batch;
   std::vector<long long> fine, inter_it, inter_solves, coarse_it, coarse_solves;
-  explicit BatchCounters(int nb)
-      : fine(nb, 0), inter_it(nb, 0), inter_solves(nb, 0), coarse_it(nb, 0),
-        coarse_solves(nb, 0) {}
+  Solve(sw_mg* m, bool many)
+      : mg(m), batch(many), fine(width(), 0), inter_it(width(), 0), inter_solves(width(), 0),
+        coarse_it(width(), 0), coarse_solves(width(), 0) {}
+  int width() const { return batch ? kMaxBatch : 1; }
+  LevelWs& at(int l, int r) { return batch ? mg->batch.lv[l][r] : mg->lev[l]; }
+  int slot(int l, int r) const { return slot_base(l) + (batch ? (r + 1) * kSlotPage : 0); }
 };
 
-void op_b(sw_mg* mg, int l, int r, const double2* in, double2* out, bool lowp,
-          BatchCounters& bc) {
-  level_op(mg, l, in, out, nullptr, lowp);
-  if (l == 0) bc.fine[r]++;
+// Waits for the norms that the last sums left in pinned memory.
+const double* norms(sw_ctx* c) {
+  SW_CUDA(cudaStreamSynchronize(c->stream));
+  if (!c->pending.empty()) timing_harvest(c);
+  return c->h_many->norm;
 }
 
-// MR smoother (zero guess) for each member: x in kx1, residual in kr1.
-void mr_b(sw_mg* mg, int l, const Set& set, const std::vector<const double2*>& b,
-          BatchCounters& bc) {
+// SW_VERBOSE >= 3: the 2-norm of a single solve's work vector on stderr (a trace of where a
+// non-finite value first appears).  Costs a host round trip per call.
+void trace_norm(Solve& S, int l, const char* what, const double2* v) {
+  sw_mg* mg = S.mg;
+  if (mg->verbose < 3 || S.batch) return;
+  blas_norm2(mg->ctx, v, level_len(mg, l), slot_base(l) + 63);
+  std::fprintf(stderr, "[sw]       level %d %s |v| %.6e\n", l + 1, what,
+               std::sqrt(slot_read(mg->ctx, slot_base(l) + 63).x));
+}
+
+void apply(Solve& S, int l, const Set& set, const Many<3>& v, bool lowp) {
+  if (l == 0)
+    for (int r : set) S.fine[r]++;
+  level_op(S.mg, l, v, lowp);
+}
+
+// MR smoother with zero initial guess (always part of the preconditioner).  Before the
+// coarse correction: x1 = kx1 and r1 = kr1 from b.  After it, on the residual in
+// kr1: out = (x1 + e) + x3, the residual it would leave is not formed.
+void mr(Solve& S, int l, const Set& set, bool post, const std::vector<const double2*>& b,
+        const std::vector<double2*>& out) {
+  sw_mg* mg = S.mg;
   sw_ctx* c = mg->ctx;
-  long n = level_len(mg, l);
-  double om = mg->p.omega;
-  for (int r : set) {
-    LevelWs& W = mg->batch.lv[l][r];
-    blas_zero(c, W.kx1, n);
-    blas_copy(c, W.kr1, b[r], n);
-  }
-  for (int it = 0; it < mg->p.smoother_iters; ++it)
+  const long n = level_len(mg, l);
+  const double om = mg->p.omega;
+  const int iters = mg->p.smoother_iters;
+  constexpr int sq = 8;
+  for (int it = 0; it < iters; ++it) {
+    const bool last = post && it == iters - 1;
+    Many<3> op, step;
+    Many<2> qr;
+    Many<4> first;
+    Many<5> end;
     for (int r : set) {
-      LevelWs& W = mg->batch.lv[l][r];
-      int sq = slot_base(l) + page(r) + 8, sqq = sq + 1;
-      op_b(mg, l, r, W.kr1, W.kq, true, bc);
-      blas_dot(c, W.kq, W.kr1, n, sq);
-      blas_norm2(c, W.kq, n, sqq);
-      blas_axpy(c, W.kx1, W.kr1, n, coef_ratio(sq, sqq, om));
-      blas_axpy(c, W.kr1, W.kq, n, coef_ratio(sq, sqq, -om));
+      LevelWs& W = S.at(l, r);
+      const int slot = S.slot(l, r);
+      const double2* res = post || it > 0 ? W.kr1 : b[r];
+      double2* x = post ? W.kx3 : W.kx1;
+      op.add(slot, res, W.kq, W.tmp);
+      qr.add(slot, W.kq, res);
+      if (last)
+        end.add(slot, out[r], x, res, W.kx1, W.ke);
+      else if (it == 0)
+        first.add(slot, x, W.kr1, res, W.kq);
+      else
+        step.add(slot, x, W.kr1, W.kq);
     }
+    apply(S, l, set, op, true);
+    many_dot_norm(c, n, qr, sq);
+    if (mg->verbose >= 3 && !S.batch) {
+      const double2 a = slot_read(c, slot_base(l) + sq), q2 = slot_read(c, slot_base(l) + sq + 1);
+      std::fprintf(stderr, "[sw]       level %d MR %d (q, r) %.6e %+.6ei |q|^2 %.6e\n", l + 1,
+                   it, a.x, a.y, q2.x);
+    }
+    many_mr_first(c, n, first, sq, om);
+    many_mr(c, n, step, sq, om);
+    many_mr_last(c, n, end, sq, om, it == 0);
+  }
+  if (iters > 0) return;
+  Many<3> init;
+  Many<2> sum, more;
+  for (int r : set) {
+    LevelWs& W = S.at(l, r);
+    init.add(S.slot(l, r), W.kx1, W.kr1, b[r]);
+    if (!post) continue;
+    sum.add(0, out[r], W.kx1);
+    more.add(0, out[r], W.ke);
+  }
+  if (!post) many_init(c, n, init, sq, nullptr);
+  many_copy(c, n, sum);
+  many_add(c, n, more);
 }
 
-void solve_level_b(sw_mg* mg, int l, const Set& set, BatchCounters& bc);
+void solve_level(Solve& S, int l, const Set& set);
 
-// out_r = M(g_r) on level l for every member of the set.
-void kcycle_b(sw_mg* mg, int l, const Set& set, const std::vector<const double2*>& g,
-              const std::vector<double2*>& out, BatchCounters& bc) {
-  sw_ctx* c = mg->ctx;
-  cudaStream_t s = c->stream;
-  MgLevel& L = mg->lev[l];
-  long n = level_len(mg, l);
-  mr_b(mg, l, set, g, bc);
+// K-cycle preconditioner: out_r = M(g_r) on level l for every member of the set.
+void kcycle(Solve& S, int l, const Set& set, const std::vector<const double2*>& g,
+            const std::vector<double2*>& out) {
+  sw_mg* mg = S.mg;
+  cudaStream_t s = mg->ctx->stream;
+  const MgLevel& L = mg->lev[l];
+  const CoarseGeom cg{L.E0, L.E1, L.nc};
+  trace_norm(S, l, "K-cycle input", g[set[0]]);
+  mr(S, l, set, false, g, out);
+  trace_norm(S, l, "pre-smoothed x", S.at(l, set[0]).kx1);
+  trace_norm(S, l, "pre-smoothed r", S.at(l, set[0]).kr1);
+  Many<2> down, up;
+  Many<3> op, sub;
   for (int r : set) {
-    LevelWs& W = mg->batch.lv[l][r];
-    LevelWs& CW = mg->batch.lv[l + 1][r];
-    if (l == 0)
-      launch_restrict_fine(mg->g, L.b0, L.b1, L.nv, L.P, W.kr1, CW.rhs, s);
-    else
-      launch_restrict_coarse(CoarseGeom{L.E0, L.E1, L.nc}, L.b0, L.b1, L.nv, L.P, W.kr1, CW.rhs, s);
+    LevelWs& W = S.at(l, r);
+    LevelWs& C = S.at(l + 1, r);
+    down.add(0, W.kr1, C.rhs);
+    up.add(0, C.sol, W.ke);
+    op.add(0, W.ke, W.kq, W.tmp);
+    sub.add(0, W.kr1, W.kr1, W.kq);
   }
-  solve_level_b(mg, l + 1, set, bc);
-  std::vector<const double2*> r2(mg->batch.nb, nullptr);
-  for (int r : set) {
-    LevelWs& W = mg->batch.lv[l][r];
-    LevelWs& CW = mg->batch.lv[l + 1][r];
-    if (l == 0)
-      launch_prolong_fine(mg->g, L.b0, L.b1, L.nv, L.P, CW.sol, W.ke, s);
-    else
-      launch_prolong_coarse(CoarseGeom{L.E0, L.E1, L.nc}, L.b0, L.b1, L.nv, L.P, CW.sol, W.ke, s);
-    op_b(mg, l, r, W.ke, W.kq, true, bc);
-    blas_sub(c, W.kr2, W.kr1, W.kq, n);
-    blas_copy(c, W.kx3, W.kx1, n);  // keep x1 while the post-smoother reuses kx1 / kr1
-    r2[r] = W.kr2;
-  }
-  mr_b(mg, l, set, r2, bc);
-  for (int r : set) {
-    LevelWs& W = mg->batch.lv[l][r];
-    blas_add3(c, out[r], W.kx3, W.ke, W.kx1, n);  // (x1 + e) + x3
-  }
+  if (l == 0)
+    many_restrict_fine(mg->g, L.b0, L.b1, L.nv, L.P, down, s, mg->fine_D ? 1 : 0);
+  else
+    many_restrict_coarse(cg, L.b0, L.b1, L.nv, L.P, down, s);
+  trace_norm(S, l + 1, "restricted r", S.at(l + 1, set[0]).rhs);
+  solve_level(S, l + 1, set);
+  if (l == 0)
+    many_prolong_fine(mg->g, L.b0, L.b1, L.nv, L.P, up, s, mg->fine_D ? 1 : 0);
+  else
+    many_prolong_coarse(cg, L.b0, L.b1, L.nv, L.P, up, s);
+  apply(S, l, set, op, true);
+  many_sub(mg->ctx, level_len(mg, l), sub);  // r2 = r1 - op e
+  mr(S, l, set, true, g, out);
 }
 
 struct SetResult {
   std::vector<int> it, restarts;
   std::vector<char> conv;
+  explicit SetResult(int n) : it(n, 0), restarts(n, 0), conv(n, 0) {}
 };
 
-// Flexible GCR (the steps of fgcr above) for every member of the set.
-SetResult fgcr_b(sw_mg* mg, int l, const Set& set, const std::vector<const double2*>& b,
-                 const std::vector<double2*>& x, const std::vector<double>& tol_abs, int restart,
-                 int maxiter, bool confirm, BatchCounters& bc) {
+// Flexible restarted GCR for every member of the set (see the oracle's fgcr for the
+// steps), to |r| <= tol[r] (rel: times |b_r|).  confirm: on the true residual.
+SetResult fgcr(Solve& S, int l, const Set& set, const std::vector<const double2*>& b,
+               const std::vector<double2*>& x, std::vector<double> tol, bool rel, int restart,
+               int maxiter, bool confirm) {
+  sw_mg* mg = S.mg;
   sw_ctx* c = mg->ctx;
-  long n = level_len(mg, l);
-  int nb = mg->batch.nb;
-  SetResult res{std::vector<int>(nb, 0), std::vector<int>(nb, 0), std::vector<char>(nb, 0)};
+  const long n = level_len(mg, l);
+  const int nb = S.width();
+  const bool lowp = l > 0;  // intermediate solves are part of the preconditioner
+  constexpr int s_rr = 0, s_qq = 2, s_a = 3, s_b = 4;
+  double* host = c->h_many->norm;
+  SetResult res(nb);
   std::vector<int> k(nb, 0);
-  std::vector<char> done(nb, 1);
-  for (int r : set) {
-    LevelWs& W = mg->batch.lv[l][r];
-    blas_zero(c, x[r], n);
-    blas_copy(c, W.gr, b[r], n);
-    done[r] = 0;
+  std::vector<double> rn(nb, 0.0);
+  Many<3> init;
+  for (int r : set) init.add(S.slot(l, r), x[r], S.at(l, r).gr, b[r]);
+  many_init(c, n, init, s_rr, host);
+  const double* hn = norms(c);
+  for (size_t m = 0; m < set.size(); ++m) {
+    rn[set[m]] = std::sqrt(hn[m]);
+    check_norm(rn[set[m]], "GCR residual");
+    if (rel) tol[set[m]] *= rn[set[m]];
   }
-  const bool lowp = l > 0;
-  for (;;) {
-    Set act;
-    for (int r : set)
-      if (!done[r]) act.push_back(r);
-    if (act.empty()) break;
-    for (int r : act) blas_norm2(c, mg->batch.lv[l][r].gr, n, slot_base(l) + page(r));
-    const double2* hs = slots_read_all(c, nb);
+  // r = b - op x from x, with its norm
+  const auto true_residual = [&](const Set& who, bool keep) {
+    Many<3> op, sub;
+    for (int r : who) {
+      LevelWs& W = S.at(l, r);
+      op.add(0, x[r], W.gtmp, W.tmp);
+      sub.add(S.slot(l, r), keep ? W.gr : W.gtmp, b[r], W.gtmp);
+    }
+    apply(S, l, who, op, lowp);
+    many_sub_norm(c, n, sub, s_rr, host);
+    hn = norms(c);
+    for (size_t m = 0; m < who.size(); ++m) {
+      rn[who[m]] = std::sqrt(hn[m]);
+      check_norm(rn[who[m]], "GCR true residual");
+    }
+  };
+  for (Set act = set; !act.empty();) {
     Set cand, go;
-    for (int r : act) {
-      double rn = std::sqrt(hs[slot_base(l) + page(r)].x);
-      check_norm(rn, "batched GCR residual");
-      if (rn <= tol_abs[r]) {
-        if (confirm) {
+    for (int r : act)
+      if (rn[r] <= tol[r]) {
+        if (confirm)
           cand.push_back(r);
-        } else {
-          done[r] = 1;
+        else
           res.conv[r] = 1;
-        }
-      } else if (res.it[r] >= maxiter) {
-        done[r] = 1;
-      } else {
+      } else if (res.it[r] < maxiter) {
         go.push_back(r);
       }
-    }
-    if (!cand.empty()) {  // confirm on the true residual, then test everybody again
+    if (!cand.empty()) {
+      true_residual(cand, false);
+      Many<2> keep;
       for (int r : cand) {
-        LevelWs& W = mg->batch.lv[l][r];
-        op_b(mg, l, r, x[r], W.gtmp, lowp, bc);
-        blas_sub(c, W.gtmp, b[r], W.gtmp, n);
-        blas_norm2(c, W.gtmp, n, slot_base(l) + page(r) + 1);
-      }
-      const double2* hs2 = slots_read_all(c, nb);
-      for (int r : cand) {
-        double rt = std::sqrt(hs2[slot_base(l) + page(r) + 1].x);
-        check_norm(rt, "batched GCR true residual");
-        if (rt <= tol_abs[r]) {
-          done[r] = 1;
+        if (rn[r] <= tol[r]) {
           res.conv[r] = 1;
-        } else {
-          LevelWs& W = mg->batch.lv[l][r];
-          blas_copy(c, W.gr, W.gtmp, n);
-          k[r] = 0;
-          res.restarts[r]++;
+          continue;
         }
+        keep.add(0, S.at(l, r).gr, S.at(l, r).gtmp);
+        k[r] = 0;
+        res.restarts[r]++;
+        if (res.it[r] < maxiter) go.push_back(r);
       }
-      continue;
+      many_copy(c, n, keep);
+      std::sort(go.begin(), go.end());
     }
-    if (go.empty()) continue;  // every active member has just stopped
+    act = go;
+    if (go.empty()) break;
     std::vector<const double2*> g(nb, nullptr);
     std::vector<double2*> p(nb, nullptr);
+    Many<3> op, scale;
+    Many<1> alone;
+    Many<2> dots;
+    Many<4> upd;
+    int most = 0;
     for (int r : go) {
-      LevelWs& W = mg->batch.lv[l][r];
+      LevelWs& W = S.at(l, r);
+      const int slot = S.slot(l, r);
+      double2* q = W.gq[k[r]];
       g[r] = W.gr;
       p[r] = W.gp[k[r]];
+      op.add(slot, p[r], q, W.tmp);
+      if (k[r] > 0)
+        dots.add(slot, W.gq[0], q);
+      else
+        alone.add(slot, q);
+      scale.add(slot, q, p[r], W.gr);
+      upd.add(slot, x[r], W.gr, p[r], q);
+      most = std::max(most, k[r]);
     }
-    if (l + 1 < mg->nlev)
-      kcycle_b(mg, l, go, g, p, bc);
-    else
-      for (int r : go) blas_copy(c, p[r], g[r], n);
-    for (int r : go) {
-      LevelWs& W = mg->batch.lv[l][r];
-      int sb = slot_base(l) + page(r);
-      int s_qq = sb + 2, s_a = sb + 3, s_b = sb + 4;
-      double2* q = W.gq[k[r]];
-      double2* pr = W.gp[k[r]];
-      op_b(mg, l, r, pr, q, lowp, bc);
-      for (int j = 0; j < k[r]; ++j) {
-        blas_dot(c, W.gq[j], q, n, s_b);
-        blas_axpy(c, q, W.gq[j], n, coef_ratio(s_b, -1, -1.0));
-        blas_axpy(c, pr, W.gp[j], n, coef_ratio(s_b, -1, -1.0));
+    kcycle(S, l, go, g, p);
+    apply(S, l, go, op, lowp);
+    many_norm(c, n, alone, s_qq);
+    many_dot(c, n, dots, s_b);
+    for (int j = 0; j < most; ++j) {
+      Many<5> mgs;
+      for (int r : go) {
+        if (k[r] <= j) continue;
+        LevelWs& W = S.at(l, r);
+        mgs.add(S.slot(l, r), W.gq[k[r]], p[r], W.gq[j], W.gp[j],
+                j + 1 < k[r] ? W.gq[j + 1] : nullptr);
       }
-      blas_norm2(c, q, n, s_qq);
-      blas_scale(c, q, n, coef_ratio(-1, s_qq, 1.0, COEF_SQRT_DEN));
-      blas_scale(c, pr, n, coef_ratio(-1, s_qq, 1.0, COEF_SQRT_DEN));
-      blas_dot(c, q, W.gr, n, s_a);
-      blas_axpy(c, x[r], pr, n, coef_ratio(s_a, -1, 1.0));
-      blas_axpy(c, W.gr, q, n, coef_ratio(s_a, -1, -1.0));
+      many_mgs(c, n, mgs, s_b, s_qq);
+    }
+    many_scale_dot(c, n, scale, s_qq, s_a);
+    many_update(c, n, upd, s_a, s_rr, host);
+    Set again;
+    for (int r : go) {
       ++k[r];
       ++res.it[r];
+      if (!S.batch && l == 1 && mg->verbose > 1)
+        std::fprintf(stderr, "[sw]   level-2 GCR %d |r| %.3e (tol %.3e)\n", res.it[r], rn[r], tol[r]);
+      if (!S.batch && l == 0 && mg->verbose)
+        std::fprintf(stderr, "[sw] outer %d |r| %.3e  inter %lld/%lld coarsest %lld/%lld\n",
+                     res.it[r], rn[r], S.inter_it[r], S.inter_solves[r], S.coarse_it[r],
+                     S.coarse_solves[r]);
       if (k[r] == restart && res.it[r] < maxiter) {
-        op_b(mg, l, r, x[r], W.gtmp, lowp, bc);
-        blas_sub(c, W.gr, b[r], W.gtmp, n);
+        again.push_back(r);
         k[r] = 0;
         res.restarts[r]++;
       }
     }
+    hn = norms(c);
+    for (size_t m = 0; m < go.size(); ++m) {
+      rn[go[m]] = std::sqrt(hn[m]);
+      check_norm(rn[go[m]], "GCR residual");
+    }
+    if (!again.empty()) true_residual(again, true);
   }
   return res;
+}
+
+void cgne_b(Solve& S, int l, const Set& set, int stall = 0);
+
+void solve_level(Solve& S, int l, const Set& set) {
+  sw_mg* mg = S.mg;
+  if (l == mg->nlev - 1) {
+    if (S.batch) return cgne_b(S, l, set);
+    S.coarse_it[0] += cgne(mg, l, S.at(l, 0).rhs, S.at(l, 0).sol);
+    S.coarse_solves[0]++;
+    return;
+  }
+  std::vector<const double2*> b(S.width(), nullptr);
+  std::vector<double2*> x(S.width(), nullptr);
+  for (int r : set) {
+    b[r] = S.at(l, r).rhs;
+    x[r] = S.at(l, r).sol;
+  }
+  const SetResult res = fgcr(S, l, set, b, x, std::vector<double>(S.width(), mg->p.inter_tol), true,
+                             mg->p.inter_restart, mg->p.inter_maxiter, false);
+  for (int r : set) {
+    S.inter_it[r] += res.it[r];
+    S.inter_solves[r]++;
+  }
 }
 
 // ---------------------------------------------------------------- autotuner
@@ -889,21 +816,21 @@ int tc_stages(sw_mg* mg, const MgLevel& L, int nb, double2* const* bptr, double2
   return best.stages;
 }
 
-void cgne_b(sw_mg* mg, int l, const Set& set, BatchCounters& bc, int stall = 0) {
+void cgne_b(Solve& S, int l, const Set& set, int stall) {
   if (set.empty()) return;
+  sw_mg* mg = S.mg;
   sw_ctx* c = mg->ctx;
   MgLevel& L = mg->lev[l];
   BatchWs& B = mg->batch;
   const int nb = (int)set.size();
   const bool tc = tc_supported(L.nc) && !B.Yf;
   const bool f32 = mg->p.batch_iterates == SW_PREC_FP32;
-  double2* hp[2 * kMaxBatch] = {nullptr};
+  double2** hp = c->h_many->ptr;  // pinned; the wait for the status below ends its use
   for (int i = 0; i < nb; ++i) {
     hp[i] = B.lv[l][set[i]].rhs;
     hp[kMaxBatch + i] = B.lv[l][set[i]].sol;
   }
-  SW_CUDA(cudaMemcpyAsync(B.dptr, hp, sizeof(hp), cudaMemcpyHostToDevice, c->stream));
-  SW_CUDA(cudaStreamSynchronize(c->stream));  // hp is a host stack array
+  SW_CUDA(cudaMemcpyAsync(B.dptr, hp, sizeof(c->h_many->ptr), cudaMemcpyHostToDevice, c->stream));
   SmLease lease(c);
   std::vector<int> its(nb, 0);
   // the CUDA-core FP32 kernel (SW_BATCH_FP32=1) takes at most 16 at a time
@@ -931,8 +858,9 @@ void cgne_b(sw_mg* mg, int l, const Set& set, BatchCounters& bc, int stall = 0) 
     timing_end(c, tk);
     if (!ran)
       throw SwError{SW_ERR_ARG, "no batched coarsest solver for nc = " + std::to_string(L.nc)};
-    int hst[2 + kMaxBatch];
-    SW_CUDA(cudaMemcpyAsync(hst, B.status, sizeof(hst), cudaMemcpyDeviceToHost, c->stream));
+    const int* hst = c->h_many->status;
+    SW_CUDA(cudaMemcpyAsync(c->h_many->status, B.status, sizeof(c->h_many->status),
+                            cudaMemcpyDeviceToHost, c->stream));
     SW_CUDA(cudaStreamSynchronize(c->stream));
     if (!c->pending.empty()) timing_harvest(c);
     if (hst[0])
@@ -947,36 +875,8 @@ void cgne_b(sw_mg* mg, int l, const Set& set, BatchCounters& bc, int stall = 0) 
     if (c->timing) c->t_count[kCatCgne + 1] += kernel_it;
   }
   for (int i = 0; i < nb; ++i) {
-    bc.coarse_it[set[i]] += its[i];
-    bc.coarse_solves[set[i]]++;
-  }
-}
-
-void solve_level_b(sw_mg* mg, int l, const Set& set, BatchCounters& bc) {
-  sw_ctx* c = mg->ctx;
-  if (l == mg->nlev - 1) {
-    cgne_b(mg, l, set, bc);
-    return;
-  }
-  long n = level_len(mg, l);
-  int nb = mg->batch.nb;
-  for (int r : set) blas_norm2(c, mg->batch.lv[l][r].rhs, n, slot_base(l) + page(r) + 5);
-  const double2* hs = slots_read_all(c, nb);
-  std::vector<double> tol(nb, 0.0);
-  std::vector<const double2*> b(nb, nullptr);
-  std::vector<double2*> x(nb, nullptr);
-  for (int r : set) {
-    double bn = std::sqrt(hs[slot_base(l) + page(r) + 5].x);
-    check_norm(bn, "batched intermediate right-hand side");
-    tol[r] = mg->p.inter_tol * bn;
-    b[r] = mg->batch.lv[l][r].rhs;
-    x[r] = mg->batch.lv[l][r].sol;
-  }
-  SetResult res =
-      fgcr_b(mg, l, set, b, x, tol, mg->p.inter_restart, mg->p.inter_maxiter, false, bc);
-  for (int r : set) {
-    bc.inter_it[r] += res.it[r];
-    bc.inter_solves[r]++;
+    S.coarse_it[set[i]] += its[i];
+    S.coarse_solves[set[i]]++;
   }
 }
 
@@ -1008,7 +908,8 @@ void batch_alloc(sw_mg* mg, int nb) {
           W.gq[k] = mg_alloc(mg, n);
         }
         W.kx1 = mg_alloc(mg, n); W.kr1 = mg_alloc(mg, n); W.kq = mg_alloc(mg, n);
-        W.ke = mg_alloc(mg, n); W.kr2 = mg_alloc(mg, n); W.kx3 = mg_alloc(mg, n);
+        W.ke = mg_alloc(mg, n); W.kx3 = mg_alloc(mg, n);
+        if (l == 0) W.tmp = mg_alloc(mg, n);
       }
     }
     B.nb = cap;
@@ -1056,6 +957,71 @@ void batch_alloc(sw_mg* mg, int nb) {
 
 }  // namespace
 
+// ---------------------------------------------------------------- solve
+int mg_solve_device(sw_mg* mg, const double2* b_lex, double2* x_lex, double tol,
+                    sw_solve_stats* st) {
+  sw_ctx* c = mg->ctx;
+  sw_gauge* g = mg->g;
+  cudaStream_t s = c->stream;
+  long N = g->N, half = N / 2;
+  auto t0 = std::chrono::steady_clock::now();
+  MgLevel& L = mg->lev[0];
+  launch_pack(g, b_lex, mg->bps, s);
+  int sb = slot_base(0);
+  blas_norm2(c, mg->bps, N, sb + 40);
+  double bn = std::sqrt(slot_read(c, sb + 40).x);
+  check_norm(bn, "right-hand side");
+  if (bn == 0.0) {
+    blas_zero(c, x_lex, N);
+    SW_CUDA(cudaStreamSynchronize(s));
+    if (st) {
+      std::memset(st, 0, sizeof(*st));
+      st->converged = 1;
+    }
+    return SW_OK;
+  }
+  Solve S(mg, false);
+  const std::vector<double> tol_abs(1, tol * bn);
+  SetResult r(1);
+  if (mg->fine_D) {
+    // Galerkin MG of D itself: flexible GCR on the full D, no KD preconditioning
+    r = fgcr(S, 0, {0}, {mg->bps}, {L.sol}, tol_abs, false, mg->p.outer_restart,
+             mg->p.outer_maxiter, true);
+    launch_unpack(g, L.sol, x_lex, s);
+  } else {
+    // b~_e = b_e - A_eo b_o = b_e - C_eo B_o^-1 b_o
+    launch_block_apply(g, mg->binv, 1, 0, mg->bps + half, L.stmp + half, s);
+    launch_hop(g, 0, -1.0, mg->bps, L.stmp + half, L.rhs, s);
+    r = fgcr(S, 0, {0}, {L.rhs}, {L.sol}, tol_abs, false, mg->p.outer_restart,
+             mg->p.outer_maxiter, true);
+    // z_o = b_o - C_oe B_e^-1 z_e ; x = B^-1 z
+    launch_block_apply(g, mg->binv, 0, 0, L.sol, L.stmp, s);
+    launch_hop(g, 1, -1.0, mg->bps + half, L.stmp, L.stmp + half, s);
+    launch_block_apply(g, mg->binv, 0, 0, L.sol, mg->xps, s);
+    launch_block_apply(g, mg->binv, 1, 0, L.stmp + half, mg->xps + half, s);
+    launch_unpack(g, mg->xps, x_lex, s);
+  }
+  // true residual ||b - D x|| / ||b|| in FP64
+  launch_dslash_lex(g, mg->mass, 0, x_lex, mg->lext, s);
+  blas_sub(c, mg->lext, b_lex, mg->lext, N);
+  blas_norm2(c, mg->lext, N, sb + 41);
+  double tr = std::sqrt(slot_read(c, sb + 41).x) / bn;
+  auto t1 = std::chrono::steady_clock::now();
+  if (st) {
+    st->converged = r.conv[0] ? 1 : 0;
+    st->outer_iters = r.it[0];
+    st->restarts = r.restarts[0];
+    st->fine_applies = S.fine[0];
+    st->inter_iters = S.inter_it[0];
+    st->inter_solves = S.inter_solves[0];
+    st->coarsest_iters = S.coarse_it[0];
+    st->coarsest_solves = S.coarse_solves[0];
+    st->true_resid = tr;
+    st->seconds = std::chrono::duration<double>(t1 - t0).count();
+  }
+  return r.conv[0] ? SW_OK : SW_ERR_NOCONV;
+}
+
 int mg_solve_batch_device(sw_mg* mg, int nb, const double2* Bl, double2* Xl, double tol,
                           sw_solve_stats* st) {
   sw_ctx* c = mg->ctx;
@@ -1068,54 +1034,69 @@ int mg_solve_batch_device(sw_mg* mg, int nb, const double2* Bl, double2* Xl, dou
   BatchWs& B = mg->batch;
   long N = g->N, half = N / 2;
   MgLevel& L = mg->lev[0];
+  Solve S(mg, true);
+  Many<1> bs;
   for (int r = 0; r < nb; ++r) {
     launch_pack(g, Bl + (long)r * N, B.bps + (long)r * N, s);
-    blas_norm2(c, B.bps + (long)r * N, N, slot_base(0) + page(r) + 40);
+    bs.add(S.slot(0, r), B.bps + (long)r * N);
   }
-  const double2* hs = slots_read_all(c, nb);
-  std::vector<double> bn(nb), tol_abs(nb);
+  many_norm(c, N, bs, 40, c->h_many->norm);
+  const double* hn = norms(c);
+  std::vector<double> bn(nb), tol_abs(kMaxBatch, 0.0);
   Set all;
   for (int r = 0; r < nb; ++r) {
-    bn[r] = std::sqrt(hs[slot_base(0) + page(r) + 40].x);
+    bn[r] = std::sqrt(hn[r]);
     check_norm(bn[r], "right-hand side");
     tol_abs[r] = tol * bn[r];
     if (bn[r] > 0.0) all.push_back(r);
   }
   std::vector<const double2*> bt(kMaxBatch, nullptr);
   std::vector<double2*> z(kMaxBatch, nullptr);
+  Many<2> odd;
+  Many<3> rhs;
   for (int r = 0; r < nb; ++r) {
-    double2* bps = B.bps + (long)r * N;
-    LevelWs& W = B.lv[0][r];
     // b~_e = b_e - C_eo B_o^-1 b_o
-    launch_block_apply(g, mg->binv, 1, 0, bps + half, L.stmp + half, s);
-    launch_hop(g, 0, -1.0, bps, L.stmp + half, W.rhs, s);
+    double2* bps = B.bps + (long)r * N;
+    double2* t = B.xps + (long)r * N;
+    LevelWs& W = B.lv[0][r];
+    odd.add(0, bps + half, t);
+    rhs.add(0, bps, t, W.rhs);
     bt[r] = W.rhs;
     z[r] = W.sol;
   }
-  BatchCounters bc(kMaxBatch);
-  SetResult res = fgcr_b(mg, 0, all, bt, z, tol_abs, mg->p.outer_restart, mg->p.outer_maxiter,
-                         true, bc);
+  many_block_apply(g, mg->binv, 1, 0, odd, s);
+  many_hop(g, 0, -1.0, rhs, s);
+  SetResult res(kMaxBatch);
+  if (!all.empty())
+    res = fgcr(S, 0, all, bt, z, tol_abs, false, mg->p.outer_restart, mg->p.outer_maxiter, true);
+  Many<2> even, xe, xo;
+  Many<3> zo, diff;
   for (int r = 0; r < nb; ++r) {
-    double2* x = Xl + (long)r * N;
     if (bn[r] == 0.0) {
-      blas_zero(c, x, N);
+      blas_zero(c, Xl + (long)r * N, N);
       continue;
     }
-    double2* bps = B.bps + (long)r * N;
-    double2* xps = B.xps + (long)r * N;
-    LevelWs& W = B.lv[0][r];
     // z_o = b_o - C_oe B_e^-1 z_e ; x = B^-1 z
-    launch_block_apply(g, mg->binv, 0, 0, W.sol, L.stmp, s);
-    launch_hop(g, 1, -1.0, bps + half, L.stmp, L.stmp + half, s);
-    launch_block_apply(g, mg->binv, 0, 0, W.sol, xps, s);
-    launch_block_apply(g, mg->binv, 1, 0, L.stmp + half, xps + half, s);
-    launch_unpack(g, xps, x, s);
     double2* t = B.lex + (long)r * N;
-    launch_dslash_lex(g, mg->mass, 0, x, t, s);
-    blas_sub(c, t, Bl + (long)r * N, t, N);
-    blas_norm2(c, t, N, slot_base(0) + page(r) + 41);
+    double2* xps = B.xps + (long)r * N;
+    even.add(0, z[r], xps);  // the even half of x as well
+    zo.add(0, B.bps + (long)r * N + half, xps, t + half);
+    xo.add(0, t + half, xps + half);
+    diff.add(S.slot(0, r), t, Bl + (long)r * N, t);
   }
-  const double2* hs2 = slots_read_all(c, nb);
+  if (!all.empty()) {
+    many_block_apply(g, mg->binv, 0, 0, even, s);
+    many_hop(g, 1, -1.0, zo, s);
+    many_block_apply(g, mg->binv, 1, 0, xo, s);
+  }
+  for (int r : all) {
+    launch_unpack(g, B.xps + (long)r * N, Xl + (long)r * N, s);
+    launch_dslash_lex(g, mg->mass, 0, Xl + (long)r * N, B.lex + (long)r * N, s);
+  }
+  many_sub_norm(c, N, diff, 41, c->h_many->norm);
+  hn = norms(c);
+  std::vector<double> rr(nb, 0.0);
+  for (size_t m = 0; m < all.size(); ++m) rr[all[m]] = hn[m];
   double secs = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
   bool ok = true;
   for (int r = 0; r < nb; ++r) {
@@ -1127,12 +1108,12 @@ int mg_solve_batch_device(sw_mg* mg, int nb, const double2* Bl, double2* Xl, dou
     o.converged = conv ? 1 : 0;
     o.outer_iters = res.it[r];
     o.restarts = res.restarts[r];
-    o.fine_applies = bc.fine[r];
-    o.inter_iters = bc.inter_it[r];
-    o.inter_solves = bc.inter_solves[r];
-    o.coarsest_iters = bc.coarse_it[r];
-    o.coarsest_solves = bc.coarse_solves[r];
-    o.true_resid = bn[r] > 0.0 ? std::sqrt(hs2[slot_base(0) + page(r) + 41].x) / bn[r] : 0.0;
+    o.fine_applies = S.fine[r];
+    o.inter_iters = S.inter_it[r];
+    o.inter_solves = S.inter_solves[r];
+    o.coarsest_iters = S.coarse_it[r];
+    o.coarsest_solves = S.coarse_solves[r];
+    o.true_resid = bn[r] > 0.0 ? std::sqrt(rr[r]) / bn[r] : 0.0;
     o.seconds = secs;
   }
   return ok ? SW_OK : SW_ERR_NOCONV;
@@ -1146,8 +1127,8 @@ int mg_batch_stall(sw_mg* mg, int nb) {
   for (int r = 0; r < nb; ++r) blas_zero(mg->ctx, mg->batch.lv[l][r].rhs, level_len(mg, l));
   Set set;
   for (int r = 0; r < nb; ++r) set.push_back(r);
-  BatchCounters bc(kMaxBatch);
-  cgne_b(mg, l, set, bc, 1);
+  Solve S(mg, true);
+  cgne_b(S, l, set, 1);
   return SW_OK;
 }
 

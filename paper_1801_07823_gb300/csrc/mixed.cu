@@ -7,6 +7,7 @@
 //  - conversion of a stencil to double-float (df64, used by the coarsest CGNE).
 #include <cuda_fp16.h>
 
+#include "many.h"
 #include "sw_internal.h"
 
 namespace {
@@ -44,8 +45,10 @@ __global__ void k_to_f32(const double2* __restrict__ in, float2* __restrict__ ou
 }
 
 // out (float) = M in (double -> float), M per KD block of one parity half
-__global__ void k_block_apply_df(const float2* __restrict__ M, const double2* __restrict__ in,
-                                 float2* __restrict__ out, int nblk) {
+template <int W>
+__global__ void k_block_apply_df(const float2* __restrict__ M, Pack<2, W> io, int nblk) {
+  const double2* __restrict__ in = io.v[0][blockIdx.y];
+  float2* __restrict__ out = (float2*)io.v[1][blockIdx.y];
   int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= nblk) return;
   float2 v[4];
@@ -67,19 +70,19 @@ __device__ __forceinline__ float2 hop_out_f(const float2* __restrict__ W, const 
   float2 acc = make_float2(0.f, 0.f);
   if (x0 & 1) {
     int t = ps_index(x0 + 1 == L0 ? 0 : x0 + 1, x1, L0, N);
-    cfmaf(acc, W[f], in[t % half]);
+    cfmaf(acc, W[f], in[t < half ? t : t - half]);
   } else {
     int t = ps_index(x0 == 0 ? L0 - 1 : x0 - 1, x1, L0, N);
-    float2 w = W[t], v = in[t % half];
+    float2 w = W[t], v = in[t < half ? t : t - half];
     acc.x -= w.x * v.x + w.y * v.y;
     acc.y -= w.x * v.y - w.y * v.x;
   }
   if (x1 & 1) {
     int t = ps_index(x0, x1 + 1 == L1 ? 0 : x1 + 1, L0, N);
-    cfmaf(acc, W[N + f], in[t % half]);
+    cfmaf(acc, W[N + f], in[t < half ? t : t - half]);
   } else {
     int t = ps_index(x0, x1 == 0 ? L1 - 1 : x1 - 1, L0, N);
-    float2 w = W[N + t], v = in[t % half];
+    float2 w = W[N + t], v = in[t < half ? t : t - half];
     acc.x -= w.x * v.x + w.y * v.y;
     acc.y -= w.x * v.y - w.y * v.x;
   }
@@ -87,9 +90,11 @@ __device__ __forceinline__ float2 hop_out_f(const float2* __restrict__ W, const 
 }
 
 // out_o (float) = M_o (C_oe in_e), per odd KD block
+template <int WIDTH>
 __global__ void k_hop_block_ff(const float2* __restrict__ W, const float2* __restrict__ M, int par,
-                               const float2* __restrict__ in, float2* __restrict__ out, int L0,
-                               int L1) {
+                               Pack<2, WIDTH> io, int L0, int L1) {
+  const float2* __restrict__ in = (const float2*)io.v[0][blockIdx.y];
+  float2* __restrict__ out = (float2*)io.v[1][blockIdx.y];
   int N = L0 * L1, half = N >> 1;
   int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= (half >> 2)) return;
@@ -104,9 +109,12 @@ __global__ void k_hop_block_ff(const float2* __restrict__ W, const float2* __res
 }
 
 // out_e (double) = src_e - C_eo in_o
-__global__ void k_hop_sub_fd(const float2* __restrict__ W, int par,
-                             const double2* __restrict__ src, const float2* __restrict__ in,
-                             double2* __restrict__ out, int L0, int L1) {
+template <int WIDTH>
+__global__ void k_hop_sub_fd(const float2* __restrict__ W, int par, Pack<3, WIDTH> io, int L0,
+                             int L1) {
+  const double2* __restrict__ src = io.v[0][blockIdx.y];
+  const float2* __restrict__ in = (const float2*)io.v[1][blockIdx.y];
+  double2* __restrict__ out = io.v[2][blockIdx.y];
   int N = L0 * L1, half = N >> 1;
   int h = blockIdx.x * blockDim.x + threadIdx.x;
   if (h >= half) return;
@@ -149,12 +157,13 @@ __global__ void k_to_half_scaled(const double2* __restrict__ Y, __half2* __restr
 // y_X = sum_d s[X][d] Yh[X][d] x_{X+d} (DAG: sum_d s[Z][opp] Yh[Z][opp]^dag x_Z, Z = X+d),
 // FP32 products and sums, FP64 vectors in and out.  Thread layout as the FP64
 // kernel: (direction d, row i), rs CTAs per site when there are few sites.
-template <int NC, bool DAG>
+// One member of a batch per blockIdx.y: the stencil comes from L2 for all but the first.
+template <int NC, bool DAG, int W>
 __global__ void __launch_bounds__(5 * NC) k_coarse_apply_h(const __half2* __restrict__ Yh,
                                                            const float* __restrict__ scale,
-                                                           const double2* __restrict__ in,
-                                                           double2* __restrict__ out, int E0,
-                                                           int E1, int rs) {
+                                                           Pack<2, W> io, int E0, int E1, int rs) {
+  const double2* __restrict__ in = io.v[0][blockIdx.y];
+  double2* __restrict__ out = io.v[1][blockIdx.y];
   __shared__ float2 xs[5][NC];
   __shared__ float2 part[5][NC];
   int rows = NC / rs;
@@ -197,10 +206,11 @@ __global__ void __launch_bounds__(5 * NC) k_coarse_apply_h(const __half2* __rest
 }
 
 // Generic-nc fallback: one thread per (site, row), all five directions.
-template <bool DAG>
+template <bool DAG, int W>
 __global__ void k_coarse_apply_h_any(const __half2* __restrict__ Yh, const float* __restrict__ scale,
-                                     const double2* __restrict__ in, double2* __restrict__ out,
-                                     int E0, int E1, int nc) {
+                                     Pack<2, W> io, int E0, int E1, int nc) {
+  const double2* __restrict__ in = io.v[0][blockIdx.y];
+  double2* __restrict__ out = io.v[1][blockIdx.y];
   long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (long)E0 * E1 * nc) return;
   int X = (int)(e / nc), i = (int)(e - (long)X * nc);
@@ -232,17 +242,18 @@ __global__ void k_to_df64(const double2* __restrict__ Y, float4* __restrict__ Yd
 
 template <int NC>
 void apply_h_nc(const CoarseGeom& g, const __half2* Yh, const float* sc, int dagger,
-                const double2* in, double2* out, cudaStream_t s) {
+                const Many<2>& io, cudaStream_t s) {
   int nsites = g.E0 * g.E1;
   int rs = 1;
-  while (rs < 8 && NC % (2 * rs) == 0 && (NC / (2 * rs)) % 8 == 0 && (long)nsites * rs < 4 * 152)
+  while (rs < 8 && NC % (2 * rs) == 0 && (NC / (2 * rs)) % 8 == 0 &&
+         (long)nsites * rs * io.n < 4 * 152)
     rs *= 2;
-  if (dagger)
-    k_coarse_apply_h<NC, true><<<nsites * rs, 5 * (NC / rs), 0, s>>>(Yh, sc, in, out, g.E0, g.E1, rs);
-  else
-    k_coarse_apply_h<NC, false><<<nsites * rs, 5 * (NC / rs), 0, s>>>(Yh, sc, in, out, g.E0, g.E1,
-                                                                      rs);
-  SW_LAUNCH_CHECK();
+  with_width(io.n, [&](auto w) {
+    constexpr int W = decltype(w)::value;
+    auto k = dagger ? k_coarse_apply_h<NC, true, W> : k_coarse_apply_h<NC, false, W>;
+    k<<<dim3(nsites * rs, io.n), 5 * (NC / rs), 0, s>>>(Yh, sc, Pack<2, W>(io), g.E0, g.E1, rs);
+    SW_LAUNCH_CHECK();
+  });
 }
 
 }  // namespace
@@ -253,17 +264,29 @@ void launch_to_f32(const double2* in, float2* out, long n, cudaStream_t s) {
 }
 
 // S x_e in FP32 arithmetic: t = B_e^-1 x_e, v = B_o^-1 C_oe t, y = x_e - C_eo v.
-// tmp: N float2.  W32: FP32 links (parity-split), binv32: FP32 B^-1 table.
-void fine_apply_S32(const sw_gauge* g, const float2* W32, const float2* binv32,
-                    const double2* in_e, double2* out_e, float2* tmp, cudaStream_t s) {
+// W32: FP32 links (parity-split), binv32: FP32 B^-1 table; t lies in out, v in tmp.
+void many_S32(const sw_gauge* g, const float2* W32, const float2* binv32, const Many<3>& v,
+              cudaStream_t s) {
   int N = g->N, half = N / 2, nblk = N / 8;
-  k_block_apply_df<<<cdiv(nblk, 128), 128, 0, s>>>(binv32, in_e, tmp, nblk);
-  SW_LAUNCH_CHECK();
-  k_hop_block_ff<<<cdiv(nblk, 128), 128, 0, s>>>(W32, binv32 + (long)nblk * 16, 1, tmp, tmp + half,
-                                                 g->L0, g->L1);
-  SW_LAUNCH_CHECK();
-  k_hop_sub_fd<<<cdiv(half, 256), 256, 0, s>>>(W32, 0, in_e, tmp + half, out_e, g->L0, g->L1);
-  SW_LAUNCH_CHECK();
+  Many<2> in_t, t_v;
+  Many<3> last;
+  for (int m = 0; m < v.n; ++m) {
+    in_t.add(0, v.v[0][m], v.v[1][m]);
+    t_v.add(0, v.v[1][m], v.v[2][m]);
+    last.add(0, v.v[0][m], v.v[2][m], v.v[1][m]);
+  }
+  with_width(v.n, [&](auto w) {
+    constexpr int W = decltype(w)::value;
+    const dim3 blocks(cdiv(nblk, 128), v.n);
+    k_block_apply_df<W><<<blocks, 128, 0, s>>>(binv32, Pack<2, W>(in_t), nblk);
+    SW_LAUNCH_CHECK();
+    k_hop_block_ff<W><<<blocks, 128, 0, s>>>(W32, binv32 + (long)nblk * 16, 1, Pack<2, W>(t_v),
+                                             g->L0, g->L1);
+    SW_LAUNCH_CHECK();
+    k_hop_sub_fd<W><<<dim3(cdiv(half, 256), v.n), 256, 0, s>>>(W32, 0, Pack<3, W>(last), g->L0,
+                                                               g->L1);
+    SW_LAUNCH_CHECK();
+  });
 }
 
 void launch_to_half_scaled(const CoarseGeom& g, const double2* Y, __half2* Yh, float* scale,
@@ -272,22 +295,27 @@ void launch_to_half_scaled(const CoarseGeom& g, const double2* Y, __half2* Yh, f
   SW_LAUNCH_CHECK();
 }
 
-void launch_coarse_apply_h(const CoarseGeom& g, const __half2* Yh, const float* scale, int dagger,
-                           const double2* in, double2* out, cudaStream_t s) {
+void many_coarse_h(const CoarseGeom& g, const __half2* Yh, const float* scale, int dagger,
+                   const Many<2>& io, cudaStream_t s) {
   switch (g.nc) {
-    case 16: return apply_h_nc<16>(g, Yh, scale, dagger, in, out, s);
-    case 24: return apply_h_nc<24>(g, Yh, scale, dagger, in, out, s);
-    case 32: return apply_h_nc<32>(g, Yh, scale, dagger, in, out, s);
-    case 48: return apply_h_nc<48>(g, Yh, scale, dagger, in, out, s);
-    case 64: return apply_h_nc<64>(g, Yh, scale, dagger, in, out, s);
+    case 16: return apply_h_nc<16>(g, Yh, scale, dagger, io, s);
+    case 24: return apply_h_nc<24>(g, Yh, scale, dagger, io, s);
+    case 32: return apply_h_nc<32>(g, Yh, scale, dagger, io, s);
+    case 48: return apply_h_nc<48>(g, Yh, scale, dagger, io, s);
+    case 64: return apply_h_nc<64>(g, Yh, scale, dagger, io, s);
     default: break;
   }
   long n = (long)g.E0 * g.E1 * g.nc;
-  if (dagger)
-    k_coarse_apply_h_any<true><<<cdiv(n, 128), 128, 0, s>>>(Yh, scale, in, out, g.E0, g.E1, g.nc);
-  else
-    k_coarse_apply_h_any<false><<<cdiv(n, 128), 128, 0, s>>>(Yh, scale, in, out, g.E0, g.E1, g.nc);
-  SW_LAUNCH_CHECK();
+  with_width(io.n, [&](auto w) {
+    constexpr int W = decltype(w)::value;
+    auto k = dagger ? k_coarse_apply_h_any<true, W> : k_coarse_apply_h_any<false, W>;
+    k<<<dim3(cdiv(n, 128), io.n), 128, 0, s>>>(Yh, scale, Pack<2, W>(io), g.E0, g.E1, g.nc);
+    SW_LAUNCH_CHECK();
+  });
+}
+void launch_coarse_apply_h(const CoarseGeom& g, const __half2* Yh, const float* scale, int dagger,
+                           const double2* in, double2* out, cudaStream_t s) {
+  many_coarse_h(g, Yh, scale, dagger, Many<2>(0, in, out), s);
 }
 
 void launch_to_df64(const double2* Y, float4* Yd, long n, cudaStream_t s) {

@@ -54,30 +54,19 @@ int guarded(sw_ctx* c, F&& f);
 // ---------------------------------------------------------------- scalars
 // Krylov coefficients live in a small device array of complex slots so that
 // kernels can use them without a host round trip.  A Coef describes
-//   value = scale * f(S[num]) / g(S[den].re)
-// with f = identity or conjugate (num < 0: 1) and g = identity or sqrt
-// (den < 0: 1).
-enum { COEF_CONJ = 1, COEF_SQRT_DEN = 2 };
+// scale * S[num] / S[den].re.
 struct Coef {
   int num;
   int den;
-  int mode;
   double scale;
 };
-static inline Coef coef_const(double s) { return Coef{-1, -1, 0, s}; }
-static inline Coef coef_ratio(int num, int den, double s = 1.0, int mode = 0) {
-  return Coef{num, den, mode, s};
-}
+static inline Coef coef_ratio(int num, int den, double s) { return Coef{num, den, s}; }
 
 __device__ __forceinline__ double2 coef_eval(const double2* S, Coef c) {
-  double2 v = (c.num >= 0) ? S[c.num] : make_double2(1.0, 0.0);
-  if (c.mode & COEF_CONJ) v.y = -v.y;
-  if (c.den >= 0) {
-    double d = S[c.den].x;
-    if (c.mode & COEF_SQRT_DEN) d = sqrt(d);
-    v.x /= d;
-    v.y /= d;
-  }
+  double2 v = S[c.num];
+  const double d = S[c.den].x;
+  v.x /= d;
+  v.y /= d;
   v.x *= c.scale;
   v.y *= c.scale;
   return v;
@@ -86,6 +75,7 @@ __device__ __forceinline__ double2 coef_eval(const double2* S, Coef c) {
 constexpr int kSlotPage = 320;  // 64 per multigrid level (up to 4), 64 for other solvers
 constexpr int kMaxBatch = 64;   // right-hand sides solved together by sw_mg_solve_batch
 constexpr int kNumSlots = kSlotPage * (kMaxBatch + 1);  // page 0: single solves; 1..64: batch
+constexpr int kManyBlocks = 608;  // CTAs of a batched sum per member, 4 x 152 SMs
 constexpr int kReduceBlocks = 304;  // 2 x 152 SMs; fixed so every sum has one order
 
 // Per-category kernel timing with CUDA events on the context stream.
@@ -93,8 +83,16 @@ constexpr int kTimeCats = 8;  // 0: fine Schur operator, l: coarse operator of l
                               // kCatCgne: the persistent coarsest CGNE kernel
 constexpr int kCatCgne = 5;
 struct TimedPair {
-  int cat;
+  int cat, n;  // n: members of the batch
   cudaEvent_t a, b;
+};
+
+// Pinned host memory of lockstep solves.
+struct HostMany {
+  double norm[kMaxBatch];          // written by the kernels
+  double2* ptr[2 * kMaxBatch];     // b and x of a batched coarsest solve
+  int ctl[4 * kMaxBatch];
+  int status[2 + kMaxBatch];
 };
 
 struct sw_ctx {
@@ -116,6 +114,10 @@ struct sw_ctx {
   unsigned* bar = nullptr;       // grid-barrier state of persistent kernels (2 words)
   int* cgstat = nullptr;         // status words of the persistent CGNE (3 ints)
   double2* h_slots = nullptr;    // pinned host mirror
+  double* many_partials = nullptr;    // device [kMaxBatch][kManyBlocks][4], sums of many.cu
+  unsigned* many_counters = nullptr;  // device [kMaxBatch]
+  int* many_ctl = nullptr;            // device [kMaxBatch][4], iteration control
+  HostMany* h_many = nullptr;         // pinned
   int sm_num = 1, sm_den = 1;    // share of the SMs its persistent kernels may hold
 };
 
@@ -204,20 +206,8 @@ void launch_block_apply(const sw_gauge* g, const double2* binv, int par, int dag
 // out_p = src_p + sign * C_{p,1-p} in_{1-p} on the sites of parity half p.
 void launch_hop(const sw_gauge* g, int par, double sign, const double2* src, const double2* in,
                 double2* out, cudaStream_t s);
-// out_p = src_p + sign * M_p (C_{p,1-p} in_{1-p}), M = B^-1 or B^-dag, per KD block.
-void launch_hop_block(const sw_gauge* g, const double2* binv, int par, int dagger, double sign,
-                      const double2* src, const double2* in, double2* out, cudaStream_t s);
 
-// Fine operator compositions on parity-split vectors (full: N, half: N/2).
-// tmp must hold N complex.
-void fine_apply_A(const sw_gauge* g, const double2* binv, const double2* in, double2* out,
-                  double2* tmp, cudaStream_t s);
-void fine_apply_Adag(const sw_gauge* g, const double2* binv, const double2* in, double2* out,
-                     cudaStream_t s);
-void fine_apply_S(const sw_gauge* g, const double2* binv, const double2* in_e, double2* out_e,
-                  double2* tmp, cudaStream_t s);
-
-// The same on lexicographic fields (out neither in nor tmp; tmp: N).
+// KD operators A, A^dag and S (many.h) on lexicographic fields (out neither in nor tmp; tmp: N).
 void fine_lex_A(const sw_gauge* g, const double2* binv, const double2* in, double2* out,
                 double2* tmp, cudaStream_t s);
 void fine_lex_Adag(const sw_gauge* g, const double2* binv, const double2* in, double2* out,
@@ -227,29 +217,23 @@ void fine_lex_S(const sw_gauge* g, const double2* binv, const double2* in, doubl
 
 // ------------------------------------------------------------- blas.cu
 // skip: optional device flag; when it holds a non-zero value the kernel does nothing.
-void blas_dot(sw_ctx* c, const double2* a, const double2* b, long n, int slot,
-              const int* skip = nullptr);
 void blas_norm2(sw_ctx* c, const double2* a, long n, int slot, const int* skip = nullptr);
 void blas_axpy(sw_ctx* c, double2* y, const double2* x, long n, Coef a,
                const int* skip = nullptr);                                    // y += a x
 void blas_xpay(sw_ctx* c, double2* y, const double2* x, long n, Coef a,
                const int* skip = nullptr);                                    // y = x + a y
-void blas_scale(sw_ctx* c, double2* y, long n, Coef a);                       // y *= a
 void blas_copy(sw_ctx* c, double2* y, const double2* x, long n);
 void blas_zero(sw_ctx* c, double2* y, long n);
 void blas_sub(sw_ctx* c, double2* out, const double2* a, const double2* b, long n);  // a - b
-void blas_add3(sw_ctx* c, double2* out, const double2* a, const double2* b, const double2* d,
-               long n);                                                               // a + b + d
 double2 slot_read(sw_ctx* c, int slot);  // synchronises the stream, harvests timings
 // Device-gated iteration control (see blas.cu); ctl points to 3 device ints.
 void iter_init(sw_ctx* c, int* ctl, int slot, double stop, int maxit);
 void iter_check(sw_ctx* c, int* ctl, int slot, double stop, int maxit);
 void iter_read(sw_ctx* c, const int* ctl, int* host3);  // synchronises
 // Timing brackets (no-ops unless c->timing): timing_begin returns a token.
-int timing_begin(sw_ctx* c, int cat);
+int timing_begin(sw_ctx* c, int cat, int members = 1);
 void timing_end(sw_ctx* c, int token);
 void timing_harvest(sw_ctx* c);  // stream must be synchronised
-void slot_set(sw_ctx* c, int slot, double2 v);
 
 // ------------------------------------------------------------- coarse.cu
 struct CoarseGeom {
@@ -323,8 +307,6 @@ bool launch_cgne_tc(const CoarseGeom& g, int stages, bool f32, const float* At, 
 void launch_adjoint_f32(const CoarseGeom& g, const double2* Y, float2* Yd, cudaStream_t s);
 
 // ------------------------------------------------------------- mixed.cu
-void fine_apply_S32(const sw_gauge* g, const float2* W32, const float2* binv32,
-                    const double2* in_e, double2* out_e, float2* tmp, cudaStream_t s);
 void launch_to_f32(const double2* in, float2* out, long n, cudaStream_t s);
 void launch_to_half_scaled(const CoarseGeom& g, const double2* Y, __half2* Yh, float* scale,
                            cudaStream_t s);
@@ -333,22 +315,8 @@ void launch_coarse_apply_h(const CoarseGeom& g, const __half2* Yh, const float* 
 void launch_to_df64(const double2* Y, float4* Yd, long n, cudaStream_t s);
 void launch_coarse_apply_df(const CoarseGeom& g, const float4* Y, int dagger, const double2* in,
                             double2* out, cudaStream_t s);
-// Level-1 transfer on the even parity half.  P: [N][nv] parity-split rows.
-// full = 1: full parity-split vectors (fine operator D) instead of the even half.
-// lex: the fine vector is a whole lexicographic field (odd sites ignored, or written as 0).
-void launch_restrict_fine(const sw_gauge* g, int a0, int a1, int nv, const double2* P,
-                          const double2* r_e, double2* out, cudaStream_t s, int full = 0,
-                          bool lex = false);
-void launch_prolong_fine(const sw_gauge* g, int a0, int a1, int nv, const double2* P,
-                         const double2* ehat, double2* e_e, cudaStream_t s, int full = 0,
-                         bool lex = false);
 void launch_build_W_identity(const sw_gauge* g, int nv, const double2* P, double2* Wv,
                              cudaStream_t s);
-// Level >= 2 transfer.  P: [sites][nc][nv].
-void launch_restrict_coarse(const CoarseGeom& g, int b0, int b1, int nv, const double2* P,
-                            const double2* r, double2* out, cudaStream_t s);
-void launch_prolong_coarse(const CoarseGeom& g, int b0, int b1, int nv, const double2* P,
-                           const double2* ehat, double2* e, cudaStream_t s);
 // Aggregate / chirality maps of a level from the transfer kernels' index maps.
 void launch_level_maps_fine(const sw_gauge* g, int a0, int a1, int* agg, int* chir,
                             cudaStream_t s);

@@ -4,11 +4,19 @@
 
 #include "sw_internal.h"
 
+// Work vectors of one right-hand side on one level of a solve.
+struct LevelWs {
+  double2 *rhs = nullptr, *sol = nullptr, *gr = nullptr, *gtmp = nullptr;
+  std::vector<double2*> gp, gq;
+  double2 *kx1 = nullptr, *kr1 = nullptr, *kq = nullptr, *ke = nullptr, *kx3 = nullptr;
+  double2* tmp = nullptr;  // scratch of the fine operator (level 0)
+};
+
 // One level of the hierarchy.  Level 0 is the fine lattice (dof = site,
 // parity-split order); level l > 0 is a coarse lattice E0 x E1 with nc dof per
 // site (dof = X * nc + k).  b0, b1, nv and P describe the transfer from this
 // level to level l + 1.
-struct MgLevel {
+struct MgLevel : LevelWs {  // the work vectors are those of single solves
   int E0 = 0, E1 = 0, nc = 1;
   long ndof = 0;
   int b0 = 0, b1 = 0, nv = 0;
@@ -19,23 +27,8 @@ struct MgLevel {
   float4* Ydf = nullptr;  // mixed precision, coarsest level: double-float stencil
   float4* cdf = nullptr;  // [2][ndof] double-float copies of r and p for its CGNE
   DigitStencil dg;        // digit entries of Y: coarsest level, and every level of an FP64 hierarchy
-  // setup work vectors
-  double2 *sr = nullptr, *sp = nullptr, *sq = nullptr, *st = nullptr;
-  // solve work vectors
-  double2 *rhs = nullptr, *sol = nullptr, *gr = nullptr, *gtmp = nullptr;
-  double2 *cp = nullptr, *cw = nullptr;
-  std::vector<double2*> gp, gq;
-  double2 *kx1 = nullptr, *kr1 = nullptr, *kq = nullptr, *ke = nullptr, *kr2 = nullptr;
-  double2 *kx3 = nullptr, *kr3 = nullptr;
+  double2 *cp = nullptr, *cw = nullptr;  // of the host-queued CGNE loop
   double2* stmp = nullptr;  // [N] scratch of the fine operators (level 0)
-};
-
-// Work vectors of one right-hand side on one level in a batched solve.
-struct LevelWs {
-  double2 *rhs = nullptr, *sol = nullptr, *gr = nullptr, *gtmp = nullptr;
-  std::vector<double2*> gp, gq;
-  double2 *kx1 = nullptr, *kr1 = nullptr, *kq = nullptr, *ke = nullptr, *kr2 = nullptr;
-  double2 *kx3 = nullptr;
 };
 
 // Workspace of batched solves (allocated on the first one).
@@ -69,14 +62,11 @@ struct sw_mg {
   bool mixed = false;            // params.precision == SW_MG_MIXED
   bool fine_D = false;           // params.fine_operator == SW_MG_COARSEN_D
   float2* binv32 = nullptr;      // FP32 B^-1 (mixed)
-  float2* s32tmp = nullptr;      // [N] FP32 scratch of the FP32 Schur operator
   std::vector<MgLevel> lev;
   std::vector<double2*> allocs;
   double2 *bps = nullptr, *xps = nullptr, *lexb = nullptr, *lexx = nullptr, *lext = nullptr;
   std::vector<int> setup_iters;
   BatchWs batch;
-  long long st_fine_applies = 0, st_inter_iters = 0, st_inter_solves = 0;
-  long long st_coarsest_iters = 0, st_coarsest_solves = 0;
 };
 
 // Device scalar slots owned by level l: [64 l, 64 l + 64).
