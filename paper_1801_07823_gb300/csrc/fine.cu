@@ -6,8 +6,8 @@
 // Links are stored pre-multiplied as W_mu(s) = eta_mu(s) U_mu(s) / 2.  In 2D
 // eta_mu(s - mu) = eta_mu(s) (eta_1 depends on x0 only), so the backward hop of
 // Eq. staggeredD is -conj(W_mu(s - mu)) x(s - mu).
+#include "intmul.cuh"
 #include "many.h"
-#include "sw_internal.h"
 
 namespace {
 
@@ -19,6 +19,11 @@ __device__ __forceinline__ void cfma(double2& acc, double2 a, double2 b) {  // a
   acc.x = fma(-a.y, b.y, acc.x);
   acc.y = fma(a.x, b.y, acc.y);
   acc.y = fma(a.y, b.x, acc.y);
+}
+__device__ __forceinline__ double2 minus_conj(double2 w) { return make_double2(-w.x, w.y); }
+__device__ __forceinline__ bool all_zero(double2 a, double2 b, double2 c, double2 d) {
+  return a.x == 0.0 && a.y == 0.0 && b.x == 0.0 && b.y == 0.0 && c.x == 0.0 && c.y == 0.0 &&
+         d.x == 0.0 && d.y == 0.0;
 }
 __device__ __forceinline__ void cfmac(double2& acc, double2 a, double2 b) {  // acc += conj(a) b
   acc.x = fma(a.x, b.x, acc.x);
@@ -32,29 +37,33 @@ __device__ __forceinline__ void cfmac(double2& acc, double2 a, double2 b) {  // 
 // sg = +1 for D, -1 for D^dag (D - m is anti-Hermitian, Sec. II).
 // One thread per site; consecutive threads take consecutive x0, so every
 // load of in and W is coalesced; neighbour values are re-read from L1/L2.
-// In FP64 the kernel is bound by the FP64 pipe (two FMAs per clock and SM), so
-// the sum starts from m in(s) and the sign is an operand's: 18 FP64 operations
-// per site, where a separate sum and a final m x + sg h took 20 (2044 x 2052:
-// 149.6 -> 132.8 us).  In FP32 it is bound by HBM.
+template <typename C2>
+struct Hops {  // a site's neighbours and their links
+  C2 xs, a, b, c, d, w0, w1, w0m, w1m;
+  long s;
+};
+template <typename C2>
+__device__ __forceinline__ Hops<C2> load_hops(const C2* __restrict__ in, const C2* __restrict__ W,
+                                              int x0, int x1, int L0, int L1) {
+  const long N = (long)L0 * L1, row = (long)x1 * L0;
+  const long sm0 = row + (x0 == 0 ? L0 - 1 : x0 - 1);
+  const long sm1 = (long)(x1 == 0 ? L1 - 1 : x1 - 1) * L0 + x0;
+  Hops<C2> h;
+  h.s = row + x0;
+  h.xs = __ldg(in + h.s);
+  h.a = __ldg(in + row + (x0 + 1 == L0 ? 0 : x0 + 1));
+  h.b = __ldg(in + sm0);
+  h.c = __ldg(in + (long)(x1 + 1 == L1 ? 0 : x1 + 1) * L0 + x0);
+  h.d = __ldg(in + sm1);
+  h.w0 = __ldg(W + h.s);
+  h.w1 = __ldg(W + N + h.s);
+  h.w0m = __ldg(W + sm0);
+  h.w1m = __ldg(W + N + sm1);
+  return h;
+}
 template <typename C2, typename R, bool DAG>
-__global__ void __launch_bounds__(256) k_dslash_lex(const C2* __restrict__ in, C2* __restrict__ out,
-                                                    const C2* __restrict__ W, R mass, int L0,
-                                                    int L1) {
-  int x0 = blockIdx.x * blockDim.x + threadIdx.x;
-  int x1 = blockIdx.y;
-  if (x0 >= L0) return;
-  long N = (long)L0 * L1;
-  long row = (long)x1 * L0;
-  long s = row + x0;
-  long sp0 = row + (x0 + 1 == L0 ? 0 : x0 + 1);
-  long sm0 = row + (x0 == 0 ? L0 - 1 : x0 - 1);
-  long sp1 = (long)(x1 + 1 == L1 ? 0 : x1 + 1) * L0 + x0;
-  long sm1 = (long)(x1 == 0 ? L1 - 1 : x1 - 1) * L0 + x0;
-  C2 xs = __ldg(in + s);
-  C2 a = __ldg(in + sp0), b = __ldg(in + sm0), c = __ldg(in + sp1), d = __ldg(in + sm1);
-  C2 w0 = __ldg(W + s), w1 = __ldg(W + N + s);
-  C2 w0m = __ldg(W + sm0), w1m = __ldg(W + N + sm1);
-  R hx = mass * xs.x, hy = mass * xs.y;
+__device__ __forceinline__ C2 sum_hops(const Hops<C2>& h, R mass) {
+  R hx = mass * h.xs.x, hy = mass * h.xs.y;
   auto fwd = [&](C2 w, C2 v) {  // +- w v
     if (DAG) { w.x = -w.x; w.y = -w.y; }
     hx = fma(w.x, v.x, hx); hx = fma(-w.y, v.y, hx);
@@ -65,14 +74,60 @@ __global__ void __launch_bounds__(256) k_dslash_lex(const C2* __restrict__ in, C
     hx = fma(-w.x, v.x, hx); hx = fma(-w.y, v.y, hx);
     hy = fma(-w.x, v.y, hy); hy = fma(w.y, v.x, hy);
   };
-  fwd(w0, a);
-  fwd(w1, c);
-  bwd(w0m, b);
-  bwd(w1m, d);
+  fwd(h.w0, h.a);
+  fwd(h.w1, h.c);
+  bwd(h.w0m, h.b);
+  bwd(h.w1m, h.d);
   C2 o;
   o.x = hx;
   o.y = hy;
-  out[s] = o;
+  return o;
+}
+// FP32: bound by HBM.
+template <bool DAG>
+__global__ void __launch_bounds__(256) k_dslash_lex32(const float2* __restrict__ in,
+                                                      float2* __restrict__ out,
+                                                      const float2* __restrict__ W, float mass,
+                                                      int L0, int L1) {
+  const int x0 = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x0 >= L0) return;
+  const Hops<float2> h = load_hops(in, W, x0, blockIdx.y, L0, L1);
+  out[h.s] = sum_hops<float2, float, DAG>(h, mass);
+}
+// FP64: of the eight warps of a CTA two belong to each quarter of the SM; one of the two
+// works in FP64 (18 operations per site, two per clock and SM) and the other forms its hops in
+// integers (intmul.cuh) with one FMA per component for the mass term, so that both
+// pipes are busy.  The warps change places from row to row, for lattices that fill half a
+// CTA.  2044 x 2052, of 39.6 us at the HBM rate: all in FP64 132.2 us, all in integers 114.9
+// (about 350 integer operations per site, 64 per clock and SM), split 88.1.  32 x 32 is one
+// launch either way (6.5 us).  Relative error 1.3e-16 against 1.5e-16 in FP64 alone.
+template <bool DAG>
+__global__ void __launch_bounds__(256) k_dslash_lex(const double2* __restrict__ in,
+                                                    double2* __restrict__ out,
+                                                    const double2* __restrict__ W, double mass,
+                                                    int L0, int L1) {
+  using namespace swint;
+  const int x0 = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x0 >= L0) return;
+  const Hops<double2> h = load_hops(in, W, x0, blockIdx.y, L0, L1);
+  const unsigned mv = max(max(magnitude(h.a), magnitude(h.b)), max(magnitude(h.c), magnitude(h.d)));
+  const unsigned mw =
+      max(max(magnitude(h.w0), magnitude(h.w1)), max(magnitude(h.w0m), magnitude(h.w1m)));
+  const int e = (int)(mv >> 20);
+  const bool ints = (((threadIdx.x >> 7) ^ blockIdx.y) & 1) && link_usable(mw);
+  if (ints && usable(e)) {
+    Csum t;
+    t.add(num(h.w0, kLinkExp), num(h.a, e));
+    t.add(num(h.w1, kLinkExp), num(h.c, e));
+    t.add(num(minus_conj(h.w0m), kLinkExp), num(h.b, e));
+    t.add(num(minus_conj(h.w1m), kLinkExp), num(h.d, e));
+    const double2 v = t.value(kLinkExp, e);
+    out[h.s] = make_double2(fma(mass, h.xs.x, DAG ? -v.x : v.x), fma(mass, h.xs.y, DAG ? -v.y : v.y));
+  } else if (ints && mv == 0 && all_zero(h.a, h.b, h.c, h.d)) {
+    out[h.s] = make_double2(mass * h.xs.x, mass * h.xs.y);  // a sparse source
+  } else {
+    out[h.s] = sum_hops<double2, double, DAG>(h, mass);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -499,14 +554,14 @@ void launch_dslash_ps(const sw_gauge* g, double mass, int dagger, const double2*
 void launch_dslash_lex(const sw_gauge* g, double mass, int dagger, const double2* in, double2* out,
                        cudaStream_t s) {
   dim3 grid(nblocks(g->L0, 256), g->L1);
-  auto k = dagger ? k_dslash_lex<double2, double, true> : k_dslash_lex<double2, double, false>;
+  auto k = dagger ? k_dslash_lex<true> : k_dslash_lex<false>;
   k<<<grid, 256, 0, s>>>(in, out, g->W_lex, mass, g->L0, g->L1);
   SW_LAUNCH_CHECK();
 }
 void launch_dslash_lex32(const sw_gauge* g, float mass, int dagger, const float2* in, float2* out,
                          cudaStream_t s) {
   dim3 grid(nblocks(g->L0, 256), g->L1);
-  auto k = dagger ? k_dslash_lex<float2, float, true> : k_dslash_lex<float2, float, false>;
+  auto k = dagger ? k_dslash_lex32<true> : k_dslash_lex32<false>;
   k<<<grid, 256, 0, s>>>(in, out, g->W_lex32, mass, g->L0, g->L1);
   SW_LAUNCH_CHECK();
 }
