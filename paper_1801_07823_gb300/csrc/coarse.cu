@@ -158,8 +158,9 @@ __global__ void __launch_bounds__(128) k_restrict_fine(const double2* __restrict
                                                        Pack<2, W> io, int L0, int L1,
                                                        int a0, int a1, int nv, int groups,
                                                        int full) {
-  const double2* __restrict__ r = io.v[0][blockIdx.y];
-  double2* __restrict__ out = io.v[1][blockIdx.y];
+  const double2* r = io.v[0][blockIdx.y];
+  double2* out = io.v[1][blockIdx.y];
+  after_previous();
   __shared__ double2 part[2 * 128];
   const int A = blockIdx.x, E0 = L0 / (2 * a0);
   const int A0 = A % E0, A1 = A / E0;
@@ -220,7 +221,7 @@ __device__ __forceinline__ void coarse_dof_map(long dof, int E0, int nc, int b0,
 // sum_i p[i] e[i] as four chains of FMAs (a dependent FP64 operation waits 64 clocks:
 // one chain of 2 x 24 takes 1.6 us, these 0.5).
 __device__ __forceinline__ double2 row_times(const double2* __restrict__ p,
-                                             const double2* __restrict__ e, int n) {
+                                             const double2* e, int n) {
   double2 s[4] = {};
   int i = 0;
   for (; i + 1 < n; i += 2)
@@ -241,8 +242,9 @@ __device__ __forceinline__ double2 row_times(const double2* __restrict__ p,
 template <bool LEX, int W>
 __global__ void k_prolong_fine(const double2* __restrict__ P, Pack<2, W> io, int L0, int L1, int a0,
                                int a1, int nv, int full) {
-  const double2* __restrict__ ehat = io.v[0][blockIdx.y];
-  double2* __restrict__ e = io.v[1][blockIdx.y];
+  const double2* ehat = io.v[0][blockIdx.y];
+  double2* e = io.v[1][blockIdx.y];
+  after_previous();
   int N = L0 * L1;
   int h = blockIdx.x * blockDim.x + threadIdx.x;
   if (h >= (full || LEX ? N : N / 2)) return;
@@ -296,8 +298,9 @@ __global__ void __launch_bounds__(kRestrictThreads) k_restrict_coarse(const doub
                                                                       int b1, int nc, int nv,
                                                                       int groups) {
   __shared__ double2 part[kRestrictThreads];
-  const double2* __restrict__ r = io.v[0][blockIdx.y];
-  double2* __restrict__ out = io.v[1][blockIdx.y];
+  const double2* r = io.v[0][blockIdx.y];
+  double2* out = io.v[1][blockIdx.y];
+  after_previous();
   const int A = blockIdx.x, F0 = E0 / b0, A0 = A % F0, A1 = A / F0;
   const int grp = threadIdx.x / (2 * nv), t = threadIdx.x - grp * 2 * nv;
   const int c = t / nv, i = t - c * nv, hn = nc / 2;
@@ -324,8 +327,9 @@ __global__ void __launch_bounds__(kRestrictThreads) k_restrict_coarse(const doub
 template <int W>
 __global__ void k_prolong_coarse(const double2* __restrict__ P, Pack<2, W> io, int E0, int E1,
                                  int b0, int b1, int nc, int nv) {
-  const double2* __restrict__ ehat = io.v[0][blockIdx.y];
-  double2* __restrict__ e = io.v[1][blockIdx.y];
+  const double2* ehat = io.v[0][blockIdx.y];
+  double2* e = io.v[1][blockIdx.y];
+  after_previous();
   long dof = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (dof >= (long)E0 * E1 * nc) return;
   int A, c;
@@ -684,8 +688,7 @@ void many_restrict_fine(const sw_gauge* g, int a0, int a1, int nv, const double2
   with_width(io.n, [&](auto w) {
     constexpr int W = decltype(w)::value;
     auto k = lex ? k_restrict_fine<true, W> : k_restrict_fine<false, W>;
-    k<<<dim3(nagg, io.n), 128, 0, s>>>(P, Pack<2, W>(io), g->L0, g->L1, a0, a1, nv, groups, full);
-    SW_LAUNCH_CHECK();
+    launch_early(k, dim3(nagg, io.n), 128, 0, s, P, Pack<2, W>(io), g->L0, g->L1, a0, a1, nv, groups, full);
   });
 }
 void many_prolong_fine(const sw_gauge* g, int a0, int a1, int nv, const double2* P,
@@ -693,9 +696,8 @@ void many_prolong_fine(const sw_gauge* g, int a0, int a1, int nv, const double2*
   with_width(io.n, [&](auto w) {
     constexpr int W = decltype(w)::value;
     auto k = lex ? k_prolong_fine<true, W> : k_prolong_fine<false, W>;
-    k<<<dim3(cdiv(full || lex ? g->N : g->N / 2, 128), io.n), 128, 0, s>>>(
-        P, Pack<2, W>(io), g->L0, g->L1, a0, a1, nv, full);
-    SW_LAUNCH_CHECK();
+    launch_early(k, dim3(cdiv(full || lex ? g->N : g->N / 2, 128), io.n), 128, 0, s,
+                 P, Pack<2, W>(io), g->L0, g->L1, a0, a1, nv, full);
   });
 }
 void many_restrict_coarse(const CoarseGeom& g, int b0, int b1, int nv, const double2* P,
@@ -704,9 +706,8 @@ void many_restrict_coarse(const CoarseGeom& g, int b0, int b1, int nv, const dou
   const int groups = kRestrictThreads / (2 * nv) < dofs ? kRestrictThreads / (2 * nv) : dofs;
   with_width(io.n, [&](auto w) {
     constexpr int W = decltype(w)::value;
-    k_restrict_coarse<W><<<dim3(nagg, io.n), kRestrictThreads, 0, s>>>(
-        P, Pack<2, W>(io), g.E0, b0, b1, g.nc, nv, groups);
-    SW_LAUNCH_CHECK();
+    launch_early(k_restrict_coarse<W>, dim3(nagg, io.n), kRestrictThreads, 0, s,
+                 P, Pack<2, W>(io), g.E0, b0, b1, g.nc, nv, groups);
   });
 }
 void many_prolong_coarse(const CoarseGeom& g, int b0, int b1, int nv, const double2* P,
@@ -714,9 +715,8 @@ void many_prolong_coarse(const CoarseGeom& g, int b0, int b1, int nv, const doub
   long n = (long)g.E0 * g.E1 * g.nc;
   with_width(io.n, [&](auto w) {
     constexpr int W = decltype(w)::value;
-    k_prolong_coarse<W><<<dim3(cdiv(n, 128), io.n), 128, 0, s>>>(P, Pack<2, W>(io), g.E0, g.E1, b0,
+    launch_early(k_prolong_coarse<W>, dim3(cdiv(n, 128), io.n), 128, 0, s, P, Pack<2, W>(io), g.E0, g.E1, b0,
                                                                  b1, g.nc, nv);
-    SW_LAUNCH_CHECK();
   });
 }
 void launch_build_W(const sw_gauge* g, int nv, const double2* binv, const double2* P,

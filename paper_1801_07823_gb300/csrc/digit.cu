@@ -58,15 +58,13 @@ __global__ void __launch_bounds__(kNT, kCtas) k_digit_apply(Shape s, const uint4
                                                             const int* __restrict__ ex,
                                                             const double2* __restrict__ Y,
                                                             Pack<2, W> io, int parts,
-                                                            const int* __restrict__ skip,
+                                                            const int* skip,
                                                             unsigned long long* exec) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int em;
   __shared__ Super sup[2][kSupers];  // of this unit and the next
-  const double2* __restrict__ in = io.v[0][blockIdx.y];
-  double2* __restrict__ out = io.v[1][blockIdx.y];
-  if (skip && skip[4 * blockIdx.y]) return;
-  if (exec && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(exec, 1ull);
+  const double2* in = io.v[0][blockIdx.y];
+  double2* out = io.v[1][blockIdx.y];
   unsigned char* B = smem;
   int4* quads = reinterpret_cast<int4*>(smem + (size_t)s.KS * 4 * kQuadBytes);
   int* S = reinterpret_cast<int*>(quads + 2 * s.KS);
@@ -100,7 +98,10 @@ __global__ void __launch_bounds__(kNT, kCtas) k_digit_apply(Shape s, const uint4
     prefetch(s, run, f, n, w);
   };
   int u = blockIdx.x;
-  if (u < nunits) enter(u);
+  if (u < nunits) enter(u);  // tables and first entries: constant, asked for before the wait
+  after_previous();
+  if (skip && skip[4 * blockIdx.y]) return;
+  if (exec && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(exec, 1ull);
   while (u < nunits) {
     if (threadIdx.x == 0) em = -kNotFinite;
     double2 x[kPer];
@@ -197,8 +198,7 @@ void many_digit(const CoarseGeom& g, const DigitStencil& t, const double2* Y, in
         SW_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     }
     auto k = dagger ? k_digit_apply<true, W> : k_digit_apply<false, W>;
-    k<<<grid, kNT, smem, st>>>(s, t.T, t.ex, Y, Pack<2, W>(io), parts, ctl, exec);
-    SW_LAUNCH_CHECK();
+    launch_early(k, grid, kNT, smem, st, s, t.T, t.ex, Y, Pack<2, W>(io), parts, ctl, exec);
   });
 }
 void launch_digit_apply(const CoarseGeom& g, const DigitStencil& t, const double2* Y, int dagger,

@@ -214,10 +214,11 @@ __global__ void k_binv_build(const double2* __restrict__ Wps, double mass, doubl
 // out = M in (or M^dag in) on nblk KD blocks; one member of a batch per blockIdx.y.
 template <int W>
 __global__ void k_block_apply(const double2* __restrict__ M, Pack<2, W> io, int nblk, int dagger,
-                              const int* __restrict__ ctl) {
+                              const int* ctl) {
+  after_previous();
   if (ctl && ctl[4 * blockIdx.y]) return;
-  const double2* __restrict__ in = io.v[0][blockIdx.y];
-  double2* __restrict__ out = io.v[1][blockIdx.y];
+  const double2* in = io.v[0][blockIdx.y];
+  double2* out = io.v[1][blockIdx.y];
   int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= nblk) return;
   double2 v[4];
@@ -236,7 +237,7 @@ __global__ void k_block_apply(const double2* __restrict__ M, Pack<2, W> io, int 
 // (C in)(s) for a site s of parity half par: the two hops of s that leave its
 // KD block.  in is the opposite parity half.
 __device__ __forceinline__ double2 hop_out(const double2* __restrict__ Wps,
-                                           const double2* __restrict__ in, int f, int L0, int L1,
+                                           const double2* in, int f, int L0, int L1,
                                            int N) {
   int x0, x1;
   ps_coords(f, L0, N, x0, x1);
@@ -271,7 +272,8 @@ __device__ __forceinline__ double2 hop_out(const double2* __restrict__ Wps,
 // full vectors; operands (src or null, in, out) of one member of a batch per blockIdx.y.
 template <int W>
 __global__ void k_hop(const double2* __restrict__ Wps, int par, double sign, Pack<3, W> io, int L0,
-                      int L1, const int* __restrict__ ctl) {
+                      int L1, const int* ctl) {
+  after_previous();
   if (ctl && ctl[4 * blockIdx.y]) return;
   const double2* src = io.v[0][blockIdx.y];
   const double2* in = io.v[1][blockIdx.y];
@@ -291,7 +293,8 @@ __global__ void k_hop(const double2* __restrict__ Wps, int par, double sign, Pac
 template <int W>
 __global__ void k_hop_block(const double2* __restrict__ Wps, const double2* __restrict__ M,
                             int par, int dagger, double sign, Pack<3, W> io, int L0, int L1,
-                            const int* __restrict__ ctl) {
+                            const int* ctl) {
+  after_previous();
   if (ctl && ctl[4 * blockIdx.y]) return;
   const double2* src = io.v[0][blockIdx.y];
   const double2* in = io.v[1][blockIdx.y];
@@ -583,26 +586,25 @@ void many_block_apply(const sw_gauge* g, const double2* binv, int par, int dagge
                       const Many<2>& io, cudaStream_t s, const int* ctl) {
   const int half = g->N / 8, nblk = par < 0 ? 2 * half : half;
   with_width(io.n, [&](auto w) {
-    k_block_apply<decltype(w)::value><<<dim3(nblocks(nblk, 128), io.n), 128, 0, s>>>(
-        binv + (par > 0 ? (long)half * 16 : 0), Pack<2, decltype(w)::value>(io), nblk, dagger, ctl);
-    SW_LAUNCH_CHECK();
+    constexpr int W = decltype(w)::value;
+    launch_early(k_block_apply<W>, dim3(nblocks(nblk, 128), io.n), 128, 0, s,
+                 binv + (par > 0 ? (long)half * 16 : 0), Pack<2, W>(io), nblk, dagger, ctl);
   });
 }
 void many_hop(const sw_gauge* g, int par, double sign, const Many<3>& io, cudaStream_t s,
               const int* ctl) {
   with_width(io.n, [&](auto w) {
-    k_hop<decltype(w)::value><<<dim3(nblocks(par < 0 ? g->N : g->N / 2, 256), io.n), 256, 0, s>>>(
-        g->W_ps, par, sign, Pack<3, decltype(w)::value>(io), g->L0, g->L1, ctl);
-    SW_LAUNCH_CHECK();
+    constexpr int W = decltype(w)::value;
+    launch_early(k_hop<W>, dim3(nblocks(par < 0 ? g->N : g->N / 2, 256), io.n), 256, 0, s, g->W_ps,
+                 par, sign, Pack<3, W>(io), g->L0, g->L1, ctl);
   });
 }
 void many_hop_block(const sw_gauge* g, const double2* binv, int par, int dagger, double sign,
                     const Many<3>& io, cudaStream_t s, const int* ctl) {
   with_width(io.n, [&](auto w) {
-    k_hop_block<decltype(w)::value>
-        <<<dim3(nblocks(par < 0 ? g->N / 4 : g->N / 8, 128), io.n), 128, 0, s>>>(
-            g->W_ps, binv, par, dagger, sign, Pack<3, decltype(w)::value>(io), g->L0, g->L1, ctl);
-    SW_LAUNCH_CHECK();
+    constexpr int W = decltype(w)::value;
+    launch_early(k_hop_block<W>, dim3(nblocks(par < 0 ? g->N / 4 : g->N / 8, 128), io.n), 128, 0, s,
+                 g->W_ps, binv, par, dagger, sign, Pack<3, W>(io), g->L0, g->L1, ctl);
   });
 }
 void launch_block_apply(const sw_gauge* g, const double2* binv, int par, int dagger,

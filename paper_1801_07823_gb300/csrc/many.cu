@@ -310,6 +310,7 @@ __global__ void __launch_bounds__(kThreads) k_many(Op op, Pack<Op::K, W> v, long
                                                    double* host, int* ctl) {
   __shared__ double cf[2];
   const int m = blockIdx.y;
+  after_previous();
   if (ctl) {
     ctl += 4 * m;
     // a kernel that sets the flag does so in its last CTA, after all of them have read it
@@ -380,9 +381,8 @@ void launch(sw_ctx* c, long n, const Op& op, const Many<Op::K>& v, double* host 
   if (Op::R > 0 && grid > kManyBlocks) grid = kManyBlocks;
   with_width(v.n, [&](auto w) {
     constexpr int W = decltype(w)::value;
-    k_many<Op, W><<<dim3((unsigned)grid, v.n), kThreads, 0, c->stream>>>(
-        op, Pack<Op::K, W>(v), n, c->slots, c->many_partials, c->many_counters, host, ctl);
-    SW_LAUNCH_CHECK();
+    launch_early(k_many<Op, W>, dim3((unsigned)grid, v.n), kThreads, 0, c->stream, op,
+                 Pack<Op::K, W>(v), n, c->slots, c->many_partials, c->many_counters, host, ctl);
   });
 }
 

@@ -47,8 +47,9 @@ __global__ void k_to_f32(const double2* __restrict__ in, float2* __restrict__ ou
 // out (float) = M in (double -> float), M per KD block of one parity half
 template <int W>
 __global__ void k_block_apply_df(const float2* __restrict__ M, Pack<2, W> io, int nblk) {
-  const double2* __restrict__ in = io.v[0][blockIdx.y];
-  float2* __restrict__ out = (float2*)io.v[1][blockIdx.y];
+  const double2* in = io.v[0][blockIdx.y];
+  float2* out = (float2*)io.v[1][blockIdx.y];
+  after_previous();
   int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= nblk) return;
   float2 v[4];
@@ -62,7 +63,7 @@ __global__ void k_block_apply_df(const float2* __restrict__ M, Pack<2, W> io, in
 }
 
 // (C in)(s) for site f of its parity half; in = opposite half (float)
-__device__ __forceinline__ float2 hop_out_f(const float2* __restrict__ W, const float2* __restrict__ in,
+__device__ __forceinline__ float2 hop_out_f(const float2* __restrict__ W, const float2* in,
                                            int f, int L0, int L1, int N) {
   int x0, x1;
   ps_coords(f, L0, N, x0, x1);
@@ -93,8 +94,9 @@ __device__ __forceinline__ float2 hop_out_f(const float2* __restrict__ W, const 
 template <int WIDTH>
 __global__ void k_hop_block_ff(const float2* __restrict__ W, const float2* __restrict__ M, int par,
                                Pack<2, WIDTH> io, int L0, int L1) {
-  const float2* __restrict__ in = (const float2*)io.v[0][blockIdx.y];
-  float2* __restrict__ out = (float2*)io.v[1][blockIdx.y];
+  const float2* in = (const float2*)io.v[0][blockIdx.y];
+  float2* out = (float2*)io.v[1][blockIdx.y];
+  after_previous();
   int N = L0 * L1, half = N >> 1;
   int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= (half >> 2)) return;
@@ -112,9 +114,10 @@ __global__ void k_hop_block_ff(const float2* __restrict__ W, const float2* __res
 template <int WIDTH>
 __global__ void k_hop_sub_fd(const float2* __restrict__ W, int par, Pack<3, WIDTH> io, int L0,
                              int L1) {
-  const double2* __restrict__ src = io.v[0][blockIdx.y];
-  const float2* __restrict__ in = (const float2*)io.v[1][blockIdx.y];
-  double2* __restrict__ out = io.v[2][blockIdx.y];
+  const double2* src = io.v[0][blockIdx.y];
+  const float2* in = (const float2*)io.v[1][blockIdx.y];
+  double2* out = io.v[2][blockIdx.y];
+  after_previous();
   int N = L0 * L1, half = N >> 1;
   int h = blockIdx.x * blockDim.x + threadIdx.x;
   if (h >= half) return;
@@ -162,8 +165,9 @@ template <int NC, bool DAG, int W>
 __global__ void __launch_bounds__(5 * NC) k_coarse_apply_h(const __half2* __restrict__ Yh,
                                                            const float* __restrict__ scale,
                                                            Pack<2, W> io, int E0, int E1, int rs) {
-  const double2* __restrict__ in = io.v[0][blockIdx.y];
-  double2* __restrict__ out = io.v[1][blockIdx.y];
+  const double2* in = io.v[0][blockIdx.y];
+  double2* out = io.v[1][blockIdx.y];
+  after_previous();
   __shared__ float2 xs[5][NC];
   __shared__ float2 part[5][NC];
   int rows = NC / rs;
@@ -209,8 +213,9 @@ __global__ void __launch_bounds__(5 * NC) k_coarse_apply_h(const __half2* __rest
 template <bool DAG, int W>
 __global__ void k_coarse_apply_h_any(const __half2* __restrict__ Yh, const float* __restrict__ scale,
                                      Pack<2, W> io, int E0, int E1, int nc) {
-  const double2* __restrict__ in = io.v[0][blockIdx.y];
-  double2* __restrict__ out = io.v[1][blockIdx.y];
+  const double2* in = io.v[0][blockIdx.y];
+  double2* out = io.v[1][blockIdx.y];
+  after_previous();
   long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (long)E0 * E1 * nc) return;
   int X = (int)(e / nc), i = (int)(e - (long)X * nc);
@@ -251,8 +256,8 @@ void apply_h_nc(const CoarseGeom& g, const __half2* Yh, const float* sc, int dag
   with_width(io.n, [&](auto w) {
     constexpr int W = decltype(w)::value;
     auto k = dagger ? k_coarse_apply_h<NC, true, W> : k_coarse_apply_h<NC, false, W>;
-    k<<<dim3(nsites * rs, io.n), 5 * (NC / rs), 0, s>>>(Yh, sc, Pack<2, W>(io), g.E0, g.E1, rs);
-    SW_LAUNCH_CHECK();
+    launch_early(k, dim3(nsites * rs, io.n), 5 * (NC / rs), 0, s, Yh, sc, Pack<2, W>(io), g.E0, g.E1,
+                 rs);
   });
 }
 
@@ -278,14 +283,11 @@ void many_S32(const sw_gauge* g, const float2* W32, const float2* binv32, const 
   with_width(v.n, [&](auto w) {
     constexpr int W = decltype(w)::value;
     const dim3 blocks(cdiv(nblk, 128), v.n);
-    k_block_apply_df<W><<<blocks, 128, 0, s>>>(binv32, Pack<2, W>(in_t), nblk);
-    SW_LAUNCH_CHECK();
-    k_hop_block_ff<W><<<blocks, 128, 0, s>>>(W32, binv32 + (long)nblk * 16, 1, Pack<2, W>(t_v),
-                                             g->L0, g->L1);
-    SW_LAUNCH_CHECK();
-    k_hop_sub_fd<W><<<dim3(cdiv(half, 256), v.n), 256, 0, s>>>(W32, 0, Pack<3, W>(last), g->L0,
-                                                               g->L1);
-    SW_LAUNCH_CHECK();
+    launch_early(k_block_apply_df<W>, blocks, 128, 0, s, binv32, Pack<2, W>(in_t), nblk);
+    launch_early(k_hop_block_ff<W>, blocks, 128, 0, s, W32, binv32 + (long)nblk * 16, 1,
+                 Pack<2, W>(t_v), g->L0, g->L1);
+    launch_early(k_hop_sub_fd<W>, dim3(cdiv(half, 256), v.n), 256, 0, s, W32, 0, Pack<3, W>(last),
+                 g->L0, g->L1);
   });
 }
 
@@ -309,8 +311,7 @@ void many_coarse_h(const CoarseGeom& g, const __half2* Yh, const float* scale, i
   with_width(io.n, [&](auto w) {
     constexpr int W = decltype(w)::value;
     auto k = dagger ? k_coarse_apply_h_any<true, W> : k_coarse_apply_h_any<false, W>;
-    k<<<dim3(cdiv(n, 128), io.n), 128, 0, s>>>(Yh, scale, Pack<2, W>(io), g.E0, g.E1, g.nc);
-    SW_LAUNCH_CHECK();
+    launch_early(k, dim3(cdiv(n, 128), io.n), 128, 0, s, Yh, scale, Pack<2, W>(io), g.E0, g.E1, g.nc);
   });
 }
 void launch_coarse_apply_h(const CoarseGeom& g, const __half2* Yh, const float* scale, int dagger,

@@ -6,6 +6,7 @@
 #include <exception>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/sw.h"
@@ -29,6 +30,37 @@ void sw_count_launch();
     sw_count_launch();            \
     SW_CUDA(cudaGetLastError());  \
   } while (0)
+// Launch of a kernel that begins with after_previous(): its CTAs may be placed while the
+// stream's previous kernel still runs, as soon as all CTAs of that one have begun their
+// work, so that the launch is hidden.  The K-cycle of a small lattice is a chain of kernels
+// of 2 to 5 us with about 2 us between them: solve at 64^2 36.9 -> 33.5 ms, setup and solve
+// there 28.0 -> 23.0, mixed solve at 128^2 36.8 -> 35.6, 16 right-hand sides at 128^2
+// 76.5 -> 75.1.
+template <typename... P, typename... A>
+void launch_early(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s,
+                  A&&... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  SW_CUDA(cudaLaunchKernelEx(&cfg, kernel, P(std::forward<A>(args))...));
+  SW_LAUNCH_CHECK();
+}
+#ifdef __CUDACC__
+// Waits until the previous kernel has finished and its writes are visible, then lets the next
+// one be placed.  Every thread calls it, before it touches memory that any kernel of the
+// stream writes; such memory is not read through pointers that promise it constant.
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
 // Debug aid: with the environment variable SW_POISON=1 every device buffer the
 // library allocates is filled with all-one bytes (NaN in every double and
 // float), so that a kernel reading memory nothing has written produces NaN.
