@@ -29,6 +29,13 @@
 // update, and in the norm with its fence, and 1 us in the barrier; at 4^2 x 24
 // that fixed part is all.
 //
+// Where it is all, the cluster form is faster: up to 16 CTAs of one cluster, the
+// cluster's hardware barrier instead of arrivals counted in the L2, norm parts in
+// every CTA's shared memory.  With more than six items per CTA (kClusterItems) the
+// products on a tenth of the SMs take longer than that saves.  It needs 16 SMs in one
+// GPC, so a context that shares the SMs with others keeps the grid form.
+// Solve at 64^2 with Nv 8/12 (4^2 x 24): 35.2 -> 32.3 ms.
+//
 // The fraction l2frac of the entries' lines, sized on the host to what the L2
 // can keep, is loaded with evict-last priority and the rest evict-first.
 //
@@ -54,6 +61,8 @@ constexpr int kMaxPairs = 1024;      // (row, component) pairs per chunk
 constexpr int kMaxSites = 56;        // sites per chunk
 constexpr int kMaxSupers = 128;      // supers per chunk
 constexpr int kMaxBytes = 176 * 1024;  // shared memory of a chunk
+constexpr int kCluster = 16;         // CTAs of the cluster form, at most
+constexpr int kClusterItems = 6 * kCluster;  // its largest problem
 
 struct Args {
   Shape s;
@@ -123,6 +132,7 @@ struct Shared {
   int f0[kWarps], n[kWarps];     // the warps' shares of the k-steps
   int em[2][kMaxSites];
   double rr, stop2, coef;
+  double parts[2][kCluster];     // norm parts of the cluster form
   int nsup, state;  // state 0: continue, 1: converged / cap, 2: non-finite
   int ok;
 };
@@ -228,18 +238,20 @@ __device__ __forceinline__ void bar_arrive(int id, int threads) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
-// Sum of the previous phase's partials, in the same order in every CTA, and
-// the scalar the phase needs (one warp).
+// Sum of the previous phase's partials (in global memory, or in shared memory in the cluster
+// form), in the same order in every CTA, and the scalar the phase needs (one warp).
+template <bool CLUSTER>
 __device__ void scalars(const Args& A, Shared& sh, int mode, const double* partials, int k) {
   const int lane = threadIdx.x & 31, G = gridDim.x;
-  constexpr int kLoads = 5;
+  constexpr int kLoads = CLUSTER ? 1 : 5;
+  const auto ld_part = [](const double* p) { return CLUSTER ? *p : __ldcg(p); };
   double s = 0.0;
   for (int q0 = 0; q0 < G; q0 += 32 * kLoads) {
     double v[kLoads];
 #pragma unroll
     for (int j = 0; j < kLoads; ++j) {
       const int q = q0 + 32 * j + lane;
-      v[j] = q < G ? __ldcg(partials + q) : 0.0;
+      v[j] = q < G ? ld_part(partials + q) : 0.0;
     }
 #pragma unroll
     for (int j = 0; j < kLoads; ++j) s += v[j];
@@ -303,6 +315,7 @@ __device__ __forceinline__ Run run_of(const Args& A, const Shared& sh, const Pla
 // w holds the first entries if there is one chunk.  em[par] is clear at the
 // start of a chunk, which clears the other half for the next.  False: the solve
 // has stopped.
+template <bool CLUSTER>
 __device__ bool phase(const Args& A, const Place& pl, Chunk& c, Shared& sh, int mode,
                       const double* partials, int k, int& par, Words& w, double& acc) {
   const bool dag = mode != kP1;
@@ -332,7 +345,7 @@ __device__ bool phase(const Args& A, const Place& pl, Chunk& c, Shared& sh, int 
       bar_arrive(2, kThreads);
       bar_sync(3, kPut);
     } else {
-      if (first) scalars(A, sh, mode, partials, k);
+      if (first) scalars<CLUSTER>(A, sh, mode, partials, k);
       __syncwarp();
       bar_sync(2, kThreads);
     }
@@ -396,6 +409,32 @@ __device__ bool grid_barrier(const Args& A, Shared& sh, double acc, double* part
   return sh.ok;
 }
 
+// The same between the CTAs of a cluster: parts go to every CTA's shared memory, and the
+// hardware's cluster barrier orders them and the vectors.  All CTAs form the same sums and
+// so leave together; nothing here waits for a CTA that might not come.
+template <typename F>
+__device__ void cluster_barrier(Shared& sh, double acc, int ph, F&& work) {
+  const Aligned a = warp_sum(acc);
+  if ((threadIdx.x & 31) == 0) sh.sum[threadIdx.x >> 5] = a;
+  __syncthreads();
+  if (threadIdx.x < gridDim.x) {
+    const double v = total<kWarps>(sh.sum);
+    unsigned there;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                 : "=r"(there)
+                 : "r"((unsigned)__cvta_generic_to_shared(&sh.parts[ph][blockIdx.x])),
+                   "r"(threadIdx.x));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(there), "d"(v) : "memory");
+  }
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  work();
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// CLUSTER: the grid is one cluster.
+template <bool CLUSTER>
 __global__ void __launch_bounds__(kThreads, 1) k_cgne64(Args A) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ Shared sh;
@@ -412,6 +451,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_cgne64(Args A) {
   asm volatile("createpolicy.fractional.L2::evict_last.L2::evict_first.b64 %0, %1;"
                : "=l"(pl.pol)
                : "f"(A.l2frac));
+  if (CLUSTER) {  // every CTA has begun before another writes to its shared memory
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
   for (int q = threadIdx.x; q < A.cs * s.RG * kSItem; q += kThreads) pl.S[q] = 0;
   if (threadIdx.x < kMaxSites) sh.em[0][threadIdx.x] = sh.em[1][threadIdx.x] = -kNotFinite;
   Chunk c = enter_chunk(A, sh, pl, pl.i0);
@@ -438,20 +481,23 @@ __global__ void __launch_bounds__(kThreads, 1) k_cgne64(Args A) {
   for (unsigned gen = 1;; ++gen) {
     // after the update of r (and at the start): x += alpha p
     const double alpha = mode == kP2 ? sh.coef : 0.0;
-    const bool ok = grid_barrier(
-        A, sh, acc, A.partials + ph * G, gen, A.stall_test && blockIdx.x == 0, [&] {
-          if (pl.single)
-            prefetch(s, run_of(A, sh, pl, mode != kP1), sh.f0[warp], sh.n[warp], w);
-          if (mode == kP2) {
+    const auto work = [&] {
+      if (pl.single) prefetch(s, run_of(A, sh, pl, mode != kP1), sh.f0[warp], sh.n[warp], w);
+      if (mode == kP2) {
 #pragma unroll 1
-            for (int q = threadIdx.x; q < nall; q += kThreads) {
-              const int e = pair(q);
-              if (e >= 0) st_comp(A.x, e, fma(alpha, ld_comp(A.p, e), ld_comp(A.x, e)));
-            }
-          }
-        });
-    if (!ok) return;
-    if (!phase(A, pl, c, sh, mode, A.partials + ph * G, k, par, w, acc)) break;
+        for (int q = threadIdx.x; q < nall; q += kThreads) {
+          const int e = pair(q);
+          if (e >= 0) st_comp(A.x, e, fma(alpha, ld_comp(A.p, e), ld_comp(A.x, e)));
+        }
+      }
+    };
+    if (CLUSTER)
+      cluster_barrier(sh, acc, ph, work);
+    else if (!grid_barrier(A, sh, acc, A.partials + ph * G, gen, A.stall_test && blockIdx.x == 0, work))
+      return;
+    if (!phase<CLUSTER>(A, pl, c, sh, mode, CLUSTER ? sh.parts[ph] : A.partials + ph * G, k, par, w,
+                        acc))
+      break;
     ph ^= 1;
     if (mode == kP1) ++k;
     mode = mode == kP1 ? kP2 : kP1;
@@ -487,10 +533,12 @@ bool launch_cgne64(const CoarseGeom& g, const DigitStencil& t, const double2* b,
     int occ = 0, coop = 0, n = 0, most = 0;
     SW_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
     cudaFuncAttributes fa;
-    SW_CUDA(cudaFuncGetAttributes(&fa, k_cgne64));
+    SW_CUDA(cudaFuncGetAttributes(&fa, k_cgne64<false>));
     most -= (int)fa.sharedSizeBytes;
-    SW_CUDA(cudaFuncSetAttribute(k_cgne64, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-    SW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cgne64, kThreads, most));
+    for (auto f : {k_cgne64<false>, k_cgne64<true>})
+      SW_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    SW_CUDA(cudaFuncSetAttribute(k_cgne64<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    SW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cgne64<false>, kThreads, most));
     SW_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device));
     SW_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device));
     if (!coop || occ < 1 || n > kReduceBlocks) return false;
@@ -506,9 +554,33 @@ bool launch_cgne64(const CoarseGeom& g, const DigitStencil& t, const double2* b,
   grid = grid < items ? grid : items;
   Args a{s, t, b, x, r, p, partials, bar, status, maxit, tol, stall_test,
          l2_fraction(16 * digit_entries(g), device), cs, unit};
+  const int all = s.E0 * s.E1 * s.RG;
+  if (all <= kClusterItems && sms_use >= sms && !stall_test) {
+    int n = 1;
+    while (2 * n <= std::min(all, kCluster)) n *= 2;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = n;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(n);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int fits = 0;
+    if (cudaOccupancyMaxActiveClusters(&fits, k_cgne64<true>, &cfg) == cudaSuccess && fits > 0) {
+      a.unit = 1;
+      SW_CUDA(cudaLaunchKernelEx(&cfg, k_cgne64<true>, a));
+      sw_count_launch();
+      return true;
+    }
+    cudaGetLastError();
+  }
   void* params[] = {&a};
-  SW_CUDA(cudaLaunchCooperativeKernel((const void*)k_cgne64, dim3(grid), dim3(kThreads), params,
-                                      smem, st));
+  SW_CUDA(cudaLaunchCooperativeKernel((const void*)k_cgne64<false>, dim3(grid), dim3(kThreads),
+                                      params, smem, st));
   sw_count_launch();
   return true;
 }
