@@ -25,12 +25,6 @@ __device__ __forceinline__ bool all_zero(double2 a, double2 b, double2 c, double
   return a.x == 0.0 && a.y == 0.0 && b.x == 0.0 && b.y == 0.0 && c.x == 0.0 && c.y == 0.0 &&
          d.x == 0.0 && d.y == 0.0;
 }
-__device__ __forceinline__ void cfmac(double2& acc, double2 a, double2 b) {  // acc += conj(a) b
-  acc.x = fma(a.x, b.x, acc.x);
-  acc.x = fma(a.y, b.y, acc.x);
-  acc.y = fma(a.x, b.y, acc.y);
-  acc.y = fma(-a.y, b.x, acc.y);
-}
 
 // ---------------------------------------------------------------------------
 // Lexicographic Dslash: out(s) = m in(s) + sg * sum_mu [W_mu(s) in(s+mu) - conj(W_mu(s-mu)) in(s-mu)]
@@ -211,7 +205,27 @@ __global__ void k_binv_build(const double2* __restrict__ Wps, double mass, doubl
     for (int j = 0; j < 4; ++j) binv[16 * b + 4 * i + j] = I[i][j];
 }
 
-// out = M in (or M^dag in) on nblk KD blocks; one member of a batch per blockIdx.y.
+// Row i of a block's B^-1 (dagger: of its adjoint) times its vector.  Four neighbouring lanes
+// hold a block, lane i its site i: with a thread per block a 64^2 lattice was 16 warps,
+// each of which waited for 56 FMAs of 64 clocks, and every load of the table touched 32 lines.
+// The diagonal is real: B - m is anti-Hermitian and couples the two site parities only.
+__device__ __forceinline__ double2 block_row(const double2* __restrict__ m, int i, double2 u,
+                                             bool dagger) {
+  const unsigned quad = 0xfu << (threadIdx.x & 28);
+  const double d = m[5 * i].x;
+  double2 acc = make_double2(d * u.x, d * u.y);
+#pragma unroll
+  for (int k = 1; k < 4; ++k) {
+    const int j = i ^ k;
+    const double2 v = make_double2(__shfl_xor_sync(quad, u.x, k), __shfl_xor_sync(quad, u.y, k));
+    double2 a = m[dagger ? 4 * j + i : 4 * i + j];
+    if (dagger) a.y = -a.y;
+    cfma(acc, a, v);
+  }
+  return acc;
+}
+// out = M in (or M^dag in) on nblk KD blocks, a thread per site; one member of a batch per
+// blockIdx.y.
 template <int W>
 __global__ void k_block_apply(const double2* __restrict__ M, Pack<2, W> io, int nblk, int dagger,
                               const int* ctl) {
@@ -219,19 +233,9 @@ __global__ void k_block_apply(const double2* __restrict__ M, Pack<2, W> io, int 
   if (ctl && ctl[4 * blockIdx.y]) return;
   const double2* in = io.v[0][blockIdx.y];
   double2* out = io.v[1][blockIdx.y];
-  int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nblk) return;
-  double2 v[4];
-  for (int j = 0; j < 4; ++j) v[j] = in[4 * b + j];
-  const double2* m = M + 16 * b;
-  for (int i = 0; i < 4; ++i) {
-    double2 acc = make_double2(0.0, 0.0);
-    if (!dagger)
-      for (int j = 0; j < 4; ++j) cfma(acc, m[4 * i + j], v[j]);
-    else
-      for (int j = 0; j < 4; ++j) cfmac(acc, m[4 * j + i], v[j]);
-    out[4 * b + i] = acc;
-  }
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= 4 * nblk) return;
+  out[t] = block_row(M + 16 * (long)(t >> 2), t & 3, in[t], dagger);
 }
 
 // (C in)(s) for a site s of parity half par: the two hops of s that leave its
@@ -299,25 +303,17 @@ __global__ void k_hop_block(const double2* __restrict__ Wps, const double2* __re
   const double2* src = io.v[0][blockIdx.y];
   const double2* in = io.v[1][blockIdx.y];
   double2* out = io.v[2][blockIdx.y];
-  int N = L0 * L1, half = N >> 1, nblk = half >> 2;
-  int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= (par < 0 ? 2 * nblk : nblk)) return;
-  if (par < 0 && b < nblk) in += half;
-  const int gb = par < 0 ? b : par * nblk + b;
-  double2 u[4];
-  for (int k = 0; k < 4; ++k) u[k] = hop_out(Wps, in, 4 * gb + k, L0, L1, N);
-  const double2* m = M + 16 * (long)gb;
-  for (int i = 0; i < 4; ++i) {
-    double2 acc = make_double2(0.0, 0.0);
-    if (!dagger)
-      for (int j = 0; j < 4; ++j) cfma(acc, m[4 * i + j], u[j]);
-    else
-      for (int j = 0; j < 4; ++j) cfmac(acc, m[4 * j + i], u[j]);
-    double2 o = src ? src[4 * b + i] : make_double2(0.0, 0.0);
-    o.x = fma(sign, acc.x, o.x);
-    o.y = fma(sign, acc.y, o.y);
-    out[4 * b + i] = o;
-  }
+  const int N = L0 * L1, half = N >> 1;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (par < 0 ? N : half)) return;
+  if (par < 0 && t < half) in += half;
+  const int f = par < 0 ? t : par * half + t;
+  const double2 u = hop_out(Wps, in, f, L0, L1, N);
+  const double2 acc = block_row(M + 16 * (long)(f >> 2), f & 3, u, dagger);
+  double2 o = src ? src[t] : make_double2(0.0, 0.0);
+  o.x = fma(sign, acc.x, o.x);
+  o.y = fma(sign, acc.y, o.y);
+  out[t] = o;
 }
 
 // Long links of the Naik term (Sec. II.A, Eq. freehisq, gauged with the
@@ -403,133 +399,87 @@ __global__ void k_dslash_ps(const double2* __restrict__ Wps, double mass, double
 // ---------------------------------------------------------------------------
 // KD operators on lexicographic fields, for callers that hand over fields in
 // that order: no packing passes, and no division in an index (row of KD blocks
-// = blockIdx.y).  One thread per KD block; its four sites are 32-byte pieces of
-// two rows, whole sectors.  Bound by the FP64 pipe (S: 176 FMAs per pair of
-// blocks, 44 us at 1036 x 1012 at 1.66 FMAs per clock and SM): 97.8 -> 72.5 us
-// there against packing, three kernels on packed halves, a clear and unpacking.
-struct KdBlock {
-  int x0, x1, par;  // corner; parity
-  long b;           // index in the B^-1 table (parity-split)
+// = blockIdx.y).  One thread per site, a block in four neighbouring lanes; its
+// sites are 32-byte pieces of two rows, whole sectors.  Bound by the FP64 pipe
+// (S: 176 FMAs per pair of blocks, 37 us at 1036 x 1012).  S there: 63.5 us (a thread
+// per block: 72.1, whose one wave of warps first waited for all loads and then for the FP64
+// pipe; packing passes and operators on halves: 97.8).
+struct KdSite {
+  int x0, x1;  // of the site
+  int j;       // its place in the block
+  long b;      // the block's index in the B^-1 table (parity-split)
+  long s;      // x0 + L0 x1
 };
-// Blocks of parity `par`, or (par < 0) all of them, in row X1.
-__device__ __forceinline__ bool kd_block(int L0, int L1, int par, int X1, KdBlock& k) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// Sites of the blocks of parity `par`, or (par < 0) of all, in row X1 of blocks.
+__device__ __forceinline__ bool kd_site(int L0, int L1, int par, int X1, KdSite& k) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, i = t >> 2;
   const int X0 = par < 0 ? i : 2 * i + ((X1 + par) & 1);
   if (X0 >= L0 / 2) return false;
-  k.x0 = 2 * X0;
-  k.x1 = 2 * X1;
-  k.par = (X0 + X1) & 1;
-  k.b = (long)k.par * ((long)L0 * L1 / 8) + (long)X1 * (L0 >> 2) + (X0 >> 1);
+  k.j = t & 3;
+  k.x0 = 2 * X0 + (k.j & 1);
+  k.x1 = 2 * X1 + (k.j >> 1);
+  k.b = (long)((X0 + X1) & 1) * ((long)L0 * L1 / 8) + (long)X1 * (L0 >> 2) + (X0 >> 1);
+  k.s = (long)k.x1 * L0 + k.x0;
   return true;
 }
-__device__ __forceinline__ long kd_site(const KdBlock& k, int j, int L0) {
-  return (long)(k.x1 + (j >> 1)) * L0 + k.x0 + (j & 1);
-}
-// C in at site j of a block: the two hops that leave the block.
-__device__ __forceinline__ double2 kd_hop(const double2* __restrict__ W,
-                                          const double2* __restrict__ in, const KdBlock& k, int j,
-                                          int L0, int L1) {
+// C in at a site: the two hops that leave its block, forward from an odd coordinate.
+__device__ __forceinline__ double2 kd_hop(const double2* __restrict__ W, const double2* in,
+                                          const KdSite& k, int L0, int L1) {
   const long N = (long)L0 * L1;
-  const int x0 = k.x0 + (j & 1), x1 = k.x1 + (j >> 1);
+  const bool f0 = k.j & 1, f1 = k.j >> 1;
+  const long t0 = (long)k.x1 * L0 + (f0 ? (k.x0 + 1 == L0 ? 0 : k.x0 + 1) : (k.x0 == 0 ? L0 - 1 : k.x0 - 1));
+  const long t1 = (long)(f1 ? (k.x1 + 1 == L1 ? 0 : k.x1 + 1) : (k.x1 == 0 ? L1 - 1 : k.x1 - 1)) * L0 + k.x0;
+  const double2 w = W[f0 ? k.s : t0], z = W[N + (f1 ? k.s : t1)];
   double2 acc = make_double2(0.0, 0.0);
-  auto back = [&](double2 w, double2 v) {
-    acc.x = fma(-w.x, v.x, acc.x);
-    acc.x = fma(-w.y, v.y, acc.x);
-    acc.y = fma(-w.x, v.y, acc.y);
-    acc.y = fma(w.y, v.x, acc.y);
-  };
-  if (j & 1) {
-    const long t = (long)x1 * L0 + (x0 + 1 == L0 ? 0 : x0 + 1);
-    cfma(acc, W[(long)x1 * L0 + x0], in[t]);
-  } else {
-    const long t = (long)x1 * L0 + (x0 == 0 ? L0 - 1 : x0 - 1);
-    back(W[t], in[t]);
-  }
-  if (j >> 1) {
-    const long t = (long)(x1 + 1 == L1 ? 0 : x1 + 1) * L0 + x0;
-    cfma(acc, W[N + (long)x1 * L0 + x0], in[t]);
-  } else {
-    const long t = (long)(x1 == 0 ? L1 - 1 : x1 - 1) * L0 + x0;
-    back(W[N + t], in[t]);
-  }
-  return acc;
-}
-template <bool DAG>
-__device__ __forceinline__ double2 kd_row(const double2* __restrict__ m, int i, const double2 (&u)[4]) {
-  double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    if (j == i) {  // real: B - m is anti-Hermitian and couples the two site parities only
-      const double d = m[5 * i].x;
-      acc.x = fma(d, u[i].x, acc.x);
-      acc.y = fma(d, u[i].y, acc.y);
-    } else if (DAG) {
-      cfmac(acc, m[4 * j + i], u[j]);
-    } else {
-      cfma(acc, m[4 * i + j], u[j]);
-    }
-  }
+  cfma(acc, f0 ? w : minus_conj(w), in[t0]);
+  cfma(acc, f1 ? z : minus_conj(z), in[t1]);
   return acc;
 }
 // out = B^-1 in on the blocks of parity par (all: par < 0).
 __global__ void __launch_bounds__(128) k_kd_block(const double2* __restrict__ binv, int par,
                                                   const double2* __restrict__ in,
                                                   double2* __restrict__ out, int L0, int L1) {
-  KdBlock k;
+  KdSite k;
   for (int X1 = blockIdx.y; X1 < L1 / 2; X1 += gridDim.y) {
-    if (!kd_block(L0, L1, par, X1, k)) return;
-    double2 u[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) u[j] = in[kd_site(k, j, L0)];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) out[kd_site(k, i, L0)] = kd_row<false>(binv + 16 * k.b, i, u);
+    if (!kd_site(L0, L1, par, X1, k)) return;
+    out[k.s] = block_row(binv + 16 * k.b, k.j, in[k.s], false);
   }
 }
-// out = M C in (DAG: src - M^dag C in) on the blocks of parity par (all: par < 0), M = B^-1.
+// out = M C in (DAG: in - M^dag C in) on the blocks of parity par (all: par < 0), M = B^-1.
+// in and out may be one field where their blocks differ.
 template <bool DAG>
 __global__ void __launch_bounds__(128) k_kd_hop_block(const double2* __restrict__ W,
                                                       const double2* __restrict__ binv, int par,
-                                                      const double2* __restrict__ in,
-                                                      double2* __restrict__ out, int L0, int L1) {
-  KdBlock k;
+                                                      const double2* in, double2* out, int L0,
+                                                      int L1) {
+  KdSite k;
   for (int X1 = blockIdx.y; X1 < L1 / 2; X1 += gridDim.y) {
-    if (!kd_block(L0, L1, par, X1, k)) return;
-    double2 u[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) u[j] = kd_hop(W, in, k, j, L0, L1);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const long s = kd_site(k, i, L0);
-      const double2 v = kd_row<DAG>(binv + 16 * k.b, i, u);
-      if (DAG) {
-        const double2 o = in[s];
-        out[s] = make_double2(o.x - v.x, o.y - v.y);
-      } else {
-        out[s] = v;
-      }
+    if (!kd_site(L0, L1, par, X1, k)) return;
+    const double2 v = block_row(binv + 16 * k.b, k.j, kd_hop(W, in, k, L0, L1), DAG);
+    if (DAG) {
+      const double2 o = in[k.s];
+      out[k.s] = make_double2(o.x - v.x, o.y - v.y);
+    } else {
+      out[k.s] = v;
     }
   }
 }
 // out = src + sign C in; EVEN: on the even blocks, and 0 on the odd block beside each (a
-// thread per pair: a warp of alternating blocks would spend its FP64 issue on idle lanes).
+// warp of alternating blocks would spend its FP64 issue on idle lanes).
 template <bool EVEN>
 __global__ void __launch_bounds__(128) k_kd_hop(const double2* __restrict__ W, double sign,
                                                 const double2* __restrict__ src,
                                                 const double2* __restrict__ in,
                                                 double2* __restrict__ out, int L0, int L1) {
-  KdBlock k;
+  KdSite k;
   for (int X1 = blockIdx.y; X1 < L1 / 2; X1 += gridDim.y) {
-    if (!kd_block(L0, L1, EVEN ? 0 : -1, X1, k)) return;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const long s = kd_site(k, j, L0);
-      const double2 c = kd_hop(W, in, k, j, L0, L1);
-      double2 o = src[s];
-      o.x = fma(sign, c.x, o.x);
-      o.y = fma(sign, c.y, o.y);
-      out[s] = o;
-      if (EVEN) out[s + ((k.x0 & 2) ? -2 : 2)] = make_double2(0.0, 0.0);
-    }
+    if (!kd_site(L0, L1, EVEN ? 0 : -1, X1, k)) return;
+    const double2 c = kd_hop(W, in, k, L0, L1);
+    double2 o = src[k.s];
+    o.x = fma(sign, c.x, o.x);
+    o.y = fma(sign, c.y, o.y);
+    out[k.s] = o;
+    if (EVEN) out[k.s + ((k.x0 & 2) ? -2 : 2)] = make_double2(0.0, 0.0);
   }
 }
 
@@ -587,7 +537,7 @@ void many_block_apply(const sw_gauge* g, const double2* binv, int par, int dagge
   const int half = g->N / 8, nblk = par < 0 ? 2 * half : half;
   with_width(io.n, [&](auto w) {
     constexpr int W = decltype(w)::value;
-    launch_early(k_block_apply<W>, dim3(nblocks(nblk, 128), io.n), 128, 0, s,
+    launch_early(k_block_apply<W>, dim3(nblocks(4L * nblk, 128), io.n), 128, 0, s,
                  binv + (par > 0 ? (long)half * 16 : 0), Pack<2, W>(io), nblk, dagger, ctl);
   });
 }
@@ -603,7 +553,7 @@ void many_hop_block(const sw_gauge* g, const double2* binv, int par, int dagger,
                     const Many<3>& io, cudaStream_t s, const int* ctl) {
   with_width(io.n, [&](auto w) {
     constexpr int W = decltype(w)::value;
-    launch_early(k_hop_block<W>, dim3(nblocks(par < 0 ? g->N / 4 : g->N / 8, 128), io.n), 128, 0, s,
+    launch_early(k_hop_block<W>, dim3(nblocks(par < 0 ? g->N : g->N / 2, 128), io.n), 128, 0, s,
                  g->W_ps, binv, par, dagger, sign, Pack<3, W>(io), g->L0, g->L1, ctl);
   });
 }
@@ -644,7 +594,7 @@ void many_S(const sw_gauge* g, const double2* binv, const Many<3>& v, cudaStream
 
 static dim3 kd_grid(const sw_gauge* g, bool half) {
   const int rows = g->L1 / 2;
-  return dim3(nblocks(g->L0 / (half ? 4 : 2), 128), rows < 32768 ? rows : 32768);
+  return dim3(nblocks(g->L0 * (half ? 1L : 2L), 128), rows < 32768 ? rows : 32768);
 }
 // The same operators on lexicographic fields; tmp must hold N complex, out may be neither in
 // nor tmp.

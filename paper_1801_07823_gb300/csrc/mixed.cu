@@ -44,22 +44,27 @@ __global__ void k_to_f32(const double2* __restrict__ in, float2* __restrict__ ou
   if (i < n) out[i] = f2(in[i]);
 }
 
-// out (float) = M in (double -> float), M per KD block of one parity half
+// Row i of a block's M times its vector, whose sites four neighbouring lanes hold.
+__device__ __forceinline__ float2 block_row_f(const float2* __restrict__ m, int i, float2 u) {
+  const unsigned quad = 0xfu << (threadIdx.x & 28);
+  float2 acc = make_float2(0.f, 0.f);
+  cfmaf(acc, m[5 * i], u);
+#pragma unroll
+  for (int k = 1; k < 4; ++k)
+    cfmaf(acc, m[4 * i + (i ^ k)],
+          make_float2(__shfl_xor_sync(quad, u.x, k), __shfl_xor_sync(quad, u.y, k)));
+  return acc;
+}
+
+// out (float) = M in (double -> float), M per KD block of one parity half; a thread per site
 template <int W>
 __global__ void k_block_apply_df(const float2* __restrict__ M, Pack<2, W> io, int nblk) {
   const double2* in = io.v[0][blockIdx.y];
   float2* out = (float2*)io.v[1][blockIdx.y];
   after_previous();
-  int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nblk) return;
-  float2 v[4];
-  for (int j = 0; j < 4; ++j) v[j] = f2(in[4 * b + j]);
-  const float2* m = M + 16 * b;
-  for (int i = 0; i < 4; ++i) {
-    float2 acc = make_float2(0.f, 0.f);
-    for (int j = 0; j < 4; ++j) cfmaf(acc, m[4 * i + j], v[j]);
-    out[4 * b + i] = acc;
-  }
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= 4 * nblk) return;
+  out[t] = block_row_f(M + 16 * (long)(t >> 2), t & 3, f2(in[t]));
 }
 
 // (C in)(s) for site f of its parity half; in = opposite half (float)
@@ -98,16 +103,10 @@ __global__ void k_hop_block_ff(const float2* __restrict__ W, const float2* __res
   float2* out = (float2*)io.v[1][blockIdx.y];
   after_previous();
   int N = L0 * L1, half = N >> 1;
-  int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= (half >> 2)) return;
-  float2 u[4];
-  for (int k = 0; k < 4; ++k) u[k] = hop_out_f(W, in, par * half + 4 * b + k, L0, L1, N);
-  const float2* m = M + 16 * b;
-  for (int i = 0; i < 4; ++i) {
-    float2 acc = make_float2(0.f, 0.f);
-    for (int j = 0; j < 4; ++j) cfmaf(acc, m[4 * i + j], u[j]);
-    out[4 * b + i] = acc;
-  }
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= half) return;
+  const float2 u = hop_out_f(W, in, par * half + t, L0, L1, N);
+  out[t] = block_row_f(M + 16 * (long)(t >> 2), t & 3, u);
 }
 
 // out_e (double) = src_e - C_eo in_o
@@ -282,7 +281,7 @@ void many_S32(const sw_gauge* g, const float2* W32, const float2* binv32, const 
   }
   with_width(v.n, [&](auto w) {
     constexpr int W = decltype(w)::value;
-    const dim3 blocks(cdiv(nblk, 128), v.n);
+    const dim3 blocks(cdiv(half, 128), v.n);
     launch_early(k_block_apply_df<W>, blocks, 128, 0, s, binv32, Pack<2, W>(in_t), nblk);
     launch_early(k_hop_block_ff<W>, blocks, 128, 0, s, W32, binv32 + (long)nblk * 16, 1,
                  Pack<2, W>(t_v), g->L0, g->L1);
