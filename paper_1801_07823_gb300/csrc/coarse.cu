@@ -12,6 +12,8 @@
 // Direction d collects the couplings carried by fine hops that leave the
 // aggregate in direction d, so the stencil is exact for any coarse extent,
 // including 1 and 2 where X + 0hat and X - 0hat coincide.
+#include <algorithm>
+
 #include "many.h"
 #include "sw_internal.h"
 
@@ -145,15 +147,15 @@ __global__ void __launch_bounds__(5 * NC) k_coarse_apply_nc(const double2* __res
 // Chirality eps of site k of a KD block: + for k = 0, 3 and - for k = 1, 2.
 // full = 1: r is a full parity-split vector and every KD block of the
 // aggregate contributes (used when the fine operator is D itself).
-// Thread (group, i) sums column i of both chiralities over every nth KD block
-// of the aggregate (their P rows are four consecutive sites, so a group reads
-// contiguous memory), and the groups are added in order: 131072 sites x 24
-// columns (512^2) are 3.1 M complex products, 20 us on the FP64 pipe; a call
-// through the C ABI on device fields took 339 us with one thread per column,
-// a serial sum over 32 sites and three allocations, and takes 50 us.
+// Thread (group, i) sums column i over every nth KD block of the aggregate, SITES: over
+// one site k of them, so that it has one chirality (a group per block and site; up to 32
+// columns), else over whole blocks and both; the groups are then added in order.  131072
+// sites x 24 columns (512^2) are 3.1 M complex products, 20.7 us on the FP64 pipe.
+// Restriction at 512^2 44.7 us, with whole blocks and both chiralities per thread 50.4 (eight
+// blocks over five groups, and a third of the FP64 issue in adding the groups up).
 // LEX: r is a lexicographic field.
 // One member of a batch per blockIdx.y.
-template <bool LEX, int W>
+template <bool LEX, bool SITES, int W>
 __global__ void __launch_bounds__(128) k_restrict_fine(const double2* __restrict__ P,
                                                        Pack<2, W> io, int L0, int L1,
                                                        int a0, int a1, int nv, int groups,
@@ -169,27 +171,39 @@ __global__ void __launch_bounds__(128) k_restrict_fine(const double2* __restrict
   if (grp < groups) {
     double2 acc[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
     // blocks of the aggregate row by row; half: every second one of a row
-    const int per = full ? a0 : a0 / 2;
-    for (int b = grp; b < per * a1; b += groups) {
+    const int per = full ? a0 : a0 / 2, step = SITES ? groups >> 2 : groups;
+#pragma unroll 4
+    for (int b = SITES ? grp >> 2 : grp; b < per * a1; b += step) {
       const int by = b / per, X1 = A1 * a1 + by;
       const int X0 = full ? A0 * a0 + (b - by * per)
                           : A0 * a0 + 2 * (b - by * per) + ((X1 + A0 * a0) & 1);
       const int h = ps_index(2 * X0, 2 * X1, L0, N);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
+      for (int q = 0; q < (SITES ? 1 : 4); ++q) {
+        const int k = SITES ? grp & 3 : q;
         const double2 v = r[LEX ? (long)(2 * X1 + (k >> 1)) * L0 + 2 * X0 + (k & 1) : h + k];
-        cfmac(acc[k == 1 || k == 2], P[(long)(h + k) * nv + i], v);
+        cfmac(acc[!SITES && (q == 1 || q == 2)], P[(long)(h + k) * nv + i], v);
       }
     }
-    part[2 * threadIdx.x] = acc[0];
-    part[2 * threadIdx.x + 1] = acc[1];
+    if (SITES) {
+      part[threadIdx.x] = acc[0];
+    } else {
+      part[2 * threadIdx.x] = acc[0];
+      part[2 * threadIdx.x + 1] = acc[1];
+    }
   }
   __syncthreads();
   for (int t = threadIdx.x; t < 2 * nv; t += blockDim.x) {
     const int c = t / nv, col = t - c * nv;
-    double2 s = part[2 * col + c];
-    for (int q = 1; q < groups; ++q) {
-      const double2 v = part[2 * (q * nv + col) + c];
+    // SITES: groups 4 q and 4 q + 3 for chirality 0, 4 q + 1 and 4 q + 2 for 1
+    const int n = SITES ? groups / 2 : groups;
+    const auto of = [&](int q) {
+      return SITES ? part[(4 * (q >> 1) + (c ? 1 + (q & 1) : 3 * (q & 1))) * nv + col]
+                   : part[2 * (q * nv + col) + c];
+    };
+    double2 s = of(0);
+    for (int q = 1; q < n; ++q) {
+      const double2 v = of(q);
       s.x += v.x;
       s.y += v.y;
     }
@@ -684,10 +698,16 @@ void many_restrict_fine(const sw_gauge* g, int a0, int a1, int nv, const double2
                         const Many<2>& io, cudaStream_t s, int full, bool lex) {
   int nagg = (g->L0 / (2 * a0)) * (g->L1 / (2 * a1));
   const int blocks = a0 * a1 / (full ? 1 : 2);
-  const int groups = 128 / nv < blocks ? 128 / nv : blocks;
+  const bool sites = 4 * nv <= 128;
+  int groups = 128 / nv < blocks ? 128 / nv : blocks;
+  if (sites) {  // as many as the rounds of the busiest one need
+    const int most = 128 / (4 * nv), rounds = std::max(1, (blocks + most - 1) / most);
+    groups = 4 * std::max(1, (blocks + rounds - 1) / rounds);
+  }
   with_width(io.n, [&](auto w) {
     constexpr int W = decltype(w)::value;
-    auto k = lex ? k_restrict_fine<true, W> : k_restrict_fine<false, W>;
+    auto k = sites ? (lex ? k_restrict_fine<true, true, W> : k_restrict_fine<false, true, W>)
+                   : (lex ? k_restrict_fine<true, false, W> : k_restrict_fine<false, false, W>);
     launch_early(k, dim3(nagg, io.n), 128, 0, s, P, Pack<2, W>(io), g->L0, g->L1, a0, a1, nv, groups, full);
   });
 }
