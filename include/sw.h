@@ -178,7 +178,13 @@ int sw_dslash(sw_gauge* g, double mass, int op, int precision, const void* in, v
  *            with coarse site index X0 + E0 X1.  NULL: drawn from seed with
  *            SplitMix64 + Box-Muller (vector i of level l: stream
  *            sw_stream_seed(seed, l, i), element j from outputs 2j, 2j+1).
- * mass must be > 0: the 2x2 block B is singular at m = 0 for some links. */
+ * mass must be > 0: the 2x2 block B is singular at m = 0 for some links.
+ * The relaxation amplifies rounding: about a thousandfold per CG step where a
+ * KD block is nearly singular (|B^-1| close to 1/m), and on any field to order
+ * one in hundreds of steps.  All operations of a setup therefore run in one
+ * fixed FP64 order and equal inputs give equal hierarchies; two
+ * implementations that round differently agree on P and Y after few steps on
+ * ordinary fields only. */
 int sw_mg_setup(sw_gauge* g, double mass, int levels, const int* block, const int* nvec,
                 const sw_mg_params* params, uint64_t seed, const double* const* psi0,
                 sw_mg** out);

@@ -51,12 +51,15 @@ inline int cdiv(long a, long b) { return (int)((a + b - 1) / b); }
 // y_X = sum_d Y[X][d] x_{X+d}, generic nc.  A CTA holds spc sites x nc rows,
 // one thread per output row; the five neighbour vectors of its sites are
 // staged in shared memory and every Y load is a coalesced column segment.
-__global__ void k_coarse_apply(const double2* __restrict__ Y, const double2* __restrict__ in,
-                               double2* __restrict__ out, int E0, int E1, int nc, int spc,
-                               int dagger, const int* __restrict__ skip,
-                               unsigned long long* exec) {
+// One member of a batch per blockIdx.y.
+template <int W>
+__global__ void k_coarse_apply(const double2* __restrict__ Y, Pack<2, W> io, int E0, int E1, int nc,
+                               int spc, int dagger, const int* skip, unsigned long long* exec) {
   extern __shared__ double2 xs[];  // [spc][5][nc]
-  if (skip && *skip) return;
+  const double2* in = io.v[0][blockIdx.y];
+  double2* out = io.v[1][blockIdx.y];
+  after_previous();
+  if (skip && skip[4 * blockIdx.y]) return;
   if (exec && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(exec, 1ull);
   int nsites = E0 * E1;
   int site0 = blockIdx.x * spc;
@@ -93,14 +96,16 @@ __global__ void k_coarse_apply(const double2* __restrict__ Y, const double2* __r
 // Y[X][d] (coalesced across i), unrolled so that many loads are in flight:
 // in FP64 the kernel is bound by the FP64 pipe, which needs every SM busy.
 // The five partial sums are added in direction order (deterministic).
-template <int NC, bool DAG>
+// One member of a batch per blockIdx.y.
+template <int NC, bool DAG, int W>
 __global__ void __launch_bounds__(5 * NC) k_coarse_apply_nc(const double2* __restrict__ Y,
-                                                            const double2* __restrict__ in,
-                                                            double2* __restrict__ out, int E0,
-                                                            int E1, int rs,
-                                                            const int* __restrict__ skip,
+                                                            Pack<2, W> io, int E0, int E1, int rs,
+                                                            const int* skip,
                                                             unsigned long long* exec) {
-  if (skip && *skip) return;
+  const double2* in = io.v[0][blockIdx.y];
+  double2* out = io.v[1][blockIdx.y];
+  after_previous();
+  if (skip && skip[4 * blockIdx.y]) return;
   if (exec && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(exec, 1ull);
   __shared__ double2 xs[5][NC];
   __shared__ double2 part[5][NC];
@@ -657,42 +662,46 @@ int pick_spc(int nc) {
 }  // namespace
 
 template <int NC>
-static void coarse_apply_nc(const CoarseGeom& g, const double2* Y, int dagger, const double2* in,
-                            double2* out, cudaStream_t s, const int* skip,
-                            unsigned long long* exec) {
+static void coarse_apply_nc(const CoarseGeom& g, const double2* Y, int dagger, const Many<2>& io,
+                            cudaStream_t s, const int* ctl, unsigned long long* exec) {
   int nsites = g.E0 * g.E1;
   // split rows over CTAs until the grid covers the GPU about four times
   int rs = 1;
-  while (rs < 8 && NC % (2 * rs) == 0 && (NC / (2 * rs)) % 8 == 0 && (long)nsites * rs < 4 * 152)
+  while (rs < 8 && NC % (2 * rs) == 0 && (NC / (2 * rs)) % 8 == 0 &&
+         (long)nsites * rs * io.n < 4 * 152)
     rs *= 2;
-  if (dagger)
-    k_coarse_apply_nc<NC, true><<<nsites * rs, 5 * (NC / rs), 0, s>>>(Y, in, out, g.E0, g.E1, rs,
-                                                                      skip, exec);
-  else
-    k_coarse_apply_nc<NC, false><<<nsites * rs, 5 * (NC / rs), 0, s>>>(Y, in, out, g.E0, g.E1, rs,
-                                                                       skip, exec);
-  SW_LAUNCH_CHECK();
+  with_width(io.n, [&](auto w) {
+    constexpr int W = decltype(w)::value;
+    auto k = dagger ? k_coarse_apply_nc<NC, true, W> : k_coarse_apply_nc<NC, false, W>;
+    launch_early(k, dim3(nsites * rs, io.n), 5 * (NC / rs), 0, s, Y, Pack<2, W>(io), g.E0, g.E1, rs,
+                 ctl, exec);
+  });
 }
 
-void launch_coarse_apply(const CoarseGeom& g, const double2* Y, int dagger, const double2* in,
-                         double2* out, cudaStream_t s, const int* skip,
-                         unsigned long long* exec) {
+void many_coarse(const CoarseGeom& g, const double2* Y, int dagger, const Many<2>& io,
+                 cudaStream_t s, const int* ctl, unsigned long long* exec) {
   switch (g.nc) {
-    case 8: return coarse_apply_nc<8>(g, Y, dagger, in, out, s, skip, exec);
-    case 12: return coarse_apply_nc<12>(g, Y, dagger, in, out, s, skip, exec);
-    case 16: return coarse_apply_nc<16>(g, Y, dagger, in, out, s, skip, exec);
-    case 24: return coarse_apply_nc<24>(g, Y, dagger, in, out, s, skip, exec);
-    case 32: return coarse_apply_nc<32>(g, Y, dagger, in, out, s, skip, exec);
-    case 48: return coarse_apply_nc<48>(g, Y, dagger, in, out, s, skip, exec);
-    case 64: return coarse_apply_nc<64>(g, Y, dagger, in, out, s, skip, exec);
+    case 8: return coarse_apply_nc<8>(g, Y, dagger, io, s, ctl, exec);
+    case 12: return coarse_apply_nc<12>(g, Y, dagger, io, s, ctl, exec);
+    case 16: return coarse_apply_nc<16>(g, Y, dagger, io, s, ctl, exec);
+    case 24: return coarse_apply_nc<24>(g, Y, dagger, io, s, ctl, exec);
+    case 32: return coarse_apply_nc<32>(g, Y, dagger, io, s, ctl, exec);
+    case 48: return coarse_apply_nc<48>(g, Y, dagger, io, s, ctl, exec);
+    case 64: return coarse_apply_nc<64>(g, Y, dagger, io, s, ctl, exec);
     default: break;
   }
   int spc = pick_spc(g.nc);
   int nsites = g.E0 * g.E1;
   size_t smem = (size_t)spc * 5 * g.nc * sizeof(double2);
-  k_coarse_apply<<<cdiv(nsites, spc), spc * g.nc, smem, s>>>(Y, in, out, g.E0, g.E1, g.nc, spc,
-                                                              dagger, skip, exec);
-  SW_LAUNCH_CHECK();
+  with_width(io.n, [&](auto w) {
+    constexpr int W = decltype(w)::value;
+    launch_early(k_coarse_apply<W>, dim3(cdiv(nsites, spc), io.n), spc * g.nc, smem, s, Y,
+                 Pack<2, W>(io), g.E0, g.E1, g.nc, spc, dagger, ctl, exec);
+  });
+}
+void launch_coarse_apply(const CoarseGeom& g, const double2* Y, int dagger, const double2* in,
+                         double2* out, cudaStream_t s) {
+  many_coarse(g, Y, dagger, Many<2>(0, in, out), s);
 }
 void many_restrict_fine(const sw_gauge* g, int a0, int a1, int nv, const double2* P,
                         const Many<2>& io, cudaStream_t s, int full, bool lex) {

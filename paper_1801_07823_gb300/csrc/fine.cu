@@ -224,6 +224,22 @@ __device__ __forceinline__ double2 block_row(const double2* __restrict__ m, int 
   }
   return acc;
 }
+// The same with all four products added in the order of the columns, the diagonal as a complex
+// number.  The kernels on parity-split fields use this one: they relax the null vectors, whose
+// values depend on every rounding (mg_setup), so their order of operations is fixed.
+__device__ __forceinline__ double2 block_row_ordered(const double2* __restrict__ m, int i,
+                                                     double2 u, bool dagger) {
+  const unsigned quad = 0xfu << (threadIdx.x & 28);
+  double2 acc = make_double2(0.0, 0.0);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const double2 v = make_double2(__shfl_sync(quad, u.x, j, 4), __shfl_sync(quad, u.y, j, 4));
+    double2 a = m[dagger ? 4 * j + i : 4 * i + j];
+    if (dagger) a.y = -a.y;
+    cfma(acc, a, v);
+  }
+  return acc;
+}
 // out = M in (or M^dag in) on nblk KD blocks, a thread per site; one member of a batch per
 // blockIdx.y.
 template <int W>
@@ -235,7 +251,7 @@ __global__ void k_block_apply(const double2* __restrict__ M, Pack<2, W> io, int 
   double2* out = io.v[1][blockIdx.y];
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 4 * nblk) return;
-  out[t] = block_row(M + 16 * (long)(t >> 2), t & 3, in[t], dagger);
+  out[t] = block_row_ordered(M + 16 * (long)(t >> 2), t & 3, in[t], dagger);
 }
 
 // (C in)(s) for a site s of parity half par: the two hops of s that leave its
@@ -309,7 +325,7 @@ __global__ void k_hop_block(const double2* __restrict__ Wps, const double2* __re
   if (par < 0 && t < half) in += half;
   const int f = par < 0 ? t : par * half + t;
   const double2 u = hop_out(Wps, in, f, L0, L1, N);
-  const double2 acc = block_row(M + 16 * (long)(f >> 2), f & 3, u, dagger);
+  const double2 acc = block_row_ordered(M + 16 * (long)(f >> 2), f & 3, u, dagger);
   double2 o = src ? src[t] : make_double2(0.0, 0.0);
   o.x = fma(sign, acc.x, o.x);
   o.y = fma(sign, acc.y, o.y);

@@ -13,8 +13,8 @@
 // and the exchange of the CTAs' parts: 2.7 us for an update, 5 with a sum.
 //
 // Every sum runs in an order that depends on n alone: a grid-stride slice per
-// thread, aligned sums over warps and CTAs, and the last CTA to finish adds the
-// CTAs' parts.  A member's scalars do not depend on the others of its batch.
+// thread, aligned sums over warps and CTAs (the setup's: trees of FP64 additions, see
+// mg_setup), and the last CTA to finish adds the CTAs' parts.  A member's scalars do not depend on the others of its batch.
 #include "many.h"
 
 #include "sums.cuh"
@@ -132,6 +132,8 @@ struct Add3 : NoCoef, NoSums {
     v(0)[i] = make_double2((a.x + b.x) + d.x, (a.y + b.y) + d.y);
   }
 };
+// Base of the operations whose sums are plain FP64 trees (the setup's).
+struct Tree {};
 struct Dot : NoCoef {
   static constexpr int K = 2, R = 2;
   int s;
@@ -148,6 +150,8 @@ struct Norm : NoCoef {
   template <typename V>
   __device__ void store(const V&, double2* S, const double* t, int*) const { S[s] = make_double2(t[0], 0.0); }
 };
+struct SetupDot : Dot, Tree {};
+struct SetupNorm : Norm, Tree {};
 struct Mgs {
   static constexpr int K = 5, R = 2;
   int s, s_qq;
@@ -219,7 +223,7 @@ struct Copy : NoCoef, NoSums {
   template <typename V>
   __device__ void elem(const V& v, long i, double2, double*) const { v(0)[i] = v(1)[i]; }
 };
-struct CgStart : NoCoef {
+struct CgStart : NoCoef, Tree {
   static constexpr int K = 4, R = 1;
   int s_rr, s_stop, maxit;
   double tol;
@@ -241,7 +245,7 @@ struct CgStart : NoCoef {
     ctl[0] = maxit <= 0 || !(rn > stop);
   }
 };
-struct CgStep {
+struct CgStep : Tree {
   static constexpr int K = 4, R = 1;
   int s_rr, s_pq, s_new, s_stop, maxit;
   __device__ double coef(const double2* S, int comp) const { return comp ? 0.0 : S[s_rr].x / S[s_pq].x; }
@@ -326,18 +330,40 @@ __global__ void __launch_bounds__(kThreads) k_many(Op op, Pack<Op::K, W> v, long
   for (long i = (long)blockIdx.x * kThreads + threadIdx.x; i < n; i += (long)gridDim.x * kThreads)
     op.elem(get, i, a, acc);
   if constexpr (R > 0) {
-    __shared__ swsum::Aligned part[R][kWarps];
+    constexpr bool tree = std::is_base_of<Tree, Op>::value;
+    using Part = typename std::conditional<tree, double, swsum::Aligned>::type;
+    __shared__ Part part[R][kWarps];
     __shared__ double sum[R];
     __shared__ bool last;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const auto cta_sums = [&]() {  // of acc, to sum
+      if constexpr (tree) {
+        const auto warp = [](double v) {
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const swsum::Aligned t = swsum::warp_sum(acc[r]);
-        if (lane == 0) part[r][w] = t;
+          for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          return v;
+        };
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const double t = warp(acc[r]);
+          if (lane == 0) part[r][w] = t;
+        }
+        __syncthreads();
+        if (w == 0)
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const double t = warp(lane < kWarps ? part[r][lane] : 0.0);
+            if (lane == 0) sum[r] = t;
+          }
+      } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const swsum::Aligned t = swsum::warp_sum(acc[r]);
+          if (lane == 0) part[r][w] = t;
+        }
+        __syncthreads();
+        if (threadIdx.x < R) sum[threadIdx.x] = swsum::total<kWarps>(part[threadIdx.x]);
       }
-      __syncthreads();
-      if (threadIdx.x < R) sum[threadIdx.x] = swsum::total<kWarps>(part[threadIdx.x]);
       __syncthreads();
     };
     cta_sums();
@@ -377,8 +403,10 @@ void launch(sw_ctx* c, long n, const Op& op, const Many<Op::K>& v, double* host 
             int* ctl = nullptr) {
   if (v.n == 0 || n <= 0) return;
   long grid = (n + kThreads - 1) / kThreads;
-  if (Op::R > 0 && n <= 2 * kThreads) grid = 1;
-  if (Op::R > 0 && grid > kManyBlocks) grid = kManyBlocks;
+  constexpr bool tree = std::is_base_of<Tree, Op>::value;  // slices of these: never change
+  if (Op::R > 0 && !tree && n <= 2 * kThreads) grid = 1;
+  const long most = tree ? kReduceBlocks : kManyBlocks;
+  if (Op::R > 0 && grid > most) grid = most;
   with_width(v.n, [&](auto w) {
     constexpr int W = decltype(w)::value;
     launch_early(k_many<Op, W>, dim3((unsigned)grid, v.n), kThreads, 0, c->stream, op,
@@ -406,9 +434,7 @@ void many_sub_norm(sw_ctx* c, long n, const Many<3>& v, int s, double* host) {
   launch(c, n, SubNorm{{}, s}, v, host);
 }
 void many_add3(sw_ctx* c, long n, const Many<4>& v) { launch(c, n, Add3{}, v); }
-void many_dot(sw_ctx* c, long n, const Many<2>& v, int s, const int* ctl) {
-  launch(c, n, Dot{{}, s}, v, nullptr, const_cast<int*>(ctl));
-}
+void many_dot(sw_ctx* c, long n, const Many<2>& v, int s) { launch(c, n, Dot{{}, s}, v); }
 void many_norm(sw_ctx* c, long n, const Many<1>& v, int s, double* host) {
   launch(c, n, Norm{{}, s}, v, host);
 }
@@ -421,17 +447,23 @@ void many_scale_dot(sw_ctx* c, long n, const Many<3>& v, int s_qq, int s_a) {
 void many_update(sw_ctx* c, long n, const Many<4>& v, int s_a, int s_rr, double* host) {
   launch(c, n, Update{s_a, s_rr}, v, host);
 }
+void many_setup_dot(sw_ctx* c, long n, const Many<2>& v, int s, const int* ctl) {
+  launch(c, n, SetupDot{{{}, s}}, v, nullptr, const_cast<int*>(ctl));
+}
+void many_setup_norm(sw_ctx* c, long n, const Many<1>& v, int s, double* host) {
+  launch(c, n, SetupNorm{{{}, s}}, v, host);
+}
 void many_copy(sw_ctx* c, long n, const Many<2>& v) { launch(c, n, Copy{}, v); }
 void many_add(sw_ctx* c, long n, const Many<2>& v) { launch(c, n, Add{}, v); }
 void many_project(sw_ctx* c, long n, const Many<2>& v, int s) { launch(c, n, Project{{}, s}, v); }
 void many_normalise(sw_ctx* c, long n, const Many<1>& v, int s) { launch(c, n, Normalise{{}, s}, v); }
 void many_cg_start(sw_ctx* c, long n, const Many<4>& v, int s_rr, int s_stop, double tol, int maxit,
                    int* ctl) {
-  launch(c, n, CgStart{{}, s_rr, s_stop, maxit, tol}, v, nullptr, ctl);
+  launch(c, n, CgStart{{}, {}, s_rr, s_stop, maxit, tol}, v, nullptr, ctl);
 }
 void many_cg_step(sw_ctx* c, long n, const Many<4>& v, int s_rr, int s_pq, int s_new, int s_stop,
                   int maxit, int* ctl) {
-  launch(c, n, CgStep{s_rr, s_pq, s_new, s_stop, maxit}, v, nullptr, ctl);
+  launch(c, n, CgStep{{}, s_rr, s_pq, s_new, s_stop, maxit}, v, nullptr, ctl);
 }
 void many_xpay(sw_ctx* c, long n, const Many<2>& v, int s_new, int s_old, const int* ctl) {
   launch(c, n, Xpay{{}, s_new, s_old}, v, nullptr, const_cast<int*>(ctl));

@@ -65,13 +65,17 @@ void many_mr_last(sw_ctx* c, long n, const Many<5>& oxrab, int s, double om, boo
 void many_sub(sw_ctx* c, long n, const Many<3>& oab);                       // o = a - b
 void many_sub_norm(sw_ctx* c, long n, const Many<3>& oab, int s, double* host);
 void many_add3(sw_ctx* c, long n, const Many<4>& oabd);                     // o = (a + b) + d
-void many_dot(sw_ctx* c, long n, const Many<2>& ab, int s, const int* ctl = nullptr);
+void many_dot(sw_ctx* c, long n, const Many<2>& ab, int s);
 void many_norm(sw_ctx* c, long n, const Many<1>& a, int s, double* host = nullptr);
 // q -= S[s] qj, p -= S[s] pj; then <qn, q> in s, or |q|^2 in s_qq for a member without qn
 void many_mgs(sw_ctx* c, long n, const Many<5>& q_p_qj_pj_qn, int s, int s_qq);
 void many_scale_dot(sw_ctx* c, long n, const Many<3>& qpr, int s_qq, int s_a);  // q, p /= |q|; <q, r>
 // x += S[s_a] p, r -= S[s_a] q; |r|^2
 void many_update(sw_ctx* c, long n, const Many<4>& xrpq, int s_a, int s_rr, double* host);
+// <a, b> and |a|^2 of the setup, like many_cg_start and many_cg_step with plain FP64 trees over
+// fixed slices (see mg_setup).
+void many_setup_dot(sw_ctx* c, long n, const Many<2>& ab, int s, const int* ctl = nullptr);
+void many_setup_norm(sw_ctx* c, long n, const Many<1>& a, int s, double* host = nullptr);
 void many_copy(sw_ctx* c, long n, const Many<2>& ob);                       // o = b
 void many_add(sw_ctx* c, long n, const Many<2>& ob);                        // o += b
 void many_project(sw_ctx* c, long n, const Many<2>& vu, int s);             // v -= S[s] u
@@ -99,6 +103,9 @@ void many_S32(const sw_gauge* g, const float2* W32, const float2* binv32, const 
 // A A^dag on full vectors; t, u: N of scratch.
 void many_normal_A(const sw_gauge* g, const double2* binv, const Many<4>& in_out_t_u,
                    cudaStream_t s, const int* ctl);
+// FP64 stencil on the FP64 pipe, its sums in a fixed order.
+void many_coarse(const CoarseGeom& g, const double2* Y, int dagger, const Many<2>& in_out,
+                 cudaStream_t s, const int* ctl = nullptr, unsigned long long* exec = nullptr);
 void many_coarse_h(const CoarseGeom& g, const __half2* Yh, const float* scale, int dagger,
                    const Many<2>& in_out, cudaStream_t s);
 void many_digit(const CoarseGeom& g, const DigitStencil& t, const double2* Y, int dagger,

@@ -86,9 +86,7 @@ void coarse_op(sw_mg* mg, int l, int dagger, const Many<2>& v, const int* ctl) {
   if (L.dg.T)
     many_digit(cg, L.dg, L.Y, dagger, v, c->device, c->stream, ctl, exec);
   else
-    for (int m = 0; m < v.n; ++m)
-      launch_coarse_apply(cg, L.Y, dagger, v.v[0][m], v.v[1][m], c->stream,
-                          ctl ? ctl + 4 * m : nullptr, exec);
+    many_coarse(cg, L.Y, dagger, v, c->stream, ctl, exec);
 }
 
 // Operator of level l in the solve on (in, out, tmp) of every member: S on level
@@ -117,7 +115,8 @@ void level_op(sw_mg* mg, int l, const Many<3>& v, bool lowp, const int* ctl = nu
   timing_end(c, tk);
 }
 // Normal operator used by the setup on level l: A A^dag on (in, out, t, u) of every
-// member (full fine vectors on level 0).
+// member (full fine vectors on level 0).  Its products are FP64 FMAs in a fixed order on
+// every level, not the digit products of the solves (see mg_setup).
 void level_normal(sw_mg* mg, int l, const Many<4>& v, const int* ctl) {
   sw_ctx* c = mg->ctx;
   if (l == 0 && mg->fine_D) {
@@ -131,8 +130,10 @@ void level_normal(sw_mg* mg, int l, const Many<4>& v, const int* ctl) {
     for (int dagger = 1; dagger >= 0; --dagger) {
       Many<2> io;
       for (int m = 0; m < v.n; ++m) io.add(0, v.v[dagger ? 0 : 2][m], v.v[dagger ? 2 : 1][m]);
+      const MgLevel& L = mg->lev[l];
       const int tk = timing_begin(c, l, v.n);
-      coarse_op(mg, l, dagger, io, ctl);
+      many_coarse(CoarseGeom{L.E0, L.E1, L.nc}, L.Y, dagger, io, c->stream, ctl,
+                  c->timing ? c->exec + l : nullptr);
       timing_end(c, tk);
     }
   }
@@ -266,7 +267,7 @@ static std::vector<int> cg_setup(sw_mg* mg, int l, const SetupVecs& v, int w) {
     if (done) break;
     for (int q = 0; q < kIterBatch && issued < maxit; ++q, ++issued) {
       level_normal(mg, l, op, ctl);
-      many_dot(c, n, pq, s_pq, ctl);
+      many_setup_dot(c, n, pq, s_pq, ctl);
       many_cg_step(c, n, step, s_rr[0], s_pq, s_rr[1], s_stop, maxit, ctl);
       many_xpay(c, n, pr, s_rr[1], s_rr[0], ctl);
       std::swap(s_rr[0], s_rr[1]);
@@ -282,6 +283,13 @@ int mg_coarsest_solve(sw_mg* mg, const double2* b, double2* x) {
 }
 
 // ---------------------------------------------------------------- setup
+// The null vectors depend on every rounding of their relaxation: CG on A A^dag multiplies a
+// rounding difference about a thousandfold per step where a KD block is nearly singular
+// (|B^-1| up to 1/m), and to order one in some hundreds of steps on any field.  Eight steps at
+// 512^2 with other sums and products of the same accuracy moved single elements of the level-2
+// stencil by 3e-2.  So that a configuration has one hierarchy, whatever kernels the solves use,
+// the operations of a setup have one order: plain FP64 products, and sums as trees over slices
+// that depend on n alone (Tree in many.cu), the same for any grouping of the vectors.
 void mg_setup(sw_mg* mg, const double* const* psi0, uint64_t seed) {
   sw_ctx* c = mg->ctx;
   sw_gauge* g = mg->g;
@@ -339,7 +347,7 @@ void mg_setup(sw_mg* mg, const double* const* psi0, uint64_t seed) {
       }
       for (int pass = 0; pass < passes; ++pass) {
         if (pass > 0) {
-          many_norm(c, n, psi, 30);
+          many_setup_norm(c, n, psi, 30);
           many_normalise(c, n, psi, 30);
         }
         level_normal(mg, l, first, nullptr);  // e solves A A^dag e = -A A^dag psi
@@ -351,14 +359,14 @@ void mg_setup(sw_mg* mg, const double* const* psi0, uint64_t seed) {
     // global modified Gram-Schmidt: vector j is normalised and taken out of the later ones
     for (int j = 0; j < nv; ++j) {
       double2* vj = V + (long)j * n;
-      many_norm(c, n, Many<1>(page(j), vj), 32, c->h_many->norm + j);
+      many_setup_norm(c, n, Many<1>(page(j), vj), 32, c->h_many->norm + j);
       many_normalise(c, n, Many<1>(page(j), vj), 32);
       Many<2> dots, later;
       for (int i = j + 1; i < nv; ++i) {
         dots.add(page(i), vj, V + (long)i * n);
         later.add(page(i), V + (long)i * n, vj);
       }
-      many_dot(c, n, dots, 31);
+      many_setup_dot(c, n, dots, 31);
       many_project(c, n, later, 31);
     }
     SW_CUDA(cudaStreamSynchronize(s));
@@ -394,13 +402,10 @@ void mg_setup(sw_mg* mg, const double* const* psi0, uint64_t seed) {
       launch_build_Y_coarse(CoarseGeom{L.E0, L.E1, L.nc}, L.b0, L.b1, nv, L.Y, L.P, T, C.Y, s);
     }
     const CoarseGeom geom{C.E0, C.E1, C.nc};
-    if (digit_entries(geom) <= kMaxDigitEntries) {
-      // digit entries: kept on the coarsest level and by FP64 hierarchies; on the other
-      // levels of a mixed hierarchy only the setup of the next level uses them
-      const bool keep = l + 2 == mg->nlev || !mg->mixed;
-      const long tn = digit_entries(geom), en = (digit_rows(geom) + 3) / 4;
-      uint4* T = (uint4*)(keep ? mg_alloc(mg, tn) : tmp.get(tn));
-      int* ex = (int*)(keep ? mg_alloc(mg, en) : tmp.get(en));
+    // digit entries for the solves: on the coarsest level and all levels of FP64 hierarchies
+    if ((l + 2 == mg->nlev || !mg->mixed) && digit_entries(geom) <= kMaxDigitEntries) {
+      uint4* T = (uint4*)mg_alloc(mg, digit_entries(geom));
+      int* ex = (int*)mg_alloc(mg, (digit_rows(geom) + 3) / 4);
       launch_pack_digits(geom, C.Y, T, ex, s);
       C.dg = DigitStencil{T, ex};
     }
@@ -418,8 +423,6 @@ void mg_setup(sw_mg* mg, const double* const* psi0, uint64_t seed) {
     }
     SW_CUDA(cudaStreamSynchronize(s));
   }
-  if (mg->mixed)
-    for (int l = 1; l + 1 < mg->nlev; ++l) mg->lev[l].dg = DigitStencil{};
   // solve workspace
   for (int l = 0; l < mg->nlev; ++l) {
     MgLevel& L = mg->lev[l];

@@ -276,8 +276,7 @@ struct CoarseGeom {
 // once per launch that did run.
 // dagger = 1 applies the adjoint stencil from the same storage.
 void launch_coarse_apply(const CoarseGeom& g, const double2* Y, int dagger, const double2* in,
-                         double2* out, cudaStream_t s, const int* skip = nullptr,
-                         unsigned long long* exec = nullptr);
+                         double2* out, cudaStream_t s);
 // A coarse stencil as digit entries (digit.cuh) with the exponent of every row,
 // for FP64 products on the tensor cores (digit.cu).  One copy serves A and A^dag.
 struct DigitStencil {
