@@ -191,11 +191,13 @@ void many_digit(const CoarseGeom& g, const DigitStencil& t, const double2* Y, in
   const dim3 grid(units < slots ? units : slots, io.n);
   with_width(io.n, [&](auto w) {
     constexpr int W = decltype(w)::value;
+    // the flag is set after the attributes: a thread that sees it may launch
     static std::atomic<bool> wide[64];
-    if (!wide[device & 63].exchange(true)) {
+    if (!wide[device & 63].load()) {
       constexpr int most = 40 * (4 * kQuadBytes + 32) + 16 * kSItem * (int)sizeof(int);  // nc = 128
       for (auto f : {k_digit_apply<true, W>, k_digit_apply<false, W>})
         SW_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+      wide[device & 63].store(true);
     }
     auto k = dagger ? k_digit_apply<true, W> : k_digit_apply<false, W>;
     launch_early(k, grid, kNT, smem, st, s, t.T, t.ex, Y, Pack<2, W>(io), parts, ctl, exec);
