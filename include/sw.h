@@ -166,6 +166,12 @@ int sw_dslash(sw_gauge* g, double mass, int op, int precision, const void* in, v
  * operator P^dag A P, recursively.  The setup runs in FP64; with
  * params->precision = SW_MG_MIXED it also keeps the reduced-precision copies
  * of the operators that the mixed solve uses.
+ * Device memory permitting, a second copy of the stencils (16 bytes per entry)
+ * of all levels, or of the coarsest one of a mixed hierarchy, is kept as digit
+ * entries, from which the solves form FP64 products on the tensor cores; levels
+ * with more than SW_DIGIT_ENTRIES entries (environment, read by the setup) or
+ * for which no memory is left are applied on the FP64 pipe, and a coarsest
+ * level without them is solved by a queued loop.
  *  levels    2, 3 or 4 (Sec. IV: the recursion applies to every coarser
  *            level).
  *  block     [levels-1][2] aggregate extents: block[0] in KD blocks (even

@@ -283,6 +283,27 @@ int mg_coarsest_solve(sw_mg* mg, const double2* b, double2* x) {
 }
 
 // ---------------------------------------------------------------- setup
+// Digit entries of a level for the solves.  They are a second copy of its stencil, without
+// which coarse_op and cgne work on Y: none where the kernels cannot index them, where there
+// would be more than SW_DIGIT_ENTRIES (environment), or where the device has no memory left.
+static void make_digits(sw_mg* mg, MgLevel& L) {
+  const CoarseGeom geom{L.E0, L.E1, L.nc};
+  const long n = digit_entries(geom);
+  const char* lim = std::getenv("SW_DIGIT_ENTRIES");
+  if (n > kMaxDigitEntries || (lim && n > std::atol(lim))) return;
+  uint4* T = nullptr;
+  try {
+    T = (uint4*)mg_alloc(mg, n + (digit_rows(geom) + 3) / 4);
+  } catch (const SwError& e) {
+    if (e.code != SW_ERR_OOM) throw;
+    if (mg->verbose) std::fprintf(stderr, "[sw] no memory for digit entries: %s\n", e.msg.c_str());
+    return;
+  }
+  int* ex = (int*)(T + n);
+  launch_pack_digits(geom, L.Y, T, ex, mg->ctx->stream);
+  L.dg = DigitStencil{T, ex};
+}
+
 // The null vectors depend on every rounding of their relaxation: CG on A A^dag multiplies a
 // rounding difference about a thousandfold per step where a KD block is nearly singular
 // (|B^-1| up to 1/m), and to order one in some hundreds of steps on any field.  Eight steps at
@@ -302,8 +323,8 @@ void mg_setup(sw_mg* mg, const double* const* psi0, uint64_t seed) {
     mg->binv32 = (float2*)mg_alloc(mg, N * 2);
     launch_to_f32(mg->binv, mg->binv32, N * 4, s);
   }
-  ScopedBuffers tmp;
   for (int l = 0; l + 1 < mg->nlev; ++l) {
+    ScopedBuffers tmp;  // returned before the next level
     MgLevel& L = mg->lev[l];
     MgLevel& C = mg->lev[l + 1];
     int nv = L.nv;
@@ -401,14 +422,6 @@ void mg_setup(sw_mg* mg, const double* const* psi0, uint64_t seed) {
       double2* T = tmp.get((long)L.E0 * L.E1 * 5 * L.nc * 2 * nv);
       launch_build_Y_coarse(CoarseGeom{L.E0, L.E1, L.nc}, L.b0, L.b1, nv, L.Y, L.P, T, C.Y, s);
     }
-    const CoarseGeom geom{C.E0, C.E1, C.nc};
-    // digit entries for the solves: on the coarsest level and all levels of FP64 hierarchies
-    if ((l + 2 == mg->nlev || !mg->mixed) && digit_entries(geom) <= kMaxDigitEntries) {
-      uint4* T = (uint4*)mg_alloc(mg, digit_entries(geom));
-      int* ex = (int*)mg_alloc(mg, (digit_rows(geom) + 3) / 4);
-      launch_pack_digits(geom, C.Y, T, ex, s);
-      C.dg = DigitStencil{T, ex};
-    }
     if (mg->mixed) {
       CoarseGeom cg{C.E0, C.E1, C.nc};
       if (l + 2 < mg->nlev) {  // intermediate level: scaled FP16 copy
@@ -451,6 +464,10 @@ void mg_setup(sw_mg* mg, const double* const* psi0, uint64_t seed) {
       mg->lext = mg_alloc(mg, N);
     }
   }
+  // last, and with the setup's scratch returned: what a hierarchy can do without
+  for (int l = 1; l < mg->nlev; ++l)
+    if (l + 1 == mg->nlev || !mg->mixed) make_digits(mg, mg->lev[l]);
+  SW_CUDA(cudaStreamSynchronize(s));
 }
 
 // ================================================================ lockstep solves

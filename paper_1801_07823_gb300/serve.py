@@ -40,7 +40,9 @@ from . import sw_context_set_sm_share, sw_mg_solve, sw_mg_solve_batch
 def hierarchy_bytes(L: int, blocks, nvec, mixed: bool, outer_restart: int = 32,
                     inter_restart: int = 8) -> int:
     """Device bytes of a 3-level (or 2-level) hierarchy and its solve workspace
-    (complex128 = 16 B), from the sizes of its arrays."""
+    (complex128 = 16 B), from the sizes of its arrays.  The scratch of a setup
+    in progress (one level's null vectors, their images and up to 200 MB of
+    Krylov vectors, returned level by level) is not counted."""
     N = L * L
     b = N * 64                                     # B^-1 table
     b += N * 16 * (4 + 3)                          # fine scratch, lexicographic/parity-split copies
