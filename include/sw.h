@@ -76,7 +76,8 @@ typedef struct {
   int inter_maxiter;     /* GCR iteration cap on intermediate levels (16) */
   double inter_tol;      /* GCR relative residual on intermediate levels (0.2) */
   int coarsest_maxiter;  /* CGNE iteration cap on the coarsest level (256) */
-  double coarsest_tol;   /* CGNE relative residual on the coarsest level (0.2) */
+  double coarsest_tol;   /* CGNE relative residual on the coarsest level (0.2);
+                            negative: always coarsest_maxiter iterations */
   int precision;         /* SW_MG_FP64 (default): every operator in FP64.
                             SW_MG_MIXED: setup, Gram-Schmidt, coarse-operator build,
                             the outer FGCR (its S, residuals, restarts) and all

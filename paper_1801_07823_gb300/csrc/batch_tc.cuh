@@ -733,7 +733,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_cgne_tc(TcArgs a) {
     if (t < K) {
       const double rr0 = sm.sum[t];
       sm.rr[t] = rr0;
-      sm.stop2[t] = a.tol * a.tol * rr0;
+      sm.stop2[t] = a.tol * fabs(a.tol) * rr0;  // below 0: no residual meets it
       sm.iters[t] = 0;
       sm.state[t] = !isfinite(rr0) ? 2 : ((a.maxit <= 0 || !(rr0 > sm.stop2[t])) ? 1 : 0);
     }

@@ -261,7 +261,7 @@ __device__ void scalars(const Args& A, Shared& sh, int mode, const double* parti
   if (lane != 0) return;
   if (mode == kInit) {  // s = |b|^2
     sh.rr = s;
-    sh.stop2 = A.tol * A.tol * s;
+    sh.stop2 = A.tol * fabs(A.tol) * s;  // below 0: no residual meets it
     sh.state = !isfinite(s) ? 2 : ((A.maxit <= 0 || !(s > sh.stop2)) ? 1 : 0);
     sh.coef = 0.0;
     return;
