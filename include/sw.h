@@ -124,10 +124,11 @@ void sw_context_free(sw_ctx* ctx);
 /* Share num/den (0 < num <= den) of the GPU's SMs that the persistent
  * (cooperative, grid-synchronised) kernels of this context (the coarsest-level
  * solvers and sw_cg_eo_solve) may hold: they run with one CTA on each of
- * floor(SMs num / den) SMs (at least
- * one).  Default 1/1.  Persistent kernels of contexts of one process whose
- * shares fit the SM count together run concurrently; a launch that does not
- * fit beside the running ones waits for them (host side).  A result depends
+ * floor(SMs num / den) SMs (at least one).  Default 1/1.  Persistent kernels
+ * of contexts of one process whose shares fit the SM count together run
+ * concurrently; a launch that does not fit beside the running ones waits for
+ * them (host side), first come first served.  sw_cg_eo_solve gives its SMs
+ * back every few iterations while other calls are in flight.  A result depends
  * on the share (the grid fixes the order of its sums), not on what else runs. */
 int sw_context_set_sm_share(sw_ctx* ctx, int num, int den);
 /* Last error message of the context (never NULL; "" after success). */
@@ -229,7 +230,7 @@ int sw_mg_solve_batch(sw_mg* mg, int nrhs, const void* B, void* X, double tol, i
  * residual divided by m) or after maxiter iterations (SW_ERR_NOCONV).
  * b, x: complex128 [L1][L0].  st (may be NULL): outer_iters = CG iterations,
  * fine_applies = applications of m^2 - D_eo D_oe, true_resid recomputed.
- * The iteration is one persistent kernel (sw_context_set_sm_share).
+ * The iterations run in persistent kernels (sw_context_set_sm_share).
  * Allocates its work buffers per call.  Synchronises the stream. */
 int sw_cg_eo_solve(sw_gauge* g, double mass, const void* b, void* x, double tol, int maxiter,
                    int on_device, sw_solve_stats* st);

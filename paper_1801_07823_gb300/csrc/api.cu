@@ -9,8 +9,9 @@
 #include <atomic>
 #include <new>
 
-#include "sw_internal.h"
+#include "lease.h"
 #include "many.h"
+#include "sw_internal.h"
 #include "sw_mg.h"
 
 void report_stale_error(cudaError_t e) {
@@ -93,6 +94,8 @@ void gauge_binv(sw_gauge* g, double mass) {
 }
 
 }  // namespace
+
+void count_call(int device, int change) { SmLease::call(device, change); }
 
 static std::atomic<long long> g_launches{0};
 void sw_count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }

@@ -20,10 +20,15 @@
 //   B  q = m^2 p - D_eo t, <p, q>          -> alpha
 //   C  x += alpha p, r -= alpha q, |r|^2   -> beta, stopping test
 // Every CTA forms the two scalars from all CTAs' parts in the same order.
+//
+// A solve shares the device: it gives its SMs back when other calls are in flight (run_cg_eo).
+// Beside a CG on 256^2 a 64^2 solve takes 31 ms (alone 25.4), 34 on the CG's own stream; while
+// one launch held the SMs to the end, the solve waited for that end.
 #include <chrono>
 #include <cmath>
 #include <cstring>
 
+#include <algorithm>
 #include <atomic>
 
 #include "lease.h"
@@ -98,6 +103,18 @@ void hop_eo(const sw_gauge* g, int par, double a, const double2* src, double c, 
 constexpr int kCgThreads = 512;
 constexpr int kCgWarps = kCgThreads / 32;
 constexpr long kCgSpins = 1L << 21;
+constexpr int kCgSlots = 256;  // above the multigrid levels' 4 x 64
+constexpr int kCgKeep = 4;  // iterations of a launch before it yields its SMs
+// Iterations of a launch, 3 to 6 ms: work that other contexts queue on the stream gets its turn.
+// A launch costs about 20 us.
+// Iterations of a launch, 3 to 6 ms: work that other contexts queue on the stream gets its turn.
+// A launch costs about 20 us.
+// Whether a launch per operation on all SMs beats the persistent kernel on `sms` of them.
+// Measured, us per iteration: queued 24 + half / 8300 (64^2 24.5, 512^2 42.3, 1024^2 87,
+// 2048 x 1024 151); persistent about 10 + half / (73 sms) (256^2 on 152 / 38 / 19 / 2 SMs: 14.8 /
+// 24.4 / 37 / 225; 1024^2 on 152 / 76 / 50: 58 / 104 / 150).
+bool cg_queued(long half, int sms) { return half * (114 - sms) > 117000L * sms; }
+int cg_slice(long half) { return (int)std::min(256L, std::max(32L, (1L << 25) / half)); }
 
 struct CgArgs {
   const double2* W;
@@ -105,14 +122,17 @@ struct CgArgs {
   double2* p[2];
   double* partials;  // [2][gridDim.x]
   unsigned* bar;     // monotone arrival counter
-  int* status;       // [0] iterations, [1] barrier timeout, [2] non-finite residual
-  int L0, L1, maxit;
+  int* status;       // [0] iterations (their complement: not finished), [1] barrier timeout,
+                     // [2] non-finite residual, [3] to yield
+  const int* yield;  // host word: other calls are in flight
+  double2* state;    // |r|^2 and beta of a solve that is to go on (k0 > 0)
+  int L0, L1, k0, slice, maxit;  // iterations before this launch, of it at most, in all
   double m2, rr, stop;
 };
 struct CgShared {
   swsum::Aligned sum[kCgWarps];
   double total;
-  int ok;
+  int ok, yield;
 };
 
 // Neighbours of site h of the half of parity par: half-lattice indices of the
@@ -180,6 +200,7 @@ __device__ bool cg_barrier(const CgArgs& a, CgShared& sh, unsigned gen, double v
     }
     __threadfence();
     sh.ok = *((volatile int*)(a.status + 1)) == 0;
+    sh.yield = *((volatile int*)(a.status + 3));
   }
   if (parts) {
     __syncthreads();
@@ -192,15 +213,22 @@ __device__ bool cg_barrier(const CgArgs& a, CgShared& sh, unsigned gen, double v
   return sh.ok;
 }
 
-__global__ void __launch_bounds__(kCgThreads, 1) k_cg_eo(CgArgs a) {
+// Two CTAs' registers per SM although one runs: beside a CTA that takes most of them (104 per
+// thread without the bound, 62 with it, at the same speed) the Dslash and the coarse stencils of
+// other contexts had no room and waited for the end of the kernel.
+__global__ void __launch_bounds__(kCgThreads, 2) k_cg_eo(CgArgs a) {
   __shared__ CgShared sh;
   __shared__ double coef;
   const long N = (long)a.L0 * a.L1, half = N / 2;
   const int h0 = (int)(half * blockIdx.x / gridDim.x), h1 = (int)(half * (blockIdx.x + 1) / gridDim.x);
-  double rr = a.rr, beta = 0.0;
+  double rr = a.k0 > 0 ? a.state->x : a.rr, beta = a.k0 > 0 ? a.state->y : 0.0;
   unsigned gen = 0;
-  int k = 0;
+  int k = a.k0;
+  const bool watch = blockIdx.x == 0 && threadIdx.x == 32;
   for (;;) {
+    // one thread looks at the host word, while phase A runs, and tells all CTAs before the
+    // iteration's last barrier
+    const int want = watch ? *(const volatile int*)a.yield : 0;
     const double2* po = a.p[k & 1];
     double2* pn = a.p[(k + 1) & 1];
     for (int h = h0 + threadIdx.x; h < h1; h += kCgThreads) {
@@ -252,6 +280,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg_eo(CgArgs a) {
       a.r[h] = r;
       acc = fma(r.x, r.x, fma(r.y, r.y, acc));
     }
+    if (want) a.status[3] = 1;
     if (!cg_barrier(a, sh, ++gen, acc, a.partials + gridDim.x)) return;
     ++k;
     const double rn = sh.total;
@@ -266,13 +295,22 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg_eo(CgArgs a) {
     __syncthreads();
     beta = coef;
     rr = rn;
+    if (k - a.k0 >= (sh.yield ? kCgKeep : a.slice)) {
+      if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.status[0] = ~k;
+        *a.state = make_double2(rr, beta);
+      }
+      return;
+    }
   }
 }
 
-// Runs CG from the residual a.r (rr = |r|^2) for at most a.maxit iterations; returns them.
+// The persistent kernel from the residual a.r (rr = |r|^2), for at most a.maxit iterations;
+// returns them.  The SMs are given back and asked for again after a slice, and every kCgKeep
+// iterations while other calls are in flight: the solve goes on from x, r, p, |r|^2 and beta,
+// with the same bits.
 int run_cg_eo(sw_ctx* c, CgArgs a) {
   static std::atomic<bool> checked[64];
-  SmLease lease(c);  // held until the kernel has finished
   if (!checked[c->device & 63].load()) {
     int coop = 0, occ = 0;
     SW_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device));
@@ -280,25 +318,32 @@ int run_cg_eo(sw_ctx* c, CgArgs a) {
     SW_REQUIRE(coop && occ >= 1, SW_ERR_CUDA, "the device cannot run the persistent CG kernel");
     checked[c->device & 63].store(true);
   }
-  // one CTA per SM; fewer where a CTA would have less than a warp of sites
-  const long half = (long)a.L0 * a.L1 / 2;
-  long grid = (half + 31) / 32;
-  if (grid > lease.sms()) grid = lease.sms();
-  if (grid > kReduceBlocks) grid = kReduceBlocks;
   a.partials = c->partials;
   a.bar = c->bar;
   a.status = c->cgstat;
-  SW_CUDA(cudaMemsetAsync(a.bar, 0, 2 * sizeof(unsigned), c->stream));
-  SW_CUDA(cudaMemsetAsync(a.status, 0, 3 * sizeof(int), c->stream));
-  void* params[] = {&a};
-  SW_CUDA(cudaLaunchCooperativeKernel((const void*)k_cg_eo, dim3((unsigned)grid), dim3(kCgThreads),
-                                      params, 0, c->stream));
-  sw_count_launch();
-  SW_CUDA(cudaMemcpyAsync(c->h_ctl, c->cgstat, 3 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  SW_CUDA(cudaStreamSynchronize(c->stream));
-  if (c->h_ctl[1]) throw SwError{SW_ERR_TIMEOUT, "even/odd CG: a grid barrier wait gave up"};
-  if (c->h_ctl[2]) throw SwError{SW_ERR_NAN, "non-finite CG residual"};
-  return c->h_ctl[0];
+  a.yield = &c->h_many->yield;
+  a.state = c->slots + kCgSlots + 5;
+  const long half = (long)a.L0 * a.L1 / 2;
+  a.slice = cg_slice(half);
+  int* h = c->h_ctl;
+  for (a.k0 = 0;; a.k0 = ~h[0]) {
+    SmLease lease(c, &c->h_many->yield);  // held until the kernel has finished
+    // one CTA per SM; fewer where a CTA would have less than a warp of sites
+    long grid = (half + 31) / 32;
+    if (grid > lease.sms()) grid = lease.sms();
+    if (grid > kReduceBlocks) grid = kReduceBlocks;
+    SW_CUDA(cudaMemsetAsync(a.bar, 0, 2 * sizeof(unsigned), c->stream));
+    SW_CUDA(cudaMemsetAsync(a.status, 0, 4 * sizeof(int), c->stream));
+    void* params[] = {&a};
+    SW_CUDA(cudaLaunchCooperativeKernel((const void*)k_cg_eo, dim3((unsigned)grid),
+                                        dim3(kCgThreads), params, 0, c->stream));
+    sw_count_launch();
+    SW_CUDA(cudaMemcpyAsync(h, c->cgstat, 4 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    SW_CUDA(cudaStreamSynchronize(c->stream));
+    if (h[1]) throw SwError{SW_ERR_TIMEOUT, "even/odd CG: a grid barrier wait gave up"};
+    if (h[2]) throw SwError{SW_ERR_NAN, "non-finite CG residual"};
+    if (h[0] >= 0) return h[0];
+  }
 }
 
 }  // namespace
@@ -316,7 +361,7 @@ int cg_eo_device(sw_gauge* g, double m, const double2* b, double2* x, double tol
   int blocks = (int)((N + 255) / 256);
   k_split_eo<<<blocks, 256, 0, s>>>(b, be, bo, g->L0, g->L1);
   SW_LAUNCH_CHECK();
-  int sb = 256;  // slots of this solver (above the multigrid levels' 4 x 64)
+  constexpr int sb = kCgSlots;
   blas_norm2(c, b, N, sb + 0);
   double bn = std::sqrt(slot_read(c, sb + 0).x);
   if (!std::isfinite(bn)) throw SwError{SW_ERR_NAN, "non-finite right-hand side"};
@@ -369,6 +414,7 @@ extern "C" int sw_cg_eo_solve(sw_gauge* g, double mass, const void* b, void* x, 
                               int maxiter, int on_device, sw_solve_stats* st) {
   if (!g || !b || !x) return SW_ERR_ARG;
   sw_ctx* c = g->ctx;
+  const CallScope scope(c);
   try {
     c->err.clear();
     SW_CUDA(cudaSetDevice(c->device));

@@ -125,6 +125,7 @@ struct HostMany {
   double2* ptr[2 * kMaxBatch];     // b and x of a batched coarsest solve
   int ctl[4 * kMaxBatch];
   int status[2 + kMaxBatch];
+  int yield;                       // of the SM lease of a CG (lease.h)
 };
 
 struct sw_ctx {
@@ -144,7 +145,7 @@ struct sw_ctx {
   unsigned long long* exec = nullptr;  // device count of executed (not skipped) timed kernels
   int* h_ctl = nullptr;          // pinned host mirror of one control block
   unsigned* bar = nullptr;       // grid-barrier state of persistent kernels (2 words)
-  int* cgstat = nullptr;         // status words of the persistent CGNE (3 ints)
+  int* cgstat = nullptr;         // status words of the persistent kernels (4 ints)
   double2* h_slots = nullptr;    // pinned host mirror
   double* many_partials = nullptr;    // device [kMaxBatch][kManyBlocks][4], sums of many.cu
   unsigned* many_counters = nullptr;  // device [kMaxBatch]
@@ -173,8 +174,20 @@ inline int fail(sw_ctx* c, int code, const std::string& msg) {
   if (c) c->err = msg;
   return code;
 }
+// A library call in flight on a context's device (lease.h).
+void count_call(int device, int change);
+struct CallScope {
+  int device;
+  explicit CallScope(const sw_ctx* c) : device(c ? c->device : -1) {
+    if (device >= 0) count_call(device, 1);
+  }
+  ~CallScope() {
+    if (device >= 0) count_call(device, -1);
+  }
+};
 template <typename F>
 int guarded(sw_ctx* c, F&& f) {
+  const CallScope scope(c);
   try {
     if (c) {
       c->err.clear();

@@ -1,0 +1,60 @@
+"""Even/odd CG beside other contexts."""
+import threading
+import time
+
+import numpy as np
+import pytest
+
+import sw_inputs as si
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sw():
+    import paper_1801_07823_gb300 as m
+    return m
+
+
+@pytest.mark.parametrize("own_streams", [False, True])
+def test_solves_advance_beside_cg(sw, own_streams):
+    """Several multigrid solves of another context, whose coarsest kernels want all SMs too, finish
+    while a CG of 20000 iterations runs (a quarter of a second by itself, ten solves long), and
+    the CG's result has the bits it has alone."""
+    import torch
+    from oracle import operators
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    made = []
+    for k, L in ((0, 256), (1, 64)):
+        ctx = sw.sw_context_create(0, streams[k].cuda_stream if own_streams else None)
+        th = si.heatbath_u1(L, L, 6.0, 10, seed=k, device="cuda")
+        made.append((ctx, sw.sw_gauge_load(ctx, th), th, si.gaussian_complex(k, L * L)))
+    (c1, g1, _, b1), (c2, g2, th2, b2) = made
+    h = sw.sw_mg_setup(g2, 0.01, 3, [(4, 4), (2, 2)], [8, 12], seed=3)
+    x2 = np.zeros_like(b2)
+    sw.sw_mg_solve(h, b2, x2, 1e-10)
+    out = [np.zeros_like(b1), np.zeros_like(b1)]
+
+    def cg(x):
+        st = sw.sw_cg_eo_solve(g1, 1e-3, b1, x, 1e-15, 20000, allow_noconv=True)
+        assert st["outer_iters"] == 20000
+
+    cg(out[0])
+    t = threading.Thread(target=cg, args=(out[1],))
+    t.start()
+    time.sleep(0.02)
+    done = 0
+    while t.is_alive() and done < 5:
+        x = np.zeros_like(b2)
+        sw.sw_mg_solve(h, b2, x, 1e-10)
+        assert np.array_equal(x, x2)
+        done += t.is_alive()
+    t.join()
+    assert done >= 3
+    assert np.array_equal(out[0], out[1])
+    r = b2 - operators.dirac(th2, 0.01) @ x2
+    assert np.linalg.norm(r) <= 1e-10 * np.linalg.norm(b2)
+    h.free()
+    for c, g, *_ in made:
+        g.free()
+        c.free()
