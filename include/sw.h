@@ -128,7 +128,9 @@ void sw_context_free(sw_ctx* ctx);
  * of contexts of one process whose shares fit the SM count together run
  * concurrently; a launch that does not fit beside the running ones waits for
  * them (host side), first come first served.  sw_cg_eo_solve gives its SMs
- * back every few iterations while other calls are in flight.  A result depends
+ * back every few iterations while other calls are in flight, and where the
+ * share is too small for the lattice it runs a kernel per operation on all SMs
+ * instead, without waiting for anyone.  A result depends
  * on the share (the grid fixes the order of its sums), not on what else runs. */
 int sw_context_set_sm_share(sw_ctx* ctx, int num, int den);
 /* Last error message of the context (never NULL; "" after success). */

@@ -23,7 +23,9 @@
 //
 // A solve shares the device: it gives its SMs back when other calls are in flight (run_cg_eo).
 // Beside a CG on 256^2 a 64^2 solve takes 31 ms (alone 25.4), 34 on the CG's own stream; while
-// one launch held the SMs to the end, the solve waited for that end.
+// one launch held the SMs to the end, the solve waited for that end.  A context with too small
+// a share of the SMs for its lattice queues a launch per operation on all of them instead
+// (cg_queued).
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -32,6 +34,7 @@
 #include <atomic>
 
 #include "lease.h"
+#include "many.h"
 #include "sums.cuh"
 
 namespace {
@@ -105,8 +108,6 @@ constexpr int kCgWarps = kCgThreads / 32;
 constexpr long kCgSpins = 1L << 21;
 constexpr int kCgSlots = 256;  // above the multigrid levels' 4 x 64
 constexpr int kCgKeep = 4;  // iterations of a launch before it yields its SMs
-// Iterations of a launch, 3 to 6 ms: work that other contexts queue on the stream gets its turn.
-// A launch costs about 20 us.
 // Iterations of a launch, 3 to 6 ms: work that other contexts queue on the stream gets its turn.
 // A launch costs about 20 us.
 // Whether a launch per operation on all SMs beats the persistent kernel on `sms` of them.
@@ -305,6 +306,40 @@ __global__ void __launch_bounds__(kCgThreads, 2) k_cg_eo(CgArgs a) {
   }
 }
 
+// CG from the residual a.r (|r|^2 in slot kCgSlots + 1) for at most a.maxit iterations, a launch
+// per operation, eight iterations queued at a time, on all SMs and without a lease.  Returns
+// the iterations.
+int run_cg_queued(sw_gauge* g, const CgArgs& a) {
+  sw_ctx* c = g->ctx;
+  cudaStream_t s = c->stream;
+  const long h = g->N / 2;
+  constexpr int s_pq = 3, s_stop = 5, kQueue = 8;
+  int s_rr[2] = {1, 2};
+  double2* p = a.p[1];
+  int* ctl = c->many_ctl;
+  c->h_slots[kCgSlots + s_stop] = make_double2(a.stop, 0.0);
+  SW_CUDA(cudaMemcpyAsync(c->slots + kCgSlots + s_stop, c->h_slots + kCgSlots + s_stop,
+                          sizeof(double2), cudaMemcpyHostToDevice, s));
+  SW_CUDA(cudaMemsetAsync(ctl, 0, 4 * sizeof(int), s));
+  blas_copy(c, p, a.r, h);
+  const int* done = c->h_many->ctl;
+  for (int issued = 0;;) {
+    for (int q = 0; q < kQueue && issued < a.maxit; ++q, ++issued) {
+      hop_eo(g, 1, 0.0, nullptr, 1.0, p, a.t, s);  // t_o = D_oe p
+      hop_eo(g, 0, a.m2, p, -1.0, a.t, a.q, s);    // q = m^2 p - D_eo t
+      many_setup_dot(c, h, Many<2>(kCgSlots, p, a.q), s_pq, ctl);
+      many_cg_step(c, h, Many<4>(kCgSlots, a.x, a.r, p, a.q), s_rr[0], s_pq, s_rr[1], s_stop,
+                   a.maxit, ctl);
+      many_xpay(c, h, Many<2>(kCgSlots, p, a.r), s_rr[1], s_rr[0], ctl);
+      std::swap(s_rr[0], s_rr[1]);
+    }
+    SW_CUDA(cudaMemcpyAsync(c->h_many->ctl, ctl, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    SW_CUDA(cudaStreamSynchronize(s));
+    if (done[2]) throw SwError{SW_ERR_NAN, "non-finite CG residual"};
+    if (done[0]) return done[1];
+  }
+}
+
 // The persistent kernel from the residual a.r (rr = |r|^2), for at most a.maxit iterations;
 // returns them.  The SMs are given back and asked for again after a slice, and every kCgKeep
 // iterations while other calls are in flight: the solve goes on from x, r, p, |r|^2 and beta,
@@ -369,7 +404,9 @@ int cg_eo_device(sw_gauge* g, double m, const double2* b, double2* x, double tol
   hop_eo(g, 0, m, be, -1.0, bo, be, s);
   blas_zero(c, xe, h);
   double stop = bn > 0.0 ? tol * m * bn : 0.0;
-  int total = 0;
+  int total = 0, sms = 0;
+  SW_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
+  const bool queued = cg_queued(h, SmLease::share(c, sms));
   // CG with reliable restarts: when the recurrence residual meets the target,
   // the true residual rhs - M x_e is recomputed; if it is still above the
   // target (recurrence drift at small m), CG restarts from it.
@@ -395,7 +432,7 @@ int cg_eo_device(sw_gauge* g, double m, const double2* b, double2* x, double tol
     a.m2 = m * m;
     a.rr = rr0;
     a.stop = stop;
-    total += run_cg_eo(c, a);
+    total += queued ? run_cg_queued(g, a) : run_cg_eo(c, a);
   }
   *iters = total;
   // x_o = (b_o - D_oe x_e) / m

@@ -1,4 +1,4 @@
-"""Even/odd CG beside other contexts."""
+"""Even/odd CG beside other contexts, and on a small share of the SMs."""
 import threading
 import time
 
@@ -58,3 +58,55 @@ def test_solves_advance_beside_cg(sw, own_streams):
     for c, g, *_ in made:
         g.free()
         c.free()
+
+
+def test_small_share(sw):
+    """A sixteenth of the SMs: the iteration on 512^2 takes no more than four times the full
+    device's (a kernel per operation 1.7 times; the persistent kernel on nine SMs takes eight)."""
+    L, n = 512, 400
+    th = si.heatbath_u1(L, L, 6.0, 5, seed=1, device="cuda")
+    b = si.gaussian_complex(1, L * L)
+    took = []
+    for den in (1, 16):
+        ctx = sw.sw_context_create(0)
+        sw.sw_context_set_sm_share(ctx, 1, den)
+        g = sw.sw_gauge_load(ctx, th)
+        x = np.zeros_like(b)
+        sw.sw_cg_eo_solve(g, 1e-3, b, x, 1e-15, 8, allow_noconv=True)
+        best = 1e9
+        for _ in range(3):
+            its = []
+            for k in (n, 3 * n):
+                t0 = time.perf_counter()
+                st = sw.sw_cg_eo_solve(g, 1e-3, b, x, 1e-15, k, allow_noconv=True)
+                its.append(time.perf_counter() - t0)
+                assert st["outer_iters"] == k
+            best = min(best, its[1] - its[0])
+        took.append(best)
+        g.free()
+        ctx.free()
+    assert took[1] <= 4 * took[0]
+
+
+@pytest.mark.parametrize("L0,L1", [(128, 96), (256, 128)])
+def test_queued_form(sw, L0, L1):
+    """A lattice too large for one SM: caps, convergence by the oracle's D, NaN."""
+    from oracle import operators
+    m = 0.05
+    th = si.heatbath_u1(L0, L1, 6.0, 10, seed=3, device="cuda")
+    ctx = sw.sw_context_create(0)
+    sw.sw_context_set_sm_share(ctx, 1, 152)
+    g = sw.sw_gauge_load(ctx, th)
+    b = si.gaussian_complex(7, L0 * L1)
+    D = operators.dirac(th, m)
+    for cap in (1, 8, 9, 100000):
+        x = np.zeros_like(b)
+        st = sw.sw_cg_eo_solve(g, m, b, x, 1e-10, cap, allow_noconv=True)
+        r = np.linalg.norm(b - D @ x) / np.linalg.norm(b)
+        assert st["outer_iters"] <= cap and abs(r - st["true_resid"]) <= 1e-12
+    assert st["converged"] and r <= 1e-10
+    b[3] = np.nan
+    with pytest.raises(sw.SwError):
+        sw.sw_cg_eo_solve(g, m, b, x, 1e-10)
+    g.free()
+    ctx.free()
