@@ -160,7 +160,14 @@ void sw_gauge_free(sw_gauge* g);
  *             hops always leave the block, so B_Naik = B with hops x 9/8).
  * precision: SW_PREC_FP64 (complex128 buffers) or SW_PREC_FP32 (complex64
  * buffers; SW_OP_D and SW_OP_DDAG only).  mass must be > 0 for A, ADAG, S,
- * ANAIK.  The Naik ops build the long links (and B_Naik^-1) on first use. */
+ * ANAIK.  The Naik ops build the long links (and B_Naik^-1) on first use.
+ * FP64 D and D^dag: half of the sites (alternating in groups of 128 along x0
+ * and from row to row) add their hops up as integers, cut to 2^-58 of the
+ * largest component among the four neighbours and rounded once.  For
+ * components of similar size that is closer than a chain of FMAs; smaller ones
+ * lose what lies below that cut (on real links, an imaginary part 2^-58 below
+ * the real one), and D of a translated field equals the translate up to
+ * rounding only. */
 int sw_dslash(sw_gauge* g, double mass, int op, int precision, const void* in, void* out,
               int on_device);
 
@@ -277,6 +284,15 @@ int sw_mg_export_Y(sw_mg* mg, int level, double* Y);
  *   SW_PREC_FP64, or in the reduced copy a mixed hierarchy keeps for that
  *   level (SW_PREC_FP16S on intermediate levels, SW_PREC_DF64 on the
  *   coarsest).  Synchronises the stream.
+ *   FP64 on a level with digit entries (sw_mg_setup) forms products in fixed
+ *   point: an entry keeps 63 bits below the largest component of its row, a
+ *   vector component 62 below the largest of the five sites (dagger: after its
+ *   multiplication with the row's power of two), and a component of the result
+ *   is off by at most 10 nc 2^-58 of the product of the two scales, and by its
+ *   own rounding.  That is below the error of FP64 sums for rows and vectors
+ *   whose parts are of similar size (Galerkin stencils on Gaussian, smooth and
+ *   localised vectors: 2 to 10 times); entries and elements 2^-k below their
+ *   largest keep 63 - k and 62 - k bits.
  * sw_mg_transfer: dir = 0 restriction out = P^dag in from level l to l + 1;
  *   dir = 1 prolongation out = P in from level l + 1 to level l.  On level 1
  *   both act on the even KD-block sites only, as inside the solver (Sec. IV:

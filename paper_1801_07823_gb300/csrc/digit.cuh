@@ -11,14 +11,17 @@
 // Numer. Algorithms 59 (2012).)
 //
 // Numbers.  A row of A is scaled by the power of two of its largest component
-// and rounded to 64 bits (u_0 - 128, u_1, .., u_7), u unsigned bytes; the vectors of a site's five neighbours share one power of two and are
-// rounded to 63 bits in balanced digits d_0 .. d_7 in [-128, 127].  Of the 64
+// and rounded to 64 bits (u_0 - 128, u_1, .., u_7), u unsigned bytes; the
+// vectors of a site's five neighbours share one power of two and are rounded to 63 bits in balanced digits d_0 .. d_7 in [-128, 127].  Of the 64
 // digit products those of level i + j <= 7 are kept; the others are below
 // 2^-59 of the largest product.  Against exact arithmetic the products are 2
 // to 10 times closer than the FP64 kernels they take the place of (the
 // operands' rounding is below FP64's accumulated rounding): measured on Galerkin
 // stencils with Gaussian, smooth and localised vectors, relative 2-norm error
-// 0.4e-16 to 0.8e-16 against 1.0e-16 to 5.9e-16.
+// 0.4e-16 to 0.8e-16 against 1.0e-16 to 5.9e-16.  Fixed point has a range: an entry 2^-k
+// below its row's largest keeps 64 - k bits, a vector element 63 - k, so that rows and vectors
+// graded against each other (large entries on small elements) lose what FP64 would keep; the
+// error bound is one of the two scales, not of every term.
 //
 // MMA shape.  mma.m16n8k16 with M = the real and imaginary parts of eight
 // output rows, N = the eight levels, K = four entries times four digits: the
