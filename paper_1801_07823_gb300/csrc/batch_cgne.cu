@@ -67,18 +67,6 @@ struct Tile {
   static_assert(kS * K * 4 <= kThreads, "per-site norm tree needs four threads per pair");
 };
 
-__device__ __forceinline__ int nbr(int X, int d, int E0, int E1) {
-  int X0 = X % E0, X1 = X / E0;
-  if (d == 1) X0 = (X0 + 1 == E0) ? 0 : X0 + 1;
-  if (d == 2) X0 = (X0 == 0) ? E0 - 1 : X0 - 1;
-  if (d == 3) X1 = (X1 + 1 == E1) ? 0 : X1 + 1;
-  if (d == 4) X1 = (X1 == 0) ? E1 - 1 : X1 - 1;
-  return X0 + E0 * X1;
-}
-__device__ __forceinline__ int opp(int d) {
-  return d == 0 ? 0 : (d == 1 ? 2 : (d == 2 ? 1 : (d == 3 ? 4 : 3)));
-}
-
 // ------------------------------------------------ mbarrier and bulk copies
 __device__ __forceinline__ unsigned su32(const void* p) {
   return static_cast<unsigned>(__cvta_generic_to_shared(p));

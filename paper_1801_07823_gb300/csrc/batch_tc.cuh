@@ -221,18 +221,6 @@ __device__ __forceinline__ void tmem_ld16(unsigned taddr, float* v) {
   for (int c = 0; c < 16; ++c) v[c] = __uint_as_float(r[c]);
 }
 
-__device__ __forceinline__ int nbr(int X, int d, int E0, int E1) {
-  int X0 = X % E0, X1 = X / E0;
-  if (d == 1) X0 = (X0 + 1 == E0) ? 0 : X0 + 1;
-  if (d == 2) X0 = (X0 == 0) ? E0 - 1 : X0 - 1;
-  if (d == 3) X1 = (X1 + 1 == E1) ? 0 : X1 + 1;
-  if (d == 4) X1 = (X1 == 0) ? E1 - 1 : X1 - 1;
-  return X0 + E0 * X1;
-}
-__device__ __forceinline__ int opp(int d) {
-  return d == 0 ? 0 : (d == 1 ? 2 : (d == 2 ? 1 : (d == 3 ? 4 : 3)));
-}
-
 // Byte offset of element (row, k) in a K-major no-swizzle tile with `rows`
 // rows: core matrix (row / 8, k / 4) at (k / 4 * rows / 8 + row / 8) * 128.
 __host__ __device__ __forceinline__ unsigned tile_off(int row, int k, int rows) {
@@ -324,9 +312,10 @@ static __device__ bool grid_barrier_tc(unsigned* bar, int* status, unsigned gen)
 // Sums over the CTAs, a warp per right-hand side, in the same order in every CTA.  Two of the
 // warps share a quarter of the SM, whose FP64 addition takes 64 clocks: a tree of shuffles
 // and FP64 additions over eight loads kept it busy for 3300 clocks a phase at K = 16.  Here a
-// lane adds only the parts that exist (64 CTAs: two) and the warp adds aligned mantissas.
-// 16 right-hand sides at 8^2 x 64: 18.6 -> 18.4 us per iteration, with a barrier that polls
-// without sleeping.
+// lane adds only the parts that exist (152 CTAs: five) and the warp adds aligned mantissas.
+// With a barrier that polls without sleeping, us per iteration with FP32 iterates (repeats within
+// 0.02): 8^2 x 64, K = 8 / 16 / 32 16.61 / 19.62 / 24.99 -> 16.14 / 19.21 / 24.20; 16^2 x 64,
+// K = 16 / 64 26.82 / 48.21 -> 26.60 / 46.74.
 template <int K>
 __device__ void grid_sums_tc(const double* part, double* out) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;

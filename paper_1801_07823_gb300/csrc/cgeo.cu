@@ -108,13 +108,13 @@ constexpr int kCgWarps = kCgThreads / 32;
 constexpr long kCgSpins = 1L << 21;
 constexpr int kCgSlots = 256;  // above the multigrid levels' 4 x 64
 constexpr int kCgKeep = 4;  // iterations of a launch before it yields its SMs
-// Iterations of a launch, 3 to 6 ms: work that other contexts queue on the stream gets its turn.
-// A launch costs about 20 us.
 // Whether a launch per operation on all SMs beats the persistent kernel on `sms` of them.
 // Measured, us per iteration: queued 24 + half / 8300 (64^2 24.5, 512^2 42.3, 1024^2 87,
 // 2048 x 1024 151); persistent about 10 + half / (73 sms) (256^2 on 152 / 38 / 19 / 2 SMs: 14.8 /
 // 24.4 / 37 / 225; 1024^2 on 152 / 76 / 50: 58 / 104 / 150).
 bool cg_queued(long half, int sms) { return half * (114 - sms) > 117000L * sms; }
+// Iterations of a launch, 3 to 6 ms: work that other contexts queue on the stream gets its turn.
+// A launch costs about 20 us.
 int cg_slice(long half) { return (int)std::min(256L, std::max(32L, (1L << 25) / half)); }
 
 struct CgArgs {

@@ -31,6 +31,7 @@
 
 namespace {
 
+
 constexpr long kSpinLimit = 1L << 24;    // ~0.3-1.5 s of polling
 
 // Double-float ("df64") arithmetic on the FP32 pipes (Dekker 1971; Knuth's
@@ -70,18 +71,6 @@ __device__ __forceinline__ void df_cmac(df2& re, df2& im, float4 a, float4 b) {
     df_mac(im, a.x, a.y, b.z, b.w);
     df_mac(im, -a.z, -a.w, b.x, b.y);
   }
-}
-
-__device__ __forceinline__ int nbr(int X, int d, int E0, int E1) {
-  int X0 = X % E0, X1 = X / E0;
-  if (d == 1) X0 = (X0 + 1 == E0) ? 0 : X0 + 1;
-  if (d == 2) X0 = (X0 == 0) ? E0 - 1 : X0 - 1;
-  if (d == 3) X1 = (X1 + 1 == E1) ? 0 : X1 + 1;
-  if (d == 4) X1 = (X1 == 0) ? E1 - 1 : X1 - 1;
-  return X0 + E0 * X1;
-}
-__device__ __forceinline__ int opp(int d) {
-  return d == 0 ? 0 : (d == 1 ? 2 : (d == 2 ? 1 : (d == 3 ? 4 : 3)));
 }
 
 struct CgneArgs {

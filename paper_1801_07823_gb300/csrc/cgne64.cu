@@ -6,8 +6,8 @@
 // grid barrier; P2 p = A^dag r + beta p, |p|^2; grid barrier.
 //
 // Work.  One CTA of 12 warps per SM.  A CTA owns a contiguous run of items (eight
-// rows of one site; pairs of them where that leaves enough for every SM), so that its entries, rows and vectors are the same ones
-// in every iteration, and what can be worked out once (offsets, shares, row
+// rows of one site; pairs of them where that leaves enough for every SM), so that
+// its entries, rows and vectors are the same ones in every iteration, and what can be worked out once (offsets, shares, row
 // exponents) is kept in shared memory.  Per phase eleven warps write the digits of
 // the sites' neighbour vectors to shared memory while the last one adds up
 // the previous phase's norm parts and forms alpha or beta, which are needed only
@@ -23,7 +23,7 @@
 // Measured, microseconds per iteration, against the FP64-pipe kernel this one
 // took the place of: 28.4 against 73.3 at 16^2 sites x 64 dof, 16.2 against 28.7
 // at 8^2 x 64, 9.9 against 16.6 at 4^2 x 24.  At 16^2 x 64 the 84 MB of entries
-// stay in the L2 (ncu: 95 % hits), and a phase spends 6 us in the products (a
+// stay in the L2 (ncu: 97 % hits), and a phase spends 6 us in the products (a
 // k-step of eight rows takes about 190 clocks of its sub-partition, of which the
 // twelve MMAs need 104), 1 us each in reading and splitting the vectors, in the
 // update, and in the norm with its fence, and 1 us in the barrier; at 4^2 x 24
@@ -46,11 +46,12 @@
 #include <algorithm>
 #include <atomic>
 
-#include "digit.cuh"
+#include "sums.cuh"
 
 namespace {
 
 using namespace swdig;
+using namespace swsum;
 
 constexpr long kSpinLimit = 1L << 21;
 constexpr int kThreads = 384;
@@ -81,44 +82,6 @@ struct Args {
 };
 
 enum { kInit = 0, kP1 = 1, kP2 = 2 };
-
-// Sum over a warp of non-negative doubles, one per lane, as s 2^(e - 1080):
-// mantissas aligned to the largest, rounded to 58 bits and added as integers.
-// An FP64 addition takes 64 clocks on this device and a warp's tree of them five
-// of those and ten shuffles; the aligned sum is also the closer one (32
-// roundings of at most 2^-59 of the largest value against five of 2^-53 of
-// the sum).  e = 2047: not finite.
-struct Aligned {
-  unsigned long long s;
-  int e;
-};
-__device__ __forceinline__ Aligned warp_sum(double v) {
-  Aligned a;
-  a.e = __reduce_max_sync(0xffffffffu, expo(v));
-  const unsigned long long m = (unsigned long long)fixed(v, 0, a.e, 5);
-  const unsigned l0 = __reduce_add_sync(0xffffffffu, (unsigned)m & 0x1fffffu);
-  const unsigned l1 = __reduce_add_sync(0xffffffffu, (unsigned)(m >> 21) & 0x1fffffu);
-  const unsigned l2 = __reduce_add_sync(0xffffffffu, (unsigned)(m >> 42));
-  a.s = l0 + ((unsigned long long)l1 << 21) + ((unsigned long long)l2 << 42);
-  return a;
-}
-// Sum of n of them, n <= 16.
-template <int n>
-__device__ __forceinline__ double total(const Aligned* a) {
-  int e = 1;
-#pragma unroll
-  for (int k = 0; k < n; ++k) e = max(e, a[k].e);
-  if (e == 2047) return __longlong_as_double(0x7ff8000000000000ll);
-  long long H = 0, M = 0;  // the sum is (H 2^32 + M) 2^(e - 1104); H < 16 2^55
-#pragma unroll
-  for (int k = 0; k < n; ++k) {
-    const int sh = e - a[k].e + 8;
-    if (sh >= 96) continue;
-    H += sh < 64 ? (long long)(a[k].s >> sh) : 0;
-    M += (unsigned)(sh < 32 ? a[k].s << (32 - sh) : a[k].s >> (sh - 32));
-  }
-  return to_double(H, M, e - 1104);
-}
 
 struct Shared {
   Aligned sum[kWarps];
@@ -243,21 +206,13 @@ __device__ __forceinline__ void bar_arrive(int id, int threads) {
 template <bool CLUSTER>
 __device__ void scalars(const Args& A, Shared& sh, int mode, const double* partials, int k) {
   const int lane = threadIdx.x & 31, G = gridDim.x;
-  constexpr int kLoads = CLUSTER ? 1 : 5;
-  const auto ld_part = [](const double* p) { return CLUSTER ? *p : __ldcg(p); };
-  double s = 0.0;
-  for (int q0 = 0; q0 < G; q0 += 32 * kLoads) {
-    double v[kLoads];
-#pragma unroll
-    for (int j = 0; j < kLoads; ++j) {
-      const int q = q0 + 32 * j + lane;
-      v[j] = q < G ? ld_part(partials + q) : 0.0;
-    }
-#pragma unroll
-    for (int j = 0; j < kLoads; ++j) s += v[j];
+  double s;
+  if (CLUSTER) {
+    const Aligned a = warp_sum(lane < G ? partials[lane] : 0.0);
+    s = total<1>(&a);
+  } else {
+    s = grid_total(partials, G);
   }
-  const Aligned a = warp_sum(s);
-  s = total<1>(&a);
   if (lane != 0) return;
   if (mode == kInit) {  // s = |b|^2
     sh.rr = s;

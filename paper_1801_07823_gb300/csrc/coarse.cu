@@ -31,20 +31,6 @@ __device__ __forceinline__ void cfmac(double2& acc, double2 a, double2 b) {  // 
   acc.y = fma(a.x, b.y, acc.y);
   acc.y = fma(-a.y, b.x, acc.y);
 }
-__host__ __device__ __forceinline__ int nbr_site(int X, int d, int E0, int E1) {
-  int X0 = X % E0, X1 = X / E0;
-  switch (d) {
-    case 1: X0 = (X0 + 1 == E0) ? 0 : X0 + 1; break;
-    case 2: X0 = (X0 == 0) ? E0 - 1 : X0 - 1; break;
-    case 3: X1 = (X1 + 1 == E1) ? 0 : X1 + 1; break;
-    case 4: X1 = (X1 == 0) ? E1 - 1 : X1 - 1; break;
-    default: break;
-  }
-  return X0 + E0 * X1;
-}
-__host__ __device__ __forceinline__ int opp_dir(int d) {
-  return d == 0 ? 0 : (d == 1 ? 2 : (d == 2 ? 1 : (d == 3 ? 4 : 3)));
-}
 inline int cdiv(long a, long b) { return (int)((a + b - 1) / b); }
 
 // ---------------------------------------------------------------------------
@@ -69,7 +55,7 @@ __global__ void k_coarse_apply(const double2* __restrict__ Y, Pack<2, W> io, int
     int r = t - ls * 5 * nc;
     int d = r / nc, j = r - d * nc;
     int X = site0 + ls;
-    if (X < nsites) xs[t] = in[(long)nbr_site(X, d, E0, E1) * nc + j];
+    if (X < nsites) xs[t] = in[(long)nbr(X, d, E0, E1) * nc + j];
   }
   __syncthreads();
   int ls = threadIdx.x / nc, i = threadIdx.x - ls * nc;
@@ -82,7 +68,7 @@ __global__ void k_coarse_apply(const double2* __restrict__ Y, Pack<2, W> io, int
     for (int dj = 0; dj < 5 * nc; ++dj) cfma(acc, __ldg(y + (long)dj * nc), xv[dj]);
   } else {
     for (int d = 0; d < 5; ++d) {
-      const double2* y = Y + (((long)nbr_site(X, d, E0, E1) * 5 + opp_dir(d)) * nc + i) * nc;
+      const double2* y = Y + (((long)nbr(X, d, E0, E1) * 5 + opp(d)) * nc + i) * nc;
       for (int j = 0; j < nc; ++j) cfmac(acc, __ldg(y + j), xv[d * nc + j]);
     }
   }
@@ -115,7 +101,7 @@ __global__ void __launch_bounds__(5 * NC) k_coarse_apply_nc(const double2* __res
   int nthr = 5 * rows;
   for (int t = threadIdx.x; t < 5 * NC; t += nthr) {
     int d = t / NC, j = t - d * NC;
-    xs[d][j] = in[(long)nbr_site(X, d, E0, E1) * NC + j];
+    xs[d][j] = in[(long)nbr(X, d, E0, E1) * NC + j];
   }
   __syncthreads();
   int d = threadIdx.x / rows;
@@ -129,7 +115,7 @@ __global__ void __launch_bounds__(5 * NC) k_coarse_apply_nc(const double2* __res
     // (A^dag)(X, X+d) = Y[X+d][opp d]^dag: row i of it is column i of that
     // block, contiguous in memory (each thread streams its own column; the
     // warp's lines are reused from L1 over consecutive j)
-    const double2* y = Y + (((long)nbr_site(X, d, E0, E1) * 5 + opp_dir(d)) * NC + i) * NC;
+    const double2* y = Y + (((long)nbr(X, d, E0, E1) * 5 + opp(d)) * NC + i) * NC;
 #pragma unroll 16
     for (int j = 0; j < NC; ++j) cfmac(acc, __ldg(y + j), xs[d][j]);
   }
@@ -473,7 +459,7 @@ __global__ void k_build_T(const double2* __restrict__ Y, const double2* __restri
   int d = (int)(t % 5);
   int x = (int)(t / 5);
   int c = col / nv, i = col - c * nv;
-  int xn = nbr_site(x, d, E0, E1);
+  int xn = nbr(x, d, E0, E1);
   int hn = nc / 2;
   const double2* y = Y + ((long)x * 5 + d) * nc * nc;
   double2 acc = make_double2(0.0, 0.0);

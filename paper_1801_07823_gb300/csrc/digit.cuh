@@ -82,18 +82,6 @@ inline Shape shape_of(const CoarseGeom& g) {
   return s;
 }
 
-__device__ __forceinline__ int nbr(int X, int d, int E0, int E1) {
-  int X0 = X % E0, X1 = X / E0;
-  if (d == 1) X0 = (X0 + 1 == E0) ? 0 : X0 + 1;
-  if (d == 2) X0 = (X0 == 0) ? E0 - 1 : X0 - 1;
-  if (d == 3) X1 = (X1 + 1 == E1) ? 0 : X1 + 1;
-  if (d == 4) X1 = (X1 == 0) ? E1 - 1 : X1 - 1;
-  return X0 + E0 * X1;
-}
-
-__device__ __forceinline__ int opp(int d) {
-  return d == 0 ? 0 : (d == 1 ? 2 : (d == 2 ? 1 : (d == 3 ? 4 : 3)));
-}
 // Place of (row i, column j) in its 4 x 4 tile.
 __host__ __device__ __forceinline__ int tile_place(int i, int j) {
   return (i & 2) * 4 + (j & 2) * 2 + (i & 1) * 2 + (j & 1);

@@ -124,14 +124,6 @@ struct Sub : NoCoef, NoSums {
     v(0)[i] = make_double2(a.x - b.x, a.y - b.y);
   }
 };
-struct Add3 : NoCoef, NoSums {
-  static constexpr int K = 4, R = 0;
-  template <typename V>
-  __device__ void elem(const V& v, long i, double2, double*) const {
-    const double2 a = v(1)[i], b = v(2)[i], d = v(3)[i];
-    v(0)[i] = make_double2((a.x + b.x) + d.x, (a.y + b.y) + d.y);
-  }
-};
 // Base of the operations whose sums are plain FP64 trees (the setup's).
 struct Tree {};
 struct Dot : NoCoef {
@@ -396,8 +388,8 @@ __global__ void __launch_bounds__(kThreads) k_many(Op op, Pack<Op::K, W> v, long
   }
 }
 
-// A sum's grid is capped, so that its parts fit one pass; up to 512 elements one CTA does
-// without the second stage.
+// A sum's grid is capped, so that the last CTA adds three parts a thread at most; up to 512
+// elements one CTA does without the second stage.
 template <typename Op>
 void launch(sw_ctx* c, long n, const Op& op, const Many<Op::K>& v, double* host = nullptr,
             int* ctl = nullptr) {
@@ -433,7 +425,6 @@ void many_sub(sw_ctx* c, long n, const Many<3>& v) { launch(c, n, Sub{}, v); }
 void many_sub_norm(sw_ctx* c, long n, const Many<3>& v, int s, double* host) {
   launch(c, n, SubNorm{{}, s}, v, host);
 }
-void many_add3(sw_ctx* c, long n, const Many<4>& v) { launch(c, n, Add3{}, v); }
 void many_dot(sw_ctx* c, long n, const Many<2>& v, int s) { launch(c, n, Dot{{}, s}, v); }
 void many_norm(sw_ctx* c, long n, const Many<1>& v, int s, double* host) {
   launch(c, n, Norm{{}, s}, v, host);

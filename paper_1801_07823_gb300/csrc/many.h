@@ -64,7 +64,6 @@ void many_mr(sw_ctx* c, long n, const Many<3>& xrq, int s, double om);
 void many_mr_last(sw_ctx* c, long n, const Many<5>& oxrab, int s, double om, bool first);
 void many_sub(sw_ctx* c, long n, const Many<3>& oab);                       // o = a - b
 void many_sub_norm(sw_ctx* c, long n, const Many<3>& oab, int s, double* host);
-void many_add3(sw_ctx* c, long n, const Many<4>& oabd);                     // o = (a + b) + d
 void many_dot(sw_ctx* c, long n, const Many<2>& ab, int s);
 void many_norm(sw_ctx* c, long n, const Many<1>& a, int s, double* host = nullptr);
 // q -= S[s] qj, p -= S[s] pj; then <qn, q> in s, or |q|^2 in s_qq for a member without qn

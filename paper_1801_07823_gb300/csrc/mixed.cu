@@ -25,17 +25,6 @@ __device__ __forceinline__ void cfmacf(float2& acc, float2 a, float2 b) {  // co
   acc.y = fmaf(-a.y, b.x, acc.y);
 }
 __device__ __forceinline__ float2 f2(double2 v) { return make_float2((float)v.x, (float)v.y); }
-__host__ __device__ __forceinline__ int nbr_site(int X, int d, int E0, int E1) {
-  int X0 = X % E0, X1 = X / E0;
-  if (d == 1) X0 = (X0 + 1 == E0) ? 0 : X0 + 1;
-  if (d == 2) X0 = (X0 == 0) ? E0 - 1 : X0 - 1;
-  if (d == 3) X1 = (X1 + 1 == E1) ? 0 : X1 + 1;
-  if (d == 4) X1 = (X1 == 0) ? E1 - 1 : X1 - 1;
-  return X0 + E0 * X1;
-}
-__host__ __device__ __forceinline__ int opp_dir(int d) {
-  return d == 0 ? 0 : (d == 1 ? 2 : (d == 2 ? 1 : (d == 3 ? 4 : 3)));
-}
 inline int cdiv(long a, long b) { return (int)((a + b - 1) / b); }
 
 // ------------------------------------------------------------------ fine FP32
@@ -175,7 +164,7 @@ __global__ void __launch_bounds__(5 * NC) k_coarse_apply_h(const __half2* __rest
   int nthr = 5 * rows;
   for (int t = threadIdx.x; t < 5 * NC; t += nthr) {
     int d = t / NC, j = t - d * NC;
-    xs[d][j] = f2(in[(long)nbr_site(X, d, E0, E1) * NC + j]);
+    xs[d][j] = f2(in[(long)nbr(X, d, E0, E1) * NC + j]);
   }
   __syncthreads();
   int d = threadIdx.x / rows;
@@ -189,7 +178,7 @@ __global__ void __launch_bounds__(5 * NC) k_coarse_apply_h(const __half2* __rest
 #pragma unroll 16
     for (int j = 0; j < NC; ++j) cfmaf(acc, __half22float2(y[j * NC]), xs[d][j]);
   } else {
-    long blk = (long)nbr_site(X, d, E0, E1) * 5 + opp_dir(d);
+    long blk = (long)nbr(X, d, E0, E1) * 5 + opp(d);
     sc = scale[blk];
     const __half2* y = Yh + (blk * NC + i) * NC;
 #pragma unroll 16
@@ -220,9 +209,9 @@ __global__ void k_coarse_apply_h_any(const __half2* __restrict__ Yh, const float
   int X = (int)(e / nc), i = (int)(e - (long)X * nc);
   float2 tot = make_float2(0.f, 0.f);
   for (int d = 0; d < 5; ++d) {
-    int Z = nbr_site(X, d, E0, E1);
+    int Z = nbr(X, d, E0, E1);
     float2 acc = make_float2(0.f, 0.f);
-    long blk = DAG ? (long)Z * 5 + opp_dir(d) : (long)X * 5 + d;
+    long blk = DAG ? (long)Z * 5 + opp(d) : (long)X * 5 + d;
     for (int j = 0; j < nc; ++j) {
       float2 xv = f2(in[(long)Z * nc + j]);
       if (!DAG)

@@ -8,8 +8,8 @@
 //
 // Scratch layout for N = L0 L1 <= kNoAllocMaxSites (complex128 units):
 //   [0, N)      copy of an input that overlaps the output
-//   [2N, 3N)    intermediate vector of the Schur operator
-//   [3N, 7N)    B^-1 table for the requested mass (rebuilt every call)
+//   [N, 2N)     intermediate vector of the Schur operator
+//   [2N, 6N)    B^-1 table for the requested mass (rebuilt every call)
 #include <cmath>
 #include <mutex>
 #include <string>
@@ -18,8 +18,8 @@
 
 namespace {
 
-constexpr long kNoAllocMaxSites = 65536;  // e.g. 256 x 256; 7.3 MB of device memory
-static __device__ __align__(256) double2 g_noalloc_scratch[7 * kNoAllocMaxSites];
+constexpr long kNoAllocMaxSites = 65536;  // e.g. 256 x 256; 6.3 MB of device memory
+static __device__ __align__(256) double2 g_noalloc_scratch[6 * kNoAllocMaxSites];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_noalloc_mutex;
@@ -52,8 +52,8 @@ extern "C" int sw_dslash_schur_noalloc(sw_gauge* g, double mass, const void* in,
     cudaStream_t s = c->stream;
     long N = g->N;
     double2* base = noalloc_scratch(c->device);
-    double2* w = base + 2 * N;
-    double2* binv = base + 3 * N;
+    double2* w = base + N;
+    double2* binv = base + 2 * N;
     launch_binv_build(g, mass, binv, s);
     const double2* x = (const double2*)in;
     double2* y = (double2*)out;

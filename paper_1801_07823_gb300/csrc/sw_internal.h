@@ -206,6 +206,19 @@ int guarded(sw_ctx* c, F&& f) {
 }
 
 // ------------------------------------------------------------- geometry
+// Coarse stencils: neighbour of site X = X0 + E0 X1 in direction d (0: X itself, 1, 2: +-0hat,
+// 3, 4: +-1hat), and the direction back.
+__host__ __device__ __forceinline__ int nbr(int X, int d, int E0, int E1) {
+  int X0 = X % E0, X1 = X / E0;
+  if (d == 1) X0 = (X0 + 1 == E0) ? 0 : X0 + 1;
+  if (d == 2) X0 = (X0 == 0) ? E0 - 1 : X0 - 1;
+  if (d == 3) X1 = (X1 + 1 == E1) ? 0 : X1 + 1;
+  if (d == 4) X1 = (X1 == 0) ? E1 - 1 : X1 - 1;
+  return X0 + E0 * X1;
+}
+__host__ __device__ __forceinline__ int opp(int d) {
+  return d == 0 ? 0 : (d == 1 ? 2 : (d == 2 ? 1 : (d == 3 ? 4 : 3)));
+}
 // Parity-split block-major order of a fine field: f = par * N/2 + 4 * hb + k,
 // KD block (X0, X1) = (x0/2, x1/2), par = (X0 + X1) & 1,
 // hb = X1 * (L0/4) + X0/2, k = (x0 & 1) + 2 (x1 & 1).
