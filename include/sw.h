@@ -355,13 +355,13 @@ int sw_fp64_peak(sw_ctx* ctx, double* tflops);
 
 /* Failure-detection check of the persistent coarsest-level CGNE: runs it
  * once with one CTA withholding its arrival at the first grid barrier, so
- * every other CTA's bounded wait runs out (about a second).  Expected result:
+ * every other CTA's bounded wait runs out (1.5 to 2 s).  Expected result:
  * SW_ERR_TIMEOUT, with the context still usable afterwards. */
 int sw_debug_cgne_stall(sw_mg* mg);
 
 /* Failure-detection check of the batched coarsest kernel: runs it once on
  * nrhs zero right-hand sides with one CTA withholding its first grid-barrier
- * arrival, so every other CTA's bounded wait runs out (about a second).
+ * arrival, so every other CTA's bounded wait runs out (1.5 to 2 s).
  * Expected result: SW_ERR_TIMEOUT, with the context still usable afterwards. */
 int sw_debug_batch_stall(sw_mg* mg, int nrhs);
 

@@ -37,7 +37,6 @@
 
 namespace {
 
-constexpr long kSpinLimit = 1L << 24;      // grid barrier polls
 constexpr long kCopySpinLimit = 1L << 22;  // mbarrier polls per stage
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;

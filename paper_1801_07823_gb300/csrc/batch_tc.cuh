@@ -48,7 +48,6 @@
 
 namespace swtc {
 
-constexpr long kSpinLimit = 1L << 21;      // grid-barrier polls, about a second
 constexpr long kWaitLimit = 1L << 22;      // mbarrier polls
 constexpr int kThreads = 256;
 constexpr int kEpiThreads = 128;           // warps 4..7

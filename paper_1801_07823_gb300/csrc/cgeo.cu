@@ -105,7 +105,6 @@ void hop_eo(const sw_gauge* g, int par, double a, const double2* src, double c, 
 // ---------------------------------------------------------------- the iteration
 constexpr int kCgThreads = 512;
 constexpr int kCgWarps = kCgThreads / 32;
-constexpr long kCgSpins = 1L << 21;
 constexpr int kCgSlots = 256;  // above the multigrid levels' 4 x 64
 constexpr int kCgKeep = 4;  // iterations of a launch before it yields its SMs
 // Whether a launch per operation on all SMs beats the persistent kernel on `sms` of them.
@@ -194,7 +193,7 @@ __device__ bool cg_barrier(const CgArgs& a, CgShared& sh, unsigned gen, double v
     for (;;) {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(a.bar) : "memory");
       if (n >= target) break;
-      if (++spins > kCgSpins) {
+      if (++spins > kSpinLimit) {
         atomicExch(a.status + 1, 1);
         break;
       }

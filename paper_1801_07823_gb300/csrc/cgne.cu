@@ -32,8 +32,6 @@
 namespace {
 
 
-constexpr long kSpinLimit = 1L << 24;    // ~0.3-1.5 s of polling
-
 // Double-float ("df64") arithmetic on the FP32 pipes (Dekker 1971; Knuth's
 // two-sum): a value is hi + lo with two floats, 48 significant bits.
 // GB300 issues FP32 FMAs at 62x the FP64 rate, so the coarsest stencil in

@@ -53,7 +53,6 @@ namespace {
 using namespace swdig;
 using namespace swsum;
 
-constexpr long kSpinLimit = 1L << 21;
 constexpr int kThreads = 384;
 constexpr int kWarps = kThreads / 32;
 constexpr int kPut = kThreads - 32;  // threads that write vector digits

@@ -205,6 +205,11 @@ int guarded(sw_ctx* c, F&& f) {
   }
 }
 
+// Polls after which a wait at a grid barrier gives up (SW_ERR_TIMEOUT).  A poll of a word in the
+// L2 takes 0.17 us (2^21 of them, withheld arrival: 0.37 s), with a sleep of 16 ns between polls
+// 0.25 (2^24: 4.1 s): 1.5 to 2 s, hundreds of times the longest phase.
+constexpr long kSpinLimit = 1L << 23;
+
 // ------------------------------------------------------------- geometry
 // Coarse stencils: neighbour of site X = X0 + E0 X1 in direction d (0: X itself, 1, 2: +-0hat,
 // 3, 4: +-1hat), and the direction back.
