@@ -40,32 +40,35 @@ WORKLOAD = dict(workload="KD-staggered MG solve, 2D U(1) 256x256, beta=6 (2000 h
                 L=256, beta=6.0, sweeps=2000, mass=1e-3, levels=3, blocks=[[4, 4], [2, 2]],
                 nvec=[24, 32], tol=1e-10, coarsest_maxiter=2048)
 FP64_PEAK_TFLOPS = 152 * 4 * 2.070e9 / 1e12  # 4 FP64 flop/clk/SM (2 DFMA) x 152 SMs x 2070 MHz
-MMA_SYNC_TFLOPS = 594.0  # 152 SMs x 944 multiply-adds per clock x 2.07 GHz, mma.sync m16n8k16 FP16
 
 
-def _hbm_peak():
+def _measured_peak(key: str, fallback: float) -> float:
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as fh:
-            return float(json.load(fh)["hbm_gbs"])
+            return float(json.load(fh)[key])
     except (OSError, KeyError, ValueError):
-        return 6800.0  # fallback copy bandwidth
+        return fallback
 
 
-HBM_PEAK_GBS = _hbm_peak()
+HBM_PEAK_GBS = _measured_peak("hbm_gbs", 6800.0)          # copy bandwidth
+TENSOR_PEAK_TFLOPS = _measured_peak("bf16_tflops", 1900.0)  # 16-bit GEMM, burst
 
 
 def _profiled_traffic(profile: str, source: str, key: str):
-    """A DRAM-traffic figure recorded in profiles/<profile> by an ncu capture,
-    or None when the kernel source has changed since that capture."""
+    """A DRAM-traffic figure recorded in profiles/<profile> by an ncu capture, or
+    None when the kernel source, or another source the profile names (headers with
+    its loads and layout), has changed since that capture."""
     import hashlib
     try:
         text = open(os.path.join(ROOT, "profiles", profile)).read()
-        want = hashlib.sha1(open(os.path.join(ROOT, source), "rb").read()).hexdigest()
+        fields = dict(line.split(": ", 1) for line in text.splitlines() if ": " in line)
+        recorded = {k[len("source_sha1 ("):-1]: v.strip() for k, v in fields.items()
+                    if k.startswith("source_sha1 (")}
+        same = all(hashlib.sha1(open(os.path.join(ROOT, f), "rb").read()).hexdigest() == sha
+                   for f, sha in recorded.items())
     except OSError:
         return None
-    fields = dict(line.split(": ", 1) for line in text.splitlines() if ": " in line)
-    sha = fields.get(f"source_sha1 ({source})")
-    if sha is None or sha.strip() != want or key not in fields:
+    if source not in recorded or not same or key not in fields:
         return None
     return float(fields[key])
 
@@ -676,8 +679,8 @@ def run_native(args, rank, world, local):
     # a complex entry takes 12 m16n8k16 MMAs per 128 of them: 384 FP16 flops for its 8 FP64 ones
     executed = 384.0 / 8.0 * achieved
     roof = {"bound": "tensor", "kernel": kname,
-            "achieved": executed, "peak": MMA_SYNC_TFLOPS, "unit": "TFLOP/s",
-            "frac": executed / MMA_SYNC_TFLOPS, "traffic": traffic,
+            "achieved": executed, "peak": TENSOR_PEAK_TFLOPS, "unit": "TFLOP/s",
+            "frac": executed / TENSOR_PEAK_TFLOPS, "traffic": traffic,
             "achieved_note": "FP16 tensor flops executed by the digit products (384 per complex "
                              "multiply-add) per launch / average launch time",
             "fp64_TFLOPs": achieved, "fp64_peak_TFLOPs": fp64_peak,
@@ -687,8 +690,7 @@ def run_native(args, rank, world, local):
                          "do not run on the FP64 pipe",
             "traffic_note": "ncu dram bytes per CGNE iteration (profiles/k_cgne64_fp64_256.md) x "
                             "iterations per launch; null if the kernel changed since",
-            "peak_source": "measured rate of independent mma.sync m16n8k16 FP16 at 2070 MHz: 944 "
-                           "multiply-adds per clock and SM",
+            "peak_source": "MEASURED_PEAKS.json bf16_tflops: 16-bit GEMM of the same GPU type",
             "fp64_peak_nominal": FP64_PEAK_TFLOPS,
             "algorithmic_flop_per_launch": flop,
             "hbm_GBps_equiv": byt / dur / 1e9, "launches": n_l, "avg_us": dur * 1e6}
