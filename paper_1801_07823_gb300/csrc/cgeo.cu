@@ -10,7 +10,7 @@
 // Layout: half-lattice vectors, site (x0, x1) of parity p at (x1 L0 + x0) / 2.
 //
 // The iteration is one persistent cooperative kernel (k_cg_eo).  As eight
-// launches per iteration it took 55 us at 256^2, most of it launch gaps; now 14.6
+// launches per iteration it took 55 us at 256^2, most of it launch gaps; now 14.8
 // us, and 13 on any smaller lattice: three barriers (1.2 us each), two sums over
 // the grid with an FP64 division each (1.5 us), three round trips to the L2 and
 // chains of dependent FP64 operations at 64 clocks each.  A CTA owns a contiguous run
